@@ -26,12 +26,15 @@
 // threshold, else the call falls back to the tridiagonal reduction.  The
 // fallback also runs when r is not decided within KRYLOV_MAX steps.
 //
-// Layout: mu (row-major complex64) is promoted once to complex128 M (the
-// same row-major order; the rebuild's working matrix, its norm and trace),
-// while the Lanczos product reads the complex64 input itself; the Krylov
-// basis Q holds one d-vector per row (vector t at Q + t d) as FP32 pairs.  y = mu x is the
-// row-major product, so the vectors are eigenvectors of mu; the rebuild of
-// project.cu works on conj(mu), whose eigenvectors are their conjugates.
+// Up to d = 1024 the run may go on to d steps, where T holds the whole spectrum
+// and nothing is left to certify; the selected values are then replaced by their
+// FP64 Rayleigh quotients (krylov_vecs.cu), so they are as exact as a reduction's.
+//
+// Layout: the products read mu as complex64 (up to d = 4096 a Hermitian copy of
+// the input's upper triangle); the Krylov basis Q holds one d-vector per row
+// (vector t at Q + t d) in double-float.  y = mu x is the row-major product, so
+// the vectors are eigenvectors of mu.  Up to d = 4096 a run of steps is one
+// persistent launch (krylov_steps.cu); beyond, one launch per operation.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -39,12 +42,13 @@
 #include <cmath>
 #include <vector>
 
+#include "dfloat.cuh"
+#include "krylov.cuh"
 #include "lre_internal.cuh"
 
 namespace lre {
 namespace {
 
-constexpr int MV_RPW = 1;          // rows of M per warp of the product (eight warps per CTA)
 constexpr int MV_CHUNK = 1024;     // x entries staged in shared memory at a time
 constexpr int RED_THREADS = 256;
 
@@ -52,6 +56,11 @@ __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+__global__ void kry_split(const double2 *__restrict__ x, float4 *__restrict__ xs, int64_t d) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x)
+    xs[i] = df::split(x[i]);
 }
 
 // ---- the Lanczos product y = mu x in double-float arithmetic on the FP32 pipes --
@@ -62,109 +71,38 @@ __device__ __forceinline__ double warp_sum(double v) {
 // Knuth's TwoSum on the leading part: about 2^-44 relative per term, against
 // 2^-53 in FP64 -- far inside the Lanczos tolerances -- at the FP32 rate,
 // where GB300's FP64 rate had made the product FP64-bound, and reading 8
-// bytes per entry of mu instead of 16.  The _rn intrinsics keep the compiler
-// from contracting the steps into FMAs, which would break the exact errors.
-__device__ __forceinline__ void df_mac(float &sh, float &sl, float m, float xh, float xl) {
-  const float p = __fmul_rn(m, xh);
-  const float e = __fmaf_rn(m, xh, -p);
-  const float t = __fadd_rn(sh, p);  // TwoSum(sh, p) = t + err exactly
-  const float bp = __fsub_rn(t, sh);
-  const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bp)), __fsub_rn(p, bp));
-  sh = t;
-  sl = __fadd_rn(sl, __fadd_rn(err, __fmaf_rn(m, xl, e)));
-}
-
-// The same for a product of two such pairs, (ah + al)(bh + bl): the leading
-// product exactly (p and its error), the cross terms into the error part.
-__device__ __forceinline__ void df_mac2(float &sh, float &sl, float ah, float al, float bh, float bl) {
-  const float p = __fmul_rn(ah, bh);
-  float e = __fmaf_rn(ah, bh, -p);
-  e = __fmaf_rn(ah, bl, e);
-  e = __fmaf_rn(al, bh, e);
-  const float t = __fadd_rn(sh, p);
-  const float bp = __fsub_rn(t, sh);
-  const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bp)), __fsub_rn(p, bp));
-  sh = t;
-  sl = __fadd_rn(sl, __fadd_rn(err, e));
-}
-
-// complex128 <-> {re hi, re lo, im hi, im lo} as FP32 (the Krylov basis, the
-// split copies of the work vector): about 2^-48 relative per component
-__device__ __forceinline__ float4 df_split(double2 v) {
-  const float rh = __double2float_rn(v.x), ih = __double2float_rn(v.y);
-  return make_float4(rh, __double2float_rn(v.x - (double)rh), ih, __double2float_rn(v.y - (double)ih));
-}
-__device__ __forceinline__ double2 df_join(float4 q) {
-  return make_double2((double)q.x + (double)q.y, (double)q.z + (double)q.w);
-}
-
-__global__ void kry_split(const double2 *__restrict__ x, float4 *__restrict__ xs, int64_t d) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x)
-    xs[i] = df_split(x[i]);
-}
-
-// y = M x with M the row-major d x d complex64 matrix and x a basis row in
-// split form; y also in split form for the reorthogonalisation.  MV_RPW rows
-// per warp, x staged in shared memory (d a multiple of MV_CHUNK or d <
-// MV_CHUNK); with one row per warp and whole chunks each lane loads its 32
-// entries of the chunk before their products (more loads in flight: 4.9
-// against 3.5 TB/s at d = 16384); the warp's partial sums are added in FP64.
-template <int RPW>
+// bytes per entry of mu instead of 16.  Packed instructions (dfloat.cuh).
+//
+// M row-major d x d (d a multiple of MV_CHUNK), x a basis row; y also in split
+// form for the reorthogonalisation.  One row per warp, x staged in shared
+// memory; each lane loads its 32 entries of a chunk before their products (more
+// loads in flight: 4.9 against 3.5 TB/s at d = 16384 loading one at a time).
 __global__ void __launch_bounds__(256, 3) kry_matvec_df(const float2 *__restrict__ M, const float4 *__restrict__ xsplit,
                                                      double2 *__restrict__ y, float4 *__restrict__ ysplit,
                                                      int64_t d) {
   __shared__ float4 xs[MV_CHUNK];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t r0 = ((int64_t)blockIdx.x * 8 + warp) * RPW;
-  float rh[RPW], rl[RPW], ih[RPW], il[RPW];
+  const int64_t r = (int64_t)blockIdx.x * 8 + warp;  // d is a multiple of 8
+  df::Sum S;
+  for (int64_t c0 = 0; c0 < d; c0 += MV_CHUNK) {
+    const float2 *row = M + r * d + c0;
+    float2 u[32];
 #pragma unroll
-  for (int r = 0; r < RPW; ++r) rh[r] = rl[r] = ih[r] = il[r] = 0.f;
-  const int64_t chunk = d < MV_CHUNK ? d : MV_CHUNK;
-  for (int64_t c0 = 0; c0 < d; c0 += chunk) {
+    for (int q = 0; q < 32; ++q) u[q] = row[lane + 32 * q];
     __syncthreads();
-    for (int k = threadIdx.x; k < chunk; k += blockDim.x) xs[k] = xsplit[c0 + k];
+    for (int k = threadIdx.x; k < MV_CHUNK; k += 256) xs[k] = xsplit[c0 + k];
     __syncthreads();
-    if (r0 < d) {
-      const float2 *row = M + r0 * d + c0;
-      if (RPW == 1 && chunk % 1024 == 0) {
-        // thirty-two entries of the row loaded ahead of their products
-        for (int k0 = lane; k0 < chunk; k0 += 1024) {
-          float2 u[32];
 #pragma unroll
-          for (int q = 0; q < 32; ++q) u[q] = row[k0 + 32 * q];
-#pragma unroll
-          for (int q = 0; q < 32; ++q) {
-            const float4 xv = xs[k0 + 32 * q];
-            df_mac(rh[0], rl[0], u[q].x, xv.x, xv.y);
-            df_mac(rh[0], rl[0], -u[q].y, xv.z, xv.w);
-            df_mac(ih[0], il[0], u[q].x, xv.z, xv.w);
-            df_mac(ih[0], il[0], u[q].y, xv.x, xv.y);
-          }
-        }
-      } else {
-        for (int k = lane; k < chunk; k += 32) {
-          const float4 xv = xs[k];  // x re = xv.x + xv.y, x im = xv.z + xv.w
-#pragma unroll
-          for (int r = 0; r < RPW; ++r) {
-            if (r0 + r < d) {
-              const float2 u = row[(int64_t)r * d + k];
-              df_mac(rh[r], rl[r], u.x, xv.x, xv.y);   // re += ur xr - ui xi
-              df_mac(rh[r], rl[r], -u.y, xv.z, xv.w);
-              df_mac(ih[r], il[r], u.x, xv.z, xv.w);   // im += ur xi + ui xr
-              df_mac(ih[r], il[r], u.y, xv.x, xv.y);
-            }
-          }
-        }
-      }
+    for (int q = 0; q < 32; ++q) {
+      const float4 x = xs[lane + 32 * q];
+      df::mac_c64(S, u[q], df::hi(x), df::lo(x));
     }
   }
-#pragma unroll
-  for (int r = 0; r < RPW; ++r) {
-    const double re = warp_sum((double)rh[r] + (double)rl[r]), im = warp_sum((double)ih[r] + (double)il[r]);
-    if (lane == 0 && r0 + r < d) {
-      y[r0 + r] = make_double2(re, im);
-      ysplit[r0 + r] = df_split(make_double2(re, im));
-    }
+  const double2 p = df::join(df::df_ab(S));
+  const double re = warp_sum(p.x), im = warp_sum(p.y);
+  if (lane == 0) {
+    y[r] = make_double2(re, im);
+    ysplit[r] = df::split(make_double2(re, im));
   }
 }
 
@@ -177,15 +115,13 @@ __global__ void __launch_bounds__(RED_THREADS) kry_dots(const float4 *__restrict
   __shared__ double sr[RED_THREADS / 32], si[RED_THREADS / 32];
   for (int t = blockIdx.x; t < m; t += gridDim.x) {
     const float4 *q = Q + (int64_t)t * d;
-    float rh = 0, rl = 0, ih = 0, il = 0;
+    df::Sum S;
     for (int64_t i = threadIdx.x; i < d; i += blockDim.x) {
-      const float4 a = q[i], b = w[i];  // conj(a) b
-      df_mac2(rh, rl, a.x, a.y, b.x, b.y);
-      df_mac2(rh, rl, a.z, a.w, b.z, b.w);
-      df_mac2(ih, il, a.x, a.y, b.z, b.w);
-      df_mac2(ih, il, -a.z, -a.w, b.x, b.y);
+      const float4 b = w[i];
+      df::mac_df(S, q[i], df::hi(b), df::lo(b));
     }
-    const double re = warp_sum((double)rh + (double)rl), im = warp_sum((double)ih + (double)il);
+    const double2 p = df::join(df::df_conj_ab(S));
+    const double re = warp_sum(p.x), im = warp_sum(p.y);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane == 0) {
       sr[warp] = re;
@@ -214,23 +150,19 @@ __global__ void __launch_bounds__(256) kry_update(double2 *__restrict__ w, float
                                                   const double2 *__restrict__ h, int64_t d) {
   extern __shared__ float4 hs[];
   __shared__ double2 part[UPD_SLICES][64];
-  for (int t = threadIdx.x; t < m; t += blockDim.x) hs[t] = df_split(h[t]);
+  for (int t = threadIdx.x; t < m; t += blockDim.x) hs[t] = df::split(h[t]);
   __syncthreads();
   const int e = threadIdx.x & 63, slice = threadIdx.x >> 6;
   for (int64_t i0 = (int64_t)blockIdx.x * 64; i0 < d; i0 += (int64_t)gridDim.x * 64) {
     const int64_t i = i0 + e;
-    float rh = 0, rl = 0, ih = 0, il = 0;
+    df::Sum S;
     if (i < d) {
       for (int t = slice; t < m; t += UPD_SLICES) {
         const float4 q = Q[(int64_t)t * d + i];
-        const float4 c = hs[t];  // q c
-        df_mac2(rh, rl, q.x, q.y, c.x, c.y);
-        df_mac2(rh, rl, -q.z, -q.w, c.z, c.w);
-        df_mac2(ih, il, q.x, q.y, c.z, c.w);
-        df_mac2(ih, il, q.z, q.w, c.x, c.y);
+        df::mac_df(S, hs[t], df::hi(q), df::lo(q));
       }
     }
-    part[slice][e] = make_double2((double)rh + (double)rl, (double)ih + (double)il);
+    part[slice][e] = df::join(df::df_ab(S));
     __syncthreads();
     if (slice == 0 && i < d) {
       double re = 0, im = 0;
@@ -243,7 +175,7 @@ __global__ void __launch_bounds__(256) kry_update(double2 *__restrict__ w, float
       v.x -= re;
       v.y -= im;
       w[i] = v;
-      ws[i] = df_split(v);
+      ws[i] = df::split(v);
     }
     __syncthreads();
   }
@@ -286,7 +218,7 @@ __global__ void kry_close(const double2 *h1, const double2 *h2, int c, const dou
   const double inv = dead ? 0.0 : 1.0 / b;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x) {
     const double2 v = w[i];
-    qn[i] = df_split(make_double2(v.x * inv, v.y * inv));  // the basis in split form
+    qn[i] = df::split(make_double2(v.x * inv, v.y * inv));  // the basis in split form
   }
 }
 
@@ -309,82 +241,9 @@ __global__ void kry_scale(const double2 *v, float4 *q, int64_t d, const double *
   const double inv = 1.0 / sqrt(*nrm2);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x) {
     const double2 a = v[i];
-    q[i] = df_split(make_double2(a.x * inv, a.y * inv));
+    q[i] = df::split(make_double2(a.x * inv, a.y * inv));
   }
 }
-
-// Ritz vectors: Z[:, k] = conj(sum_t S[t + k J] q_t) for k < m (Z column-major
-// d x m, S column-major J x m real); eight columns per thread.
-__global__ void __launch_bounds__(256) kry_ritz(const float4 *__restrict__ Q, int J, const double *__restrict__ S,
-                                                int m, double2 *__restrict__ Z, int64_t d) {
-  const int k0 = blockIdx.y * 8;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x) {
-    double re[8], im[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) re[k] = im[k] = 0.0;
-    for (int t = 0; t < J; ++t) {
-      const double2 q = df_join(Q[(int64_t)t * d + i]);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        if (k0 + k < m) {
-          const double c = S[t + (int64_t)(k0 + k) * J];
-          re[k] = fma(q.x, c, re[k]);
-          im[k] = fma(q.y, c, im[k]);
-        }
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k0 + k < m) Z[i + (int64_t)(k0 + k) * d] = make_double2(re[k], -im[k]);
-  }
-}
-
-// Row-major copy of the conjugate Ritz vectors back into basis rows (for the
-// certification run): Q[t][i] = conj(Z[i + t d]).
-__global__ void kry_seed(const double2 *Z, int m, float4 *Q, int64_t d) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)m * d;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const double2 v = Z[e];
-    Q[e] = df_split(make_double2(v.x, -v.y));
-  }
-}
-
-// *acc += sum of the real diagonal of M (zeroed by the caller).
-__global__ void __launch_bounds__(RED_THREADS) kry_trace(const double2 *__restrict__ M, int64_t d, double *acc) {
-  __shared__ double s[RED_THREADS / 32];
-  double v = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < d; i += (int64_t)gridDim.x * blockDim.x)
-    v += M[i * d + i].x;
-  v = warp_sum(v);
-  if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0;
-    for (int k = 0; k < RED_THREADS / 32; ++k) t += s[k];
-    atomicAdd(acc, t);
-  }
-}
-
-// Last components S[J-1 + k J] of the m inverse-iteration vectors.
-__global__ void kry_last(const double *S, int J, int m, double *out) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x)
-    out[k] = S[(J - 1) + (int64_t)k * J];
-}
-
-// Promote the row-major complex64 input to complex128 (same order) into M and
-// into C (the rebuild's working matrix, read there as column-major conj(mu)).
-__global__ void kry_promote(const float2 *in, double2 *M, double2 *C, int64_t N) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    const float2 v = in[i];
-    const double2 w = make_double2((double)v.x, (double)v.y);
-    M[i] = w;
-    C[i] = w;
-  }
-}
-
-}  // namespace
-
-namespace {
 
 constexpr int KRY_CHECK = 64;           // Lanczos steps between convergence checks
 constexpr int KRY_VERIFY = 64;          // steps of the certification run
@@ -398,26 +257,34 @@ __global__ void kry_eig_rho(const double *w_asc, int64_t r, double shift, double
 }
 
 struct KryBuffers {
-  double2 *M, *W, *h1, *h2, *Z;
-  float4 *Q;          // the Krylov basis, one row per vector, in split form (about 48 bits)
-  const float2 *M32;  // the complex64 input, read by the double-float product
-  float4 *Ws;         // the work vector W in split form
+  double2 *W, *h1, *h2;  // FP64 work vector and coefficients of the multi-launch form
+  float4 *Q;             // the Krylov basis, one row per vector, double-float (about 48 bits)
+  float4 *Z;             // selected Ritz vectors, rows
+  const float2 *A;       // mu (d <= KRY_STEPS_MAX_D: the Hermitian copy of the input)
+  float4 *Ws;            // the work vector in double-float form; persistent steps: a step's product
+  float4 *Hs, *Wn;       // persistent steps: the corrections, a step's result before normalising
+  void *sync;            // persistent steps: the grid barrier and what the CTAs exchange
   double *alpha, *beta, *b2, *stats, *Wr, *Xr, *lu, *last, *nrm;
   int *cl, *nclust, *breakdown;
-  SmolinResult *res;
   int64_t rows, ct_max;
 };
 
-// Ritz values and last eigenvector components of the J x J Lanczos matrix
-// (alpha, beta) for its CB smallest and CT largest eigenvalues (ascending in
-// Wr[0..CB+CT), vectors in Xr), copied to the host with beta[J-1].
+// The J x J Lanczos matrix's CB smallest and CT largest eigenvalues
+// (ascending), the magnitudes of their unit eigenvectors' last components,
+// beta[J-1] and ||T||.
 struct RitzEnds {
   std::vector<double> w, last;
   double beta_next = 0, tnorm = 0;
 };
 
-lre_status ritz_ends(lre_ctx *ctx, const KryBuffers &B, const double *alpha, const double *beta, int J, int CB,
-                     int CT, cudaStream_t s, RitzEnds &out) {
+// Convergence check.  The residual of a Ritz pair is beta_J |s_J|, s_J the last
+// component of its eigenvector, which one inverse-iteration solve from the
+// eigenvalue (computed to 4 eps ||T||) gives to far below the tolerance; the
+// vectors that are used get all rounds (ritz_vectors) and are looked at again.
+// Values placed less exactly will not do: an unconverged neighbour's last
+// component comes through with the value's error over their gap.
+lre_status ritz_values(lre_ctx *ctx, const KryBuffers &B, const double *alpha, const double *beta, int J, int CB,
+                       int CT, bool want_last, cudaStream_t s, RitzEnds &out) {
   {
     Launch L(ctx, "kry_tri_prepare", s);
     tri_prepare<<<1, 256, 0, s>>>(alpha, beta, J, B.b2, B.stats);
@@ -429,39 +296,24 @@ lre_status ritz_ends(lre_ctx *ctx, const KryBuffers &B, const double *alpha, con
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "Lanczos matrix bounds");
   const double tnorm = fmax(fabs(hst[0]), fabs(hst[1]));
-  const double pivmin = DBL_MIN * fmax(1.0, hst[2]);
-  const double pad = 2.0 * DBL_EPSILON * tnorm + 2.0 * pivmin;
-  const double tol = 4.0 * DBL_EPSILON * fmax(tnorm, DBL_MIN);
+  const double pad = 2.0 * DBL_EPSILON * tnorm + 2.0 * DBL_MIN;
   const int m = CB + CT;
+  const size_t smem = (size_t)24 * J;
+  e = cudaFuncSetAttribute(tri_ends_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "Ritz values");
   {
-    Launch L(ctx, "kry_bisect", s, 2);  // one warp per Ritz value, two per CTA
-    if (CB > 0)
-      tri_multisect_kernel<<<(CB + 1) / 2, 64, 0, s>>>(alpha, B.b2, J, hst[0] - pad, hst[1] + pad, tol, pivmin,
-                                                       B.Wr, 0, CB);
-    tri_multisect_kernel<<<(CT + 1) / 2, 64, 0, s>>>(alpha, B.b2, J, hst[0] - pad, hst[1] + pad, tol, pivmin,
-                                                     B.Wr + CB, J - CT, CT);
+    Launch L(ctx, "kry_bisect", s);
+    tri_ends_kernel<<<m, 128, smem, s>>>(alpha, B.b2, J, hst[0] - pad, hst[1] + pad, tnorm, B.Wr, CB, CT);
   }
-  int hk = 0;
-  {
-    Launch L(ctx, "kry_clusters", s);
-    tri_clusters<<<1, 32, 0, s>>>(B.Wr, m, 1e-8 * tnorm, B.cl, B.nclust);
-  }
-  e = cudaMemcpyAsync(&hk, B.nclust, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "Ritz clusters");
-  {
-    Launch L(ctx, "kry_inverse_iteration", s, 2 + 2 * TRI_ROUNDS);
-    tri_factor<<<(m + 31) / 32, 32, 0, s>>>(alpha, beta, J, B.Wr, m, tnorm, B.lu);
-    for (int it = 0; it < TRI_ROUNDS; ++it) {
-      tri_solve<<<(m + 31) / 32, 32, 0, s>>>(B.lu, J, m, B.Xr, it == 0);
-      tri_orthonormalise<<<hk, TRI_THREADS, 0, s>>>(B.Xr, J, B.cl);
-    }
-    kry_last<<<(m + 255) / 256, 256, 0, s>>>(B.Xr, J, m, B.last);
+  if (want_last) {
+    Launch L(ctx, "kry_residuals", s);
+    tri_residual<<<(m + 31) / 32, 32, 0, s>>>(alpha, beta, J, B.Wr, m, tnorm, B.lu, B.last);
   }
   out.w.resize(m);
-  out.last.resize(m);
+  out.last.assign(m, 0.0);
   e = cudaMemcpyAsync(out.w.data(), B.Wr, m * sizeof(double), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(out.last.data(), B.last, m * sizeof(double), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess && want_last)
+    e = cudaMemcpyAsync(out.last.data(), B.last, m * sizeof(double), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "Ritz values");
   out.beta_next = bnext;
@@ -469,11 +321,44 @@ lre_status ritz_ends(lre_ctx *ctx, const KryBuffers &B, const double *alpha, con
   return LRE_OK;
 }
 
+// Unit eigenvectors of the J x J Lanczos matrix for its m eigenvalues w
+// (device, ascending) into Xr, and their last components on the host: inverse
+// iteration, orthonormalised within clusters of values closer than 1e-6 ||T||
+// (beyond that the solves' own error, eps ||T|| / gap, is below 1e-9).
+lre_status ritz_vectors(lre_ctx *ctx, const KryBuffers &B, const double *alpha, const double *beta, int J,
+                        const double *w, int m, double tnorm, cudaStream_t s, std::vector<double> &last) {
+  int hk = 0;
+  {
+    Launch L(ctx, "kry_clusters", s);
+    tri_clusters<<<1, 32, 0, s>>>(w, m, 1e-6 * tnorm, B.cl, B.nclust);
+  }
+  cudaError_t e = cudaMemcpyAsync(&hk, B.nclust, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "Ritz clusters");
+  {
+    Launch L(ctx, "kry_inverse_iteration", s, 2 + 2 * TRI_ROUNDS);
+    tri_factor<<<(m + 31) / 32, 32, 0, s>>>(alpha, beta, J, w, m, tnorm, B.lu);
+    for (int it = 0; it < TRI_ROUNDS; ++it) {
+      tri_solve<<<(m + 31) / 32, 32, 0, s>>>(B.lu, J, m, B.Xr, it == 0);
+      tri_orthonormalise<<<hk, TRI_THREADS, 0, s>>>(B.Xr, J, B.cl);
+    }
+    tri_last<<<(m + 3) / 4, 128, 0, s>>>(B.Xr, J, m, B.last);
+  }
+  last.resize(m);
+  e = cudaMemcpyAsync(last.data(), B.last, m * sizeof(double), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  return e == cudaSuccess ? LRE_OK : cuda_fail(ctx, e, "Ritz vectors");
+}
+
 // Lanczos steps [j0, j1) on basis rows base + j (rows 0..base + j - 1 fixed):
 // every step reorthogonalises against all earlier rows (classical
 // Gram-Schmidt, twice) and writes alpha[j], beta[j] and row base + j + 1.
 lre_status lanczos_steps(lre_ctx *ctx, const KryBuffers &B, int64_t d, int64_t base, int j0, int j1, double *alpha,
                          double *beta, double tiny, cudaStream_t s) {
+  if (d <= KRY_STEPS_MAX_D) {
+    const KryStepBuffers K{B.A, B.Q, B.Ws, B.Wn, B.Hs, B.sync, B.breakdown, B.rows};
+    return kry_steps_run(ctx, K, d, base, j0, j1, alpha, beta, tiny, s);
+  }
   const int red_grid = (int)std::min<int64_t>((d + RED_THREADS - 1) / RED_THREADS, (int64_t)ctx->num_sms * 4);
   const int upd_grid = (int)((d + 63) / 64);
   for (int j = j0; j < j1; ++j) {
@@ -481,8 +366,7 @@ lre_status lanczos_steps(lre_ctx *ctx, const KryBuffers &B, int64_t d, int64_t b
     const int cols = (int)(c + 1);
     {
       Launch L(ctx, "kry_matvec", s);  // W = mu q_j and its split copy
-      kry_matvec_df<MV_RPW><<<(unsigned)((d + 8 * MV_RPW - 1) / (8 * MV_RPW)), 256, 0, s>>>(B.M32, B.Q + c * d, B.W,
-                                                                                          B.Ws, d);
+      kry_matvec_df<<<(unsigned)(d / 8), 256, 0, s>>>(B.A, B.Q + c * d, B.W, B.Ws, d);
     }
     {
       Launch L(ctx, "kry_reorth", s, 4);
@@ -530,61 +414,63 @@ lre_status start_vector(lre_ctx *ctx, const KryBuffers &B, int64_t d, int64_t ro
 
 }  // namespace
 
-lre_status project_krylov(lre_ctx *ctx, cublasContext *blas, const lre_c64 *rho_in, int64_t d, lre_c64 *rho_out,
-                          double *eig_rho, cudaStream_t s, bool *fallback) {
+lre_status project_krylov(lre_ctx *ctx, const lre_c64 *rho_in, int64_t d, lre_c64 *rho_out, double *eig_rho,
+                          cudaStream_t s, bool *fallback) {
   *fallback = true;
-  const int64_t kmax = std::min<int64_t>(d / 2, KRY_MAX_STEPS);
+  // up to d = 1024 the run may go to d steps, where T holds the whole spectrum;
+  // beyond, 2048 steps (and half of d) bound it
+  const bool whole = d <= KRY_MAX_VECS;
+  const int64_t kmax = whole ? d : std::min<int64_t>(d / 2, KRY_MAX_STEPS);
+  const int64_t vecs = std::min<int64_t>(d, KRY_MAX_VECS);
   KryBuffers B{};
-  B.rows = std::max<int64_t>(kmax + 1, KRY_MAX_VECS + KRY_VERIFY + 1);
-  B.ct_max = KRY_MAX_VECS + 64;
+  B.rows = whole ? d + 1 : std::max<int64_t>(kmax + 1, KRY_MAX_VECS + KRY_VERIFY + 1);
+  B.ct_max = whole ? d + 1 : vecs + 64;  // whole: 88 d^2 bytes in all, less than the reduction path's 96 d^2
+  const bool copy = d <= KRY_STEPS_MAX_D;  // the steps read a Hermitian copy of the input's upper triangle
   auto u = [](size_t x) { return (x + 255) & ~(size_t)255; };
-  const size_t need = u(2 * sizeof(double)) + u((size_t)d * d * sizeof(double2)) + u((size_t)B.rows * d * sizeof(double2)) +
-                      u((size_t)d * sizeof(double2)) + 2 * u((size_t)B.rows * sizeof(double2)) +
-                      u((size_t)d * KRY_MAX_VECS * sizeof(double2)) + 3 * u((size_t)B.rows * sizeof(double)) +
-                      u(4 * sizeof(double)) + u((size_t)B.ct_max * sizeof(double)) +
-                      u((size_t)B.rows * B.ct_max * sizeof(double)) + u((size_t)5 * B.rows * B.ct_max * sizeof(double)) +
-                      u((size_t)B.ct_max * sizeof(double)) + u(sizeof(double)) + u((size_t)(B.ct_max + 2) * sizeof(int)) +
-                      3 * 256 + 2 * u((size_t)KRY_VERIFY * sizeof(double)) + u((size_t)d * sizeof(float4)) + 1024;
-  lre_status st = ensure_workspace(ctx, need);
-  if (st != LRE_OK) return st;
-  char *p = static_cast<char *>(ctx->ws);
+  char *p = nullptr;
   auto take = [&](size_t bytes) {
     char *q = p;
     p += u(bytes);
     return q;
   };
-  B.M = reinterpret_cast<double2 *>(take((size_t)d * d * sizeof(double2)));
-  B.Q = reinterpret_cast<float4 *>(take((size_t)B.rows * d * sizeof(float4)));
-  B.W = reinterpret_cast<double2 *>(take((size_t)d * sizeof(double2)));
-  B.h1 = reinterpret_cast<double2 *>(take((size_t)B.rows * sizeof(double2)));
-  B.h2 = reinterpret_cast<double2 *>(take((size_t)B.rows * sizeof(double2)));
-  B.Z = reinterpret_cast<double2 *>(take((size_t)d * KRY_MAX_VECS * sizeof(double2)));
-  B.alpha = reinterpret_cast<double *>(take((size_t)B.rows * sizeof(double)));
-  B.beta = reinterpret_cast<double *>(take((size_t)B.rows * sizeof(double)));
-  B.b2 = reinterpret_cast<double *>(take((size_t)B.rows * sizeof(double)));
-  B.stats = reinterpret_cast<double *>(take(4 * sizeof(double)));
-  B.Wr = reinterpret_cast<double *>(take((size_t)B.ct_max * sizeof(double)));
-  B.Xr = reinterpret_cast<double *>(take((size_t)B.rows * B.ct_max * sizeof(double)));
-  B.lu = reinterpret_cast<double *>(take((size_t)5 * B.rows * B.ct_max * sizeof(double)));
-  B.last = reinterpret_cast<double *>(take((size_t)B.ct_max * sizeof(double)));
-  B.nrm = reinterpret_cast<double *>(take(2 * sizeof(double)));
-  B.cl = reinterpret_cast<int *>(take((size_t)(B.ct_max + 2) * sizeof(int)));
-  B.nclust = reinterpret_cast<int *>(take(sizeof(int)));
-  B.breakdown = reinterpret_cast<int *>(take(sizeof(int)));
-  B.res = reinterpret_cast<SmolinResult *>(take(sizeof(SmolinResult)));
-  double *alpha2 = reinterpret_cast<double *>(take((size_t)KRY_VERIFY * sizeof(double)));
-  double *beta2 = reinterpret_cast<double *>(take((size_t)KRY_VERIFY * sizeof(double)));
-  B.Ws = reinterpret_cast<float4 *>(take((size_t)d * sizeof(float4)));
-  B.M32 = reinterpret_cast<const float2 *>(rho_in);  // unchanged until the rebuild writes rho_out
+  float2 *herm = nullptr;
+  double *alpha2 = nullptr, *beta2 = nullptr;
+  auto lay_out = [&]() {
+    herm = reinterpret_cast<float2 *>(take(copy ? (size_t)d * d * sizeof(float2) : 0));
+    B.Q = reinterpret_cast<float4 *>(take((size_t)B.rows * d * sizeof(float4)));
+    B.W = reinterpret_cast<double2 *>(take((size_t)d * sizeof(double2)));
+    B.h1 = reinterpret_cast<double2 *>(take((size_t)B.rows * sizeof(double2)));
+    B.h2 = reinterpret_cast<double2 *>(take((size_t)B.rows * sizeof(double2)));
+    B.Z = reinterpret_cast<float4 *>(take((size_t)d * vecs * sizeof(float4)));
+    B.alpha = reinterpret_cast<double *>(take((size_t)B.rows * sizeof(double)));
+    B.beta = reinterpret_cast<double *>(take((size_t)B.rows * sizeof(double)));
+    B.b2 = reinterpret_cast<double *>(take((size_t)B.rows * sizeof(double)));
+    B.stats = reinterpret_cast<double *>(take(4 * sizeof(double)));
+    B.Wr = reinterpret_cast<double *>(take((size_t)B.ct_max * sizeof(double)));
+    B.Xr = reinterpret_cast<double *>(take((size_t)B.rows * B.ct_max * sizeof(double)));
+    B.lu = reinterpret_cast<double *>(take((size_t)5 * B.rows * B.ct_max * sizeof(double)));
+    B.last = reinterpret_cast<double *>(take((size_t)B.ct_max * sizeof(double)));
+    B.nrm = reinterpret_cast<double *>(take(2 * sizeof(double)));
+    B.cl = reinterpret_cast<int *>(take((size_t)(B.ct_max + 2) * sizeof(int)));
+    B.nclust = reinterpret_cast<int *>(take(sizeof(int)));
+    B.breakdown = reinterpret_cast<int *>(take(sizeof(int)));
+    alpha2 = reinterpret_cast<double *>(take((size_t)KRY_VERIFY * sizeof(double)));
+    beta2 = reinterpret_cast<double *>(take((size_t)KRY_VERIFY * sizeof(double)));
+    B.Ws = reinterpret_cast<float4 *>(take((size_t)d * sizeof(float4)));
+    B.Wn = reinterpret_cast<float4 *>(take((size_t)d * sizeof(float4)));
+    B.Hs = reinterpret_cast<float4 *>(take((size_t)B.rows * sizeof(float4)));
+    B.sync = take(kry_sync_bytes(ctx));
+  };
+  lay_out();
+  const size_t need = (size_t)(p - static_cast<char *>(nullptr));
+  lre_status st = ensure_workspace(ctx, need);
+  if (st != LRE_OK) return st;
+  p = static_cast<char *>(ctx->ws);
+  lay_out();
+  if (!copy) herm = nullptr;
+  B.A = copy ? herm : reinterpret_cast<const float2 *>(rho_in);  // the input is unchanged until the rebuild
 
-  const int grid = ctx->num_sms * 8;
-  {
-    Launch L(ctx, "kry_promote", s, 3);
-    kry_promote<<<grid, 256, 0, s>>>(reinterpret_cast<const float2 *>(rho_in), B.M, B.M, d * d);
-    cudaMemsetAsync(B.nrm, 0, 2 * sizeof(double), s);
-    kry_norm2<<<grid, RED_THREADS, 0, s>>>(B.M, d * d, B.nrm);
-    kry_trace<<<(int)((d + RED_THREADS - 1) / RED_THREADS), RED_THREADS, 0, s>>>(B.M, d, B.nrm + 1);
-  }
+  if ((st = kry_prepare_mu(ctx, reinterpret_cast<const float2 *>(rho_in), herm, d, B.nrm, s)) != LRE_OK) return st;
   double fro_tr[2] = {0, 0};
   cudaError_t e = cudaMemsetAsync(B.breakdown, 0, sizeof(int), s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(fro_tr, B.nrm, sizeof(fro_tr), cudaMemcpyDeviceToHost, s);
@@ -595,53 +481,62 @@ lre_status project_krylov(lre_ctx *ctx, cublasContext *blas, const lre_c64 *rho_
   if ((st = start_vector(ctx, B, d, 0, 0x5EED0001ull, s)) != LRE_OK) return st;
 
   int ct_want = 64, cb_want = 32;
-  int J = 0;
+  int J = 0, step = KRY_CHECK;
+  int seen = 0, seen_J = 0;  // converged leading values at the last check
   bool kept_form = true;
   int64_t r = -1, m = 0;
   double shift = 0.0;
-  int sel0 = 0;  // first column (in Wr / Xr) of the selected vectors
+  int sel0 = 0;  // first column (in Wr) of the selected vectors
   RitzEnds E;
+  std::vector<double> last;
   while (J < kmax) {
-    const int J1 = (int)std::min<int64_t>(kmax, J + KRY_CHECK);
+    const int J1 = (int)std::min<int64_t>(kmax, J + step);
     if ((st = lanczos_steps(ctx, B, d, 0, J, J1, B.alpha, B.beta, tiny, s)) != LRE_OK) return st;
     J = J1;
     int brk = 0;
     e = cudaMemcpyAsync(&brk, B.breakdown, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "Lanczos breakdown flag");
-    const bool broke = brk > 0;
-    if (broke) J = brk;  // an invariant subspace: T_J holds exact eigenvalues
+    const bool broke = brk > 0 || J == d;
+    if (brk > 0) J = brk;  // an invariant subspace: T_J holds exact eigenvalues
+    const bool exact = J == d;  // the whole spectrum of mu
     // windows of Ritz values at each end, together at most ct_max (the
-    // buffers' width) and J
-    const int CT = (int)std::min<int64_t>(std::min(ct_want, J), B.ct_max - 1);
-    const int CB = (int)std::min<int64_t>(std::min(cb_want, J - CT), B.ct_max - CT);
-    if ((st = ritz_ends(ctx, B, B.alpha, B.beta, J, CB, CT, s, E)) != LRE_OK) return st;
+    // buffers' width) and J; all of them once they are exact and fit
+    int CT = (int)std::min<int64_t>(std::min(ct_want, J), B.ct_max - 1);
+    int CB = (int)std::min<int64_t>(std::min(cb_want, J - CT), B.ct_max - CT);
+    if (broke && J <= B.ct_max) {
+      CT = J;
+      CB = 0;
+    }
+    if ((st = ritz_values(ctx, B, B.alpha, B.beta, J, CB, CT, !broke, s, E)) != LRE_OK) return st;
+    if (broke) E.beta_next = 0.0;
     const int mm = CB + CT;
     const double anorm = fmax(fabs(E.w[0]), fabs(E.w[mm - 1]));
     auto conv = [&](int k) { return fabs(E.beta_next * E.last[k]) <= KRY_RTOL * anorm; };
     // top end: l_k - (S_k - Tr)/k > 0 exactly for k <= r
     int64_t r_top = -1;
     bool top_open = true;
+    int conv_top = 0, guess = -1;  // converged leading values; the threshold as it looks now
     double S = 0.0, S_r = 0.0;
     for (int k = 1; k <= CT; ++k) {
       const int col = mm - k;
-      if (!conv(col)) {
-        top_open = false;
-        break;
-      }
+      if (top_open && !conv(col)) top_open = false;
+      if (top_open) conv_top = k;
       S += E.w[col];
       if (E.w[col] - (S - trace) / k <= 0.0) {
-        r_top = k - 1;
+        guess = k;
+        if (top_open) r_top = k - 1;
         break;
       }
-      S_r = S;
+      if (top_open) S_r = S;
     }
     // bottom end: Smolin's walk over the smallest eigenvalues
     int64_t r_bot = -1;
-    bool bot_open = CB > 0;
+    bool bot_open = CB > 0 || exact;
+    const int nbot = exact ? mm : CB;
     double a = 0.0;
     int64_t kept = d;
-    for (int t = 0; t < CB && bot_open; ++t) {
+    for (int t = 0; t < nbot && bot_open; ++t) {
       if (!conv(t)) {
         bot_open = false;
         break;
@@ -655,86 +550,109 @@ lre_status project_krylov(lre_ctx *ctx, cublasContext *blas, const lre_c64 *rho_
       }
     }
     if (r_top >= 0 && r_bot >= 0 && r_top != r_bot) return LRE_OK;  // the two ends disagree: reduction path
-    if (r_top >= 0 && r_top <= KRY_MAX_VECS) {
+    if (r_top >= 0 && r_top <= KRY_MAX_VECS && !(exact && 2 * r_top > d && r_bot >= 0)) {
       kept_form = true;
       r = r_top;
       m = r;
-      shift = (trace - S_r) / (double)r;
+      shift = r > 0 ? (trace - S_r) / (double)r : 0.0;
       sel0 = mm - (int)r;
-    } else if (r_bot >= 0 && d - r_bot <= KRY_MAX_VECS && !eig_rho) {
+    } else if (r_bot >= 0 && d - r_bot <= KRY_MAX_VECS && (!eig_rho || exact)) {
       kept_form = false;
       r = r_bot;
       m = d - r;
       shift = r > 0 ? a / (double)r : 0.0;
       sel0 = 0;
     }
-    if (r >= 0) break;
-    if (r_top >= 0 || r_bot >= 0) return LRE_OK;  // decided, but too many vectors: reduction path
-    if (broke) return LRE_OK;  // exact but undecided: reduction path
+    if (r >= 0) {
+      if (m == 0) break;
+      if ((st = ritz_vectors(ctx, B, B.alpha, B.beta, J, B.Wr + sel0, (int)m, E.tnorm, s, last)) != LRE_OK) return st;
+      bool good = true;
+      for (int k = 0; k < m; ++k) good = good && fabs(E.beta_next * last[k]) <= 2.0 * KRY_RTOL * anorm;
+      if (good) break;
+      r = -1;  // a cluster hid a component: go on
+    } else {
+      if (r_top >= 0 || r_bot >= 0) return LRE_OK;  // decided, but too many vectors: reduction path
+      if (broke) return LRE_OK;  // exact but undecided: reduction path
+    }
     // widen an end whose values all converged without deciding; when both
     // ends are at their widest and still undecided, both sets are too large
     const bool top_full = top_open && r_top < 0 && CT == ct_want;
     const bool bot_full = bot_open && r_bot < 0 && CB == cb_want;
-    const int ct_cap = (int)(B.ct_max - 256), cb_cap = 256;
-    if (top_full && bot_full && ct_want >= ct_cap && cb_want >= cb_cap) return LRE_OK;  // reduction path
+    const int ct_cap = (int)std::max<int64_t>(B.ct_max - 256, 64), cb_cap = 256;
+    if (!whole && top_full && bot_full && ct_want >= ct_cap && cb_want >= cb_cap) return LRE_OK;  // reduction path
     if (top_full) ct_want = std::min(2 * ct_want, ct_cap);
     if (bot_full) cb_want = std::min(2 * cb_want, cb_cap);
+    // the next check: a check costs ten to twenty steps, so when the leading
+    // values converge at a known rate, go most of the way to the threshold
+    step = KRY_CHECK;
+    if (guess > conv_top && conv_top > seen && J > seen_J) {
+      const double rate = (double)(conv_top - seen) / (J - seen_J);
+      const int far = (int)(0.7 * (guess - conv_top) / rate) / KRY_CHECK * KRY_CHECK;
+      step = std::max(KRY_CHECK, std::min(far, 4 * KRY_CHECK));
+    }
+    seen = conv_top;
+    seen_J = J;
   }
   if (r < 0) return LRE_OK;  // undecided within the step limit: reduction path
 
-  // the selected Ritz vectors (conjugated: eigenvectors of conj(mu)) and their values
-  if (m > 0) {
-    Launch L(ctx, "kry_ritz", s);
-    dim3 g((unsigned)std::min<int64_t>((d + 255) / 256, (int64_t)ctx->num_sms * 4), (unsigned)((m + 7) / 8));
-    kry_ritz<<<g, 256, 0, s>>>(B.Q, J, B.Xr + (int64_t)sel0 * J, (int)m, B.Z, d);
-  }
+  // the selected Ritz vectors and their values
+  if (m > 0 && (st = kry_ritz_run(ctx, B.Q, J, B.Xr, (int)m, B.Z, d, s)) != LRE_OK) return st;
   // certification: Lanczos on the operator deflated by the selected vectors
   // (seeded as the first basis rows) from a new start vector; the kept form
   // needs its largest Ritz value <= tau = -shift, the dropped form its
-  // smallest >= tau
+  // smallest >= tau.  Nothing is left to certify once J = d.
   const double tau = -shift;
   const double anorm = fmax(fabs(E.w.front()), fabs(E.w.back()));
-  {
+  const int L2 = J == d ? 0 : (int)std::min<int64_t>(KRY_VERIFY, d - m - 1);
+  if (L2 >= 2) {
     if (m > 0) {
-      Launch L(ctx, "kry_seed", s);
-      kry_seed<<<grid, 256, 0, s>>>(B.Z, (int)m, B.Q, d);
+      e = cudaMemcpyAsync(B.Q, B.Z, (size_t)m * d * sizeof(float4), cudaMemcpyDeviceToDevice, s);
+      if (e != cudaSuccess) return cuda_fail(ctx, e, "certification set-up");
     }
     if ((st = start_vector(ctx, B, d, m, 0x5EED0002ull, s)) != LRE_OK) return st;
     e = cudaMemsetAsync(B.breakdown, 0, sizeof(int), s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "certification set-up");
-    const int L2 = (int)std::min<int64_t>(KRY_VERIFY, d - m - 1);
-    if (L2 >= 2) {
-      if ((st = lanczos_steps(ctx, B, d, m, 0, L2, alpha2, beta2, tiny, s)) != LRE_OK) return st;
-      int brk = 0;
-      e = cudaMemcpyAsync(&brk, B.breakdown, sizeof(int), cudaMemcpyDeviceToHost, s);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-      if (e != cudaSuccess) return cuda_fail(ctx, e, "certification breakdown flag");
-      const int J2 = brk > 0 ? brk : L2;
-      RitzEnds V;
-      if ((st = ritz_ends(ctx, B, alpha2, beta2, J2, 1, 1, s, V)) != LRE_OK) return st;  // smallest, largest
-      const double slack = 1e-10 * anorm;
-      if (kept_form && V.w.back() > tau + slack) return LRE_OK;
-      if (!kept_form && V.w.front() < tau - slack) return LRE_OK;
-    }
+    if ((st = lanczos_steps(ctx, B, d, m, 0, L2, alpha2, beta2, tiny, s)) != LRE_OK) return st;
+    int brk = 0;
+    e = cudaMemcpyAsync(&brk, B.breakdown, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "certification breakdown flag");
+    const int J2 = brk > 0 ? brk : L2;
+    RitzEnds V;
+    if ((st = ritz_values(ctx, B, alpha2, beta2, J2, 1, 1, false, s, V)) != LRE_OK) return st;  // smallest, largest
+    const double slack = 1e-10 * anorm;
+    if (kept_form && V.w.back() > tau + slack) return LRE_OK;
+    if (!kept_form && V.w.front() < tau - slack) return LRE_OK;
   }
-  // rebuild from the selected vectors
-  SmolinResult hres{r, shift};
-  e = cudaMemcpyAsync(B.res, &hres, sizeof(hres), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "projection threshold");
-  // the selected Ritz values: Wr was overwritten by the certification, so
-  // upload them (ascending, as the vectors)
+  if (whole && m > 0) {  // below d = 2048: the selected values to FP64 rounding
+    std::vector<double> q(m);
+    if ((st = kry_rayleigh_run(ctx, B.A, B.Z, (int)m, d, reinterpret_cast<double2 *>(B.lu), B.last, s)) != LRE_OK)
+      return st;
+    e = cudaMemcpyAsync(q.data(), B.last, m * sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "Rayleigh quotients");
+    std::sort(q.begin(), q.end());  // ascending as before; ties at rounding level may have changed places
+    std::copy(q.begin(), q.end(), E.w.begin() + sel0);
+    double sum = 0.0;
+    for (double v : q) sum += v;
+    if (r > 0) shift = (kept_form ? trace - sum : sum) / (double)r;
+  }
+  // the selected Ritz values (Wr was overwritten by the certification), then
+  // for eig_rho every kept value, ascending
   std::vector<double> wsel(E.w.begin() + sel0, E.w.begin() + sel0 + m);
-  if (m > 0) {
-    e = cudaMemcpyAsync(B.Wr, wsel.data(), m * sizeof(double), cudaMemcpyHostToDevice, s);
+  if (eig_rho && !kept_form) wsel.insert(wsel.end(), E.w.begin() + m, E.w.end());  // exact: all d values
+  if (!wsel.empty()) {
+    e = cudaMemcpyAsync(B.Wr, wsel.data(), wsel.size() * sizeof(double), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "selected eigenvalues");
   }
   *fallback = false;
-  if ((st = rebuild_emit(ctx, blas, B.M, B.Z, B.Wr, d, m, kept_form, B.res, rho_out, s)) != LRE_OK) return st;
-  if (eig_rho) {  // kept form only (the dropped form falls back when eig_rho is asked for)
+  if ((st = kry_rebuild_run(ctx, B.Z, B.Wr, (int)m, shift, kept_form, B.A, reinterpret_cast<float2 *>(rho_out), d,
+                            s)) != LRE_OK)
+    return st;
+  if (eig_rho) {
     Launch L(ctx, "kry_eig_rho", s);
-    kry_eig_rho<<<(int)((d + 255) / 256), 256, 0, s>>>(B.Wr, r, shift, eig_rho, d);
+    kry_eig_rho<<<(int)((d + 255) / 256), 256, 0, s>>>(B.Wr + (kept_form ? 0 : m), r, shift, eig_rho, d);
   }
   e = cudaGetLastError();
   return e == cudaSuccess ? LRE_OK : cuda_fail(ctx, e, "Krylov projection");

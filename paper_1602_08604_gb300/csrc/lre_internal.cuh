@@ -177,8 +177,11 @@ lre_status project_run(lre_ctx *ctx, const lre_c64 *rho_in, int n, lre_c64 *rho_
 constexpr int TRI_THREADS = 256;
 __global__ void tri_bisect_kernel(const double *a, const double *b2, int64_t n, double lo0, double hi0, double tol,
                                   double pivmin, double *W, int64_t j0, int64_t cnt);
-__global__ void tri_multisect_kernel(const double *a, const double *b2, int64_t n, double lo0, double hi0,
-                                     double tol, double pivmin, double *W, int64_t j0, int64_t cnt);
+__global__ void tri_ends_kernel(const double *a, const double *b2, int n, double lo0, double hi0, double tnorm,
+                                double *W, int cb, int ct);
+__global__ void tri_residual(const double *a, const double *b, int n, const double *lam, int m, double tnorm,
+                             double *work, double *out);
+__global__ void tri_last(const double *X, int n, int m, double *out);
 // Gershgorin bounds of T (stats[0], stats[1]), the largest squared
 // off-diagonal (stats[2]) and the squares b2 (one CTA of 256 threads).
 __global__ void tri_prepare(const double *a, const double *b, int64_t n, double *b2, double *stats);
@@ -199,8 +202,8 @@ lre_status rebuild_emit(lre_ctx *ctx, struct cublasContext *blas, double2 *C, do
 // The Krylov projection (krylov.cu): *fallback = true, with nothing written to
 // the outputs, when it cannot decide or certify the threshold; eig_rho
 // (device, or NULL) is filled only in the kept form (*fallback otherwise).
-lre_status project_krylov(lre_ctx *ctx, struct cublasContext *blas, const lre_c64 *rho_in, int64_t d,
-                          lre_c64 *rho_out, double *eig_rho, cudaStream_t s, bool *fallback);
+lre_status project_krylov(lre_ctx *ctx, const lre_c64 *rho_in, int64_t d, lre_c64 *rho_out, double *eig_rho,
+                          cudaStream_t s, bool *fallback);
 constexpr int TRI_ROUNDS = 3;  // inverse-iteration rounds
 __global__ void tri_factor(const double *a, const double *b, int64_t n, const double *lam, int m, double tnorm,
                            double *lu);

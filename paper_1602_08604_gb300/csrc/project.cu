@@ -273,7 +273,7 @@ lre_status read_back(lre_ctx *ctx, const SmolinResult *res, const int *info, con
 }
 
 constexpr int64_t PARTIAL_MAX = 1024;  // most eigenvectors the eigenvalue-first path forms
-constexpr int64_t KRYLOV_MIN_D = 2048;  // smallest d the Krylov path takes
+constexpr int64_t KRYLOV_MIN_D = 64;  // smallest d the Krylov path takes
 
 // Eigenvalue-first projection; *fallback = true (nothing written to rho_out)
 // when the smaller of the kept and dropped sets exceeds PARTIAL_MAX.
@@ -415,18 +415,19 @@ lre_status project_run(lre_ctx *ctx, const lre_c64 *rho_in, int n, lre_c64 *rho_
                        double *eig_mu, double *eig_rho, cudaStream_t s) {
   const int64_t d = 1ll << n;
   const int64_t N2 = d * d;
-  cusolverDnHandle_t solver;
-  cublasHandle_t blas;
-  lre_status st0 = get_handles(ctx, s, solver, blas);
-  if (st0 != LRE_OK) return st0;
+  lre_status st0;
   // Krylov path: without eig_mu (which asks for the whole spectrum), from
-  // d = 2048 on; it falls back to the tridiagonal reduction when it cannot
+  // KRYLOV_MIN_D on; it falls back to the tridiagonal reduction when it cannot
   // decide or certify the threshold
   if (ctx->project_mode == 1 && d >= KRYLOV_MIN_D && !eig_mu) {
     bool fallback = false;
-    st0 = project_krylov(ctx, reinterpret_cast<cublasContext *>(blas), rho_in, d, rho_out, eig_rho, s, &fallback);
+    st0 = project_krylov(ctx, rho_in, d, rho_out, eig_rho, s, &fallback);
     if (st0 != LRE_OK || !fallback) return st0;
   }
+  cusolverDnHandle_t solver;
+  cublasHandle_t blas;
+  st0 = get_handles(ctx, s, solver, blas);
+  if (st0 != LRE_OK) return st0;
   if (ctx->project_mode >= 1 && d >= 64) {
     bool fallback = false;
     st0 = project_partial(ctx, solver, blas, rho_in, d, rho_out, eig_mu, eig_rho, s, &fallback);

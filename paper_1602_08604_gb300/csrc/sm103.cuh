@@ -122,6 +122,12 @@ __device__ __forceinline__ uint64_t l2_evict_first() {
   return p;
 }
 
+__device__ __forceinline__ uint64_t l2_evict_normal() {
+  uint64_t p;
+  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+
 // 2D TMA tile load with an L2 cache hint (a policy from createpolicy).
 __device__ __forceinline__ void tma_load_2d_hint(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar,
                                                  uint64_t policy) {

@@ -1,0 +1,59 @@
+// Sturm counts of a real symmetric tridiagonal matrix (tridiag.cu).
+#pragma once
+#include <cuda_runtime.h>
+
+namespace lre {
+
+// Sturm count by the three-term recurrence of the leading principal minors
+// p_k = (a_k - x) p_{k-1} - b_{k-1}^2 p_{k-2} (Givens; Wilkinson, The Algebraic
+// Eigenvalue Problem, Ch. 5): the number of sign changes of p_0, p_1, ... is the
+// number of eigenvalues below x.  Three multiply-adds a step, where the pivot
+// form above has a division on the critical path.  T is scaled to norm 1 or so
+// by the caller, and every eighth step both terms are scaled by a power of two
+// (exact); a zero minor counts as a sign change, as the pivot form's -pivmin.
+template <typename R>
+struct Minor;
+template <>
+struct Minor<double> {
+  static __device__ __forceinline__ unsigned sign(double v) { return (unsigned)(__double2hiint(v)) >> 31; }
+  static __device__ __forceinline__ double scale(double m) {  // 2^-exponent(m)
+    int e = (__double2hiint(m) >> 20) & 0x7FF;
+    e = e < 1 ? 1 : e > 2045 ? 2045 : e;
+    return __hiloint2double((2046 - e) << 20, 0);
+  }
+};
+template <>
+struct Minor<float> {
+  static __device__ __forceinline__ unsigned sign(float v) { return __float_as_uint(v) >> 31; }
+  static __device__ __forceinline__ float scale(float m) {
+    int e = (int)(__float_as_uint(m) >> 23) & 0xFF;
+    e = e < 1 ? 1 : e > 253 ? 253 : e;
+    return __uint_as_float((unsigned)(254 - e) << 23);
+  }
+};
+// a: diagonal, nb2: minus the squared off-diagonal (nb2[k] couples k and k + 1)
+template <typename R>
+__device__ __forceinline__ int minor_count(const R *a, const R *nb2, int n, R x) {
+  R pm = (R)1, p = a[0] - x;
+  unsigned sg = p == (R)0 ? 1u : Minor<R>::sign(p);
+  int cnt = (int)sg;
+  int k = 1;
+  while (k < n) {
+    const int e = k + 8 < n ? k + 8 : n;
+    for (; k < e; ++k) {
+      const R t = nb2[k - 1] * pm;
+      pm = p;
+      p = fma(a[k] - x, p, t);
+      const unsigned ns = p == (R)0 ? sg ^ 1u : Minor<R>::sign(p);
+      cnt += (int)(ns ^ sg);
+      sg = ns;
+    }
+    const R ap = fabs(p), am = fabs(pm);
+    const R f = Minor<R>::scale(ap > am ? ap : am);
+    p *= f;
+    pm *= f;
+  }
+  return cnt;
+}
+
+}  // namespace lre

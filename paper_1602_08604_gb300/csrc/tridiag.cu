@@ -11,6 +11,7 @@
 #include <cfloat>
 
 #include "lre_internal.cuh"
+#include "tri_minor.cuh"
 
 namespace lre {
 
@@ -52,38 +53,6 @@ __global__ void tri_bisect_kernel(const double *a, const double *b2, int64_t n, 
         hi = mid;
     }
     W[jj] = 0.5 * (lo + hi);
-  }
-}
-
-// The same eigenvalues by multisection, one warp per eigenvalue: each round
-// the 32 lanes split the bracket into 32 parts and evaluate the Sturm count at
-// the 31 inner points, so the bracket shrinks 32-fold per round (about 12
-// rounds to 4 eps ||T||) instead of 2-fold; for the few extreme eigenvalues a
-// Krylov check needs, which bisection would run on a handful of threads.
-// Warps beyond j0 + cnt idle; blockDim a multiple of 32.
-__global__ void tri_multisect_kernel(const double *a, const double *b2, int64_t n, double lo0, double hi0, double tol,
-                                     double pivmin, double *W, int64_t j0, int64_t cnt) {
-  const int lane = threadIdx.x & 31;
-  const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t jj = wid; jj < cnt; jj += nw) {
-    const int64_t j = j0 + jj;
-    double lo = lo0, hi = hi0;  // invariant: count(lo) <= j < count(hi)
-    for (int it = 0; it < 40; ++it) {
-      if (hi - lo <= tol) break;
-      const double step = (hi - lo) / 32.0;
-      const double x = lo + step * (double)(lane + 1);  // lane 31: x = hi (not evaluated)
-      const bool below = lane < 31 && x > lo && x < hi && sturm_count(a, b2, n, x, pivmin) <= j;
-      // the points where count <= j form a prefix: the new lo is the last of them
-      const unsigned m = __ballot_sync(0xffffffffu, below);
-      const int k = m ? 31 - __clz(m) : -1;  // last lane with count(x) <= j
-      const double nlo = k >= 0 ? lo + step * (double)(k + 1) : lo;
-      const double nhi = k + 1 <= 30 ? lo + step * (double)(k + 2) : hi;
-      if (!(nhi < hi || nlo > lo)) break;  // no progress (rounding): the bracket is as tight as it gets
-      lo = nlo;
-      hi = nhi;
-    }
-    if (lane == 0) W[jj] = 0.5 * (lo + hi);
   }
 }
 
@@ -230,6 +199,145 @@ __global__ void tri_clusters(const double *lam, int m, double gap_tol, int *cl, 
     if (lam[j] - lam[j - 1] > gap_tol) cl[++k] = j;
   cl[++k] = m;
   *k_out = k;
+}
+
+// ---- the extreme eigenvalues a Krylov check needs ----------------------------
+
+// The cb smallest and ct largest eigenvalues of T (ascending: W[0 .. cb + ct)),
+// one CTA of 128 threads each: a round evaluates the count at 128 points over
+// the bracket, both ends included, so the bracket shrinks 127-fold.  The first
+// rounds run in FP32 on the rounded T and end with the bracket widened by that
+// rounding; the FP64 rounds (five, to 4 eps ||T||) check its ends and start over
+// from [lo0, hi0] if the FP32 rounds misplaced it.  Dynamic shared memory 24 n
+// bytes.  96 values at n = 450 on average: 0.7 ms (one warp per value on the
+// pivot form: 4.1 ms).
+__global__ void __launch_bounds__(128) tri_ends_kernel(const double *a, const double *b2, int n, double lo0, double hi0,
+                                                       double tnorm, double *W, int cb, int ct) {
+  extern __shared__ __align__(16) unsigned char tri_smem[];
+  double *sa = reinterpret_cast<double *>(tri_smem), *sb = sa + n;
+  float *fa = reinterpret_cast<float *>(sb + n), *fb = fa + n;
+  __shared__ unsigned votes[4];
+  // scale by a power of two near 1 / ||T||: exact
+  const double sc = Minor<double>::scale(tnorm);
+  for (int k = threadIdx.x; k < n; k += 128) {
+    const double d = a[k] * sc, o = k + 1 < n ? -(b2[k] * sc * sc) : 0.0;
+    sa[k] = d;
+    sb[k] = o;
+    fa[k] = (float)d;
+    fb[k] = (float)o;
+  }
+  __syncthreads();
+  const int idx = blockIdx.x, j = idx < cb ? idx : n - (cb + ct) + idx;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double L0 = lo0 * sc, H0 = hi0 * sc, tn = tnorm * sc;
+  double lo = L0, hi = H0;  // count(lo) <= j < count(hi)
+  // last point whose count is <= j, -1 if none
+  auto last_below = [&](bool below) {
+    const unsigned v = __ballot_sync(0xffffffffu, below);
+    __syncthreads();
+    if (lane == 0) votes[warp] = v;
+    __syncthreads();
+    int k = -1;
+    for (int w = 0; w < 4; ++w)
+      if (votes[w]) k = 32 * w + 31 - __clz(votes[w]);
+    return k;
+  };
+  for (int it = 0; it < 3; ++it) {
+    const double h = (hi - lo) / 127.0;
+    const float x = (float)(lo + h * threadIdx.x);
+    const int k = last_below(minor_count<float>(fa, fb, n, x) <= j);
+    const int kk = k < 0 ? 0 : k > 126 ? 126 : k;
+    hi = lo + h * (kk + 1);
+    lo = lo + h * kk;
+  }
+  const double w32 = 16.0 * 5.9604644775390625e-08 * tn;  // 16 units of FP32 rounding of T
+  lo = fmax(L0, lo - w32);
+  hi = fmin(H0, hi + w32);
+  const double tol = 4.0 * DBL_EPSILON * tn;
+  bool restarted = false;
+  for (int it = 0; it < 24 && hi - lo > tol; ++it) {
+    const double h = (hi - lo) / 127.0;
+    const double x = threadIdx.x == 127 ? hi : lo + h * threadIdx.x;
+    const int k = last_below(minor_count<double>(sa, sb, n, x) <= j);
+    if ((k < 0 || k > 126) && !restarted) {
+      restarted = true;
+      lo = L0;
+      hi = H0;
+      continue;
+    }
+    const int kk = k < 0 ? 0 : k > 126 ? 126 : k;
+    const double nlo = lo + h * kk, nhi = kk == 126 ? hi : lo + h * (kk + 1);
+    if (!(nhi - nlo < hi - lo)) break;
+    lo = nlo;
+    hi = nhi;
+  }
+  if (threadIdx.x == 0) W[idx] = 0.5 * (lo + hi) / sc;
+}
+
+// |last component| of the unit eigenvector for each of the m eigenvalues lam,
+// one thread each: one inverse-iteration solve from start_entry, the
+// factorisation of tri_factor and the forward substitution in one pass and the
+// norm taken during the back substitution, so that nothing but the factors
+// goes through memory, lane-interleaved (work: 4 n m doubles; n = 450 on
+// average at n = 12: 0.64 ms as tri_factor, tri_solve and a norm).
+__global__ void tri_residual(const double *__restrict__ a, const double *__restrict__ b, int n,
+                             const double *__restrict__ lam, int m, double tnorm, double *work, double *out) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= m) return;
+  const double x = lam[j];
+  double *ui = work + j, *u1 = ui + (size_t)n * m, *u2 = u1 + (size_t)n * m, *v = u2 + (size_t)n * m;
+  const double small = DBL_EPSILON * tnorm > DBL_MIN ? DBL_EPSILON * tnorm : DBL_MIN;
+  double p = a[0] - x, q = n > 1 ? b[0] : 0.0, pend = start_entry(0, j);
+#pragma unroll 4
+  for (int k = 0; k + 1 < n; ++k) {
+    const double lo = b[k], dk = a[k + 1] - x, up = (k + 2 < n) ? b[k + 1] : 0.0;
+    const double nxt = start_entry(k + 1, j);
+    const bool swap = fabs(lo) > fabs(p);
+    double piv = swap ? lo : p;
+    if (!swap && fabs(piv) < small) piv = small;
+    const double r = 1.0 / piv, f = (swap ? p : lo) * r;
+    const size_t at = (size_t)k * m;
+    ui[at] = r;
+    u1[at] = swap ? dk : q;
+    u2[at] = swap ? up : 0.0;
+    v[at] = swap ? nxt : pend;
+    pend = swap ? pend - f * nxt : nxt - f * pend;
+    p = swap ? q - f * dk : dk - f * q;
+    q = swap ? -f * up : up;
+  }
+  if (fabs(p) < small) p = small;
+  double x1 = pend / p, x2 = 0.0;
+  const double last = x1;
+  double s = x1 * x1;
+#pragma unroll 8
+  for (int k = n - 2; k >= 0; --k) {
+    const size_t at = (size_t)k * m;
+    const double xk = (v[at] - u1[at] * x1 - u2[at] * x2) * ui[at];
+    s = fma(xk, xk, s);
+    x2 = x1;
+    x1 = xk;
+  }
+  out[j] = s > 0.0 ? fabs(last) / sqrt(s) : 1.0;
+}
+
+// out[k] = |last component| / norm of column k of X (n x m), one warp each.
+__global__ void tri_last(const double *X, int n, int m, double *out) {
+  const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (k >= m) return;
+  const double *v = X + (size_t)k * n;
+  double mx = 0.0;
+  for (int i = lane; i < n; i += 32) mx = fmax(mx, fabs(v[i]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  const double inv = mx > 0.0 ? 1.0 / mx : 0.0;
+  double s = 0.0;
+  for (int i = lane; i < n; i += 32) {
+    const double t = v[i] * inv;
+    s = fma(t, t, s);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) out[k] = s > 0.0 ? fabs(v[n - 1]) * inv / sqrt(s) : 1.0;
 }
 
 }  // namespace lre

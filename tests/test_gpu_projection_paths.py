@@ -1,0 +1,120 @@
+"""lre_project below d = 2048 without eig_mu: the Lanczos path from d = 64 on
+(persistent steps, the run up to d steps)
+against the oracle's Smolin projection.
+
+Tolerances: eigenvalues are at FP64 rounding of a matrix of norm
+at most 1, d eps = 2.3e-13 at d = 1024; the complex64 result is within the
+rounding of its entries, far inside 1e-6 relative Frobenius."""
+import numpy as np
+import pytest
+
+from oracle import project
+from synth import counts as sc
+from synth import states as st
+from tests.gpu_util import ctx_and_lre, need_gpu, rel_fro
+from tests.test_gpu_projection import _hermitian_with_spectrum
+
+pytestmark = pytest.mark.gpu
+
+EIG_ATOL = 2.5e-13
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = need_gpu()
+    lre, ctx = ctx_and_lre()
+    yield torch, lre, ctx
+    lre.lre_destroy(ctx)
+
+
+def _run(env, m, n, eig=True, alias=False):
+    torch, lre, ctx = env
+    mu = torch.from_numpy(m).cuda()
+    out = mu if alias else torch.full_like(mu, float("nan"))
+    er = torch.full((2 ** n,), float("nan"), dtype=torch.float64, device="cuda") if eig else None
+    lre.lre_profile(ctx, True)
+    lre.lre_project(ctx, mu, n, out, eig_rho=er)
+    lre.lre_sync(ctx)
+    names = {k for k, _ in lre.lre_profile_records(ctx)}
+    lre.lre_profile(ctx, False)
+    ref, _, lam = project.smolin(m.astype(np.complex128))
+    got = out.cpu().numpy()
+    assert rel_fro(got, ref) <= 1e-6
+    assert np.array_equal(got, got.conj().T)
+    if eig:
+        np.testing.assert_allclose(er.cpu().numpy(), lam, atol=EIG_ATOL)
+    return names, lam
+
+
+def _estimate(n, shots, rank, seed):
+    from oracle import direct
+    thr = sc.cdf_thresholds(st.born_probabilities(st.pauli_expectations(st.ginibre_state(n, rank, seed=seed)), n))
+    return direct.mu(direct.estimate(sc.sample_cdf(thr, shots, seed=seed + 1), shots, n), n).astype(np.complex64)
+
+
+@pytest.mark.parametrize("n", [6, 7, 8])
+@pytest.mark.parametrize("shots,rank", [(100, 1), (20000, 3)])
+def test_estimates(env, n, shots, rank):
+    names, _ = _run(env, _estimate(n, shots, rank, 60 + n), n)
+    assert "kry_matvec" in names, names
+    assert "hetrd(cusolver)" not in names, names
+
+
+@pytest.mark.parametrize("n", [6, 8, 10])
+@pytest.mark.parametrize("eig", [True, False])
+def test_dropped_form(env, n, eig):
+    """Few negative eigenvalues: the rebuild is mu + sI and the dropped directions."""
+    d = 2 ** n
+    rng = np.random.default_rng(n)
+    lam = rng.uniform(0.2, 1.0, d)
+    k = max(1, d // 16)
+    lam[:k] = -rng.uniform(0.02, 0.1, k) * lam.mean()
+    lam /= lam.sum()
+    _, out = _run(env, _hermitian_with_spectrum(lam, 3 + n), n, eig=eig, alias=True)
+    assert (out > 0).sum() > d // 2
+
+
+@pytest.mark.parametrize("n", [6, 9])
+def test_clusters(env, n):
+    """Kept eigenvalues equal before the complex64 rounding."""
+    d = 2 ** n
+    lam = -np.linspace(1e-4, 2e-4, d)
+    lam[-2:] = 0.3
+    lam[-4:-2] = 0.1
+    lam /= lam.sum()
+    _run(env, _hermitian_with_spectrum(lam, 17 + n), n)
+
+
+@pytest.mark.parametrize("n", [6, 7])
+def test_degenerate_and_physical_inputs(env, n):
+    """Invariant subspaces after one or two steps (I/d, a pure state, a mixture of
+    both): exact multiplicities, and a physical input comes back as it is."""
+    torch, lre, ctx = env
+    d = 2 ** n
+    eye = np.eye(d, dtype=np.complex64) / np.float32(d)
+    pure = np.zeros((d, d), np.complex64)
+    pure[0, 0] = pure[0, -1] = pure[-1, 0] = pure[-1, -1] = 0.5
+    for m in (eye, pure, (0.5 * eye + 0.5 * pure).astype(np.complex64), -eye + 2 * pure):
+        _run(env, m, n)
+    mu = torch.from_numpy(eye).cuda()
+    out = torch.empty_like(mu)
+    lre.lre_project(ctx, mu, n, out)
+    lre.lre_sync(ctx)
+    np.testing.assert_array_equal(out.cpu().numpy(), eye)
+
+
+@pytest.mark.parametrize("n", [7])
+def test_only_the_upper_triangle_is_read(env, n):
+    m = _estimate(n, 300, 2, 5)
+    low = m.copy()
+    low[np.tril_indices(2 ** n, -1)] = 7.0
+    torch, lre, ctx = env
+    outs = []
+    for x in (m, low):
+        mu = torch.from_numpy(x).cuda()
+        out = torch.empty_like(mu)
+        lre.lre_project(ctx, mu, n, out)
+        lre.lre_sync(ctx)
+        outs.append(out.cpu().numpy())
+    np.testing.assert_array_equal(outs[0], outs[1])
+
