@@ -173,6 +173,10 @@ LastScaleArgs int_assembly_scale(int n, int64_t shots);
 lre_status project_run(lre_ctx *ctx, const lre_c64 *rho_in, int n, lre_c64 *rho_out,
                        double *eig_mu, double *eig_rho, cudaStream_t s);
 
+// The same for n <= 5 in one launch (project_small.cu); eig_mu, eig_rho may be NULL.
+lre_status project_small_run(lre_ctx *ctx, const lre_c64 *rho_in, int n, lre_c64 *rho_out, double *eig_mu,
+                             double *eig_rho, cudaStream_t s);
+
 // tridiagonal eigenproblem kernels (tridiag.cu)
 constexpr int TRI_THREADS = 256;
 __global__ void tri_bisect_kernel(const double *a, const double *b2, int64_t n, double lo0, double hi0, double tol,

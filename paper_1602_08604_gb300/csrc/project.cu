@@ -416,6 +416,7 @@ lre_status project_run(lre_ctx *ctx, const lre_c64 *rho_in, int n, lre_c64 *rho_
   const int64_t d = 1ll << n;
   const int64_t N2 = d * d;
   lre_status st0;
+  if (ctx->project_mode >= 1 && n <= 5) return project_small_run(ctx, rho_in, n, rho_out, eig_mu, eig_rho, s);
   // Krylov path: without eig_mu (which asks for the whole spectrum), from
   // KRYLOV_MIN_D on; it falls back to the tridiagonal reduction when it cannot
   // decide or certify the threshold

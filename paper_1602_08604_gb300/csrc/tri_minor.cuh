@@ -1,4 +1,5 @@
-// Sturm counts of a real symmetric tridiagonal matrix (tridiag.cu).
+// Sturm counts of a real symmetric tridiagonal matrix (tridiag.cu,
+// project_small.cu).
 #pragma once
 #include <cuda_runtime.h>
 

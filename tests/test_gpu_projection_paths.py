@@ -1,8 +1,8 @@
 """lre_project below d = 2048 without eig_mu: the Lanczos path from d = 64 on
-(persistent steps, the run up to d steps)
+(persistent steps, the run up to d steps) and the one-launch path for n <= 5,
 against the oracle's Smolin projection.
 
-Tolerances: eigenvalues are at FP64 rounding of a matrix of norm
+Tolerances: eigenvalues of both paths are at FP64 rounding of a matrix of norm
 at most 1, d eps = 2.3e-13 at d = 1024; the complex64 result is within the
 rounding of its entries, far inside 1e-6 relative Frobenius."""
 import numpy as np
@@ -52,15 +52,16 @@ def _estimate(n, shots, rank, seed):
     return direct.mu(direct.estimate(sc.sample_cdf(thr, shots, seed=seed + 1), shots, n), n).astype(np.complex64)
 
 
-@pytest.mark.parametrize("n", [6, 7, 8])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 6, 7, 8])
 @pytest.mark.parametrize("shots,rank", [(100, 1), (20000, 3)])
 def test_estimates(env, n, shots, rank):
     names, _ = _run(env, _estimate(n, shots, rank, 60 + n), n)
-    assert "kry_matvec" in names, names
+    assert ("project_small" in names) == (n <= 5)
+    assert ("kry_matvec" in names) == (n >= 6)
     assert "hetrd(cusolver)" not in names, names
 
 
-@pytest.mark.parametrize("n", [6, 8, 10])
+@pytest.mark.parametrize("n", [2, 5, 6, 8, 10])
 @pytest.mark.parametrize("eig", [True, False])
 def test_dropped_form(env, n, eig):
     """Few negative eigenvalues: the rebuild is mu + sI and the dropped directions."""
@@ -74,7 +75,7 @@ def test_dropped_form(env, n, eig):
     assert (out > 0).sum() > d // 2
 
 
-@pytest.mark.parametrize("n", [6, 9])
+@pytest.mark.parametrize("n", [3, 5, 6, 9])
 def test_clusters(env, n):
     """Kept eigenvalues equal before the complex64 rounding."""
     d = 2 ** n
@@ -85,7 +86,7 @@ def test_clusters(env, n):
     _run(env, _hermitian_with_spectrum(lam, 17 + n), n)
 
 
-@pytest.mark.parametrize("n", [6, 7])
+@pytest.mark.parametrize("n", [1, 4, 6, 7])
 def test_degenerate_and_physical_inputs(env, n):
     """Invariant subspaces after one or two steps (I/d, a pure state, a mixture of
     both): exact multiplicities, and a physical input comes back as it is."""
@@ -103,7 +104,7 @@ def test_degenerate_and_physical_inputs(env, n):
     np.testing.assert_array_equal(out.cpu().numpy(), eye)
 
 
-@pytest.mark.parametrize("n", [7])
+@pytest.mark.parametrize("n", [4, 7])
 def test_only_the_upper_triangle_is_read(env, n):
     m = _estimate(n, 300, 2, 5)
     low = m.copy()
