@@ -303,6 +303,8 @@ lre_status lre_estimate(lre_ctx *ctx, const void *counts, lre_count_kind kind, c
     counts = dc;
     kind = ck;
   }
+  if (!shots && estimate_small_takes(counts, n, shots_uniform))
+    return estimate_small_run(ctx, counts, kind, n, shots_uniform, theta, rho, s);
   FoldArgs fa{counts, kind, n, shots, shots_uniform, theta, nullptr};
   fa.T = T;
   if ((st = fold_run(ctx, fa, ctx->ws, shared, s)) != LRE_OK) return st;

@@ -169,6 +169,11 @@ struct LastScaleArgs {
 };
 LastScaleArgs int_assembly_scale(int n, int64_t shots);
 
+// ---- steps (i)+(ii) for n <= 6, uniform shots, in one launch (estimate_small.cu) --
+bool estimate_small_takes(const void *counts, int n, int64_t shots);
+lre_status estimate_small_run(lre_ctx *ctx, const void *counts, lre_count_kind kind, int n, int64_t shots,
+                              double *theta, lre_c64 *rho, cudaStream_t s);
+
 // ---- step (iii): rho -> physical rho ----------------------------------------
 lre_status project_run(lre_ctx *ctx, const lre_c64 *rho_in, int n, lre_c64 *rho_out,
                        double *eig_mu, double *eig_rho, cudaStream_t s);
