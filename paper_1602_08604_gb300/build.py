@@ -13,7 +13,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "liblre.so")
-SOURCES = ["abi.cu", "fold.cu", "assemble.cu", "estimate_small.cu", "project.cu", "project_small.cu", "host.cu", "noalloc.cu", "batch.cu", "fold_mma.cu", "fold_tma.cu", "tridiag.cu", "records.cu", "krylov.cu", "krylov_steps.cu", "krylov_vecs.cu", "slab.cu", "ic4.cu", "stream.cu"]
+SOURCES = ["abi.cu", "fold.cu", "assemble.cu", "assemble_top.cu", "estimate_small.cu", "project.cu", "project_small.cu", "host.cu", "noalloc.cu", "batch.cu", "fold_mma.cu", "fold_tma.cu", "tridiag.cu", "records.cu", "krylov.cu", "krylov_steps.cu", "krylov_vecs.cu", "slab.cu", "ic4.cu", "stream.cu"]
 HEADERS = [os.path.join(CSRC, "lre_internal.cuh"), os.path.join(CSRC, "sm103.cuh"),
            os.path.join(CSRC, "passes.cuh"), os.path.join(CSRC, "dfloat.cuh"), os.path.join(CSRC, "krylov.cuh"),
            os.path.join(CSRC, "tri_minor.cuh"),

@@ -308,10 +308,11 @@ lre_status lre_estimate(lre_ctx *ctx, const void *counts, lre_count_kind kind, c
   FoldArgs fa{counts, kind, n, shots, shots_uniform, theta, nullptr};
   fa.T = T;
   if ((st = fold_run(ctx, fa, ctx->ws, shared, s)) != LRE_OK) return st;
-  if (rho)
-    st = int_asm ? assemble_int_run(ctx, T, n, shots_uniform, rho, ctx->ws, s)
-                 : assemble_run(ctx, theta, n, rho, ctx->ws, s);
-  return st;
+  if (!rho) return LRE_OK;
+  if (!int_asm) return assemble_run(ctx, theta, n, rho, ctx->ws, s);
+  const int top = fold_top_qubits(ctx, fa);
+  return top ? assemble_top_run(ctx, T, n, top, shots_uniform, rho, ctx->ws, s)
+             : assemble_int_run(ctx, T, n, shots_uniform, rho, ctx->ws, s);
 }
 
 lre_status lre_assemble(lre_ctx *ctx, const double *theta, int n, lre_c64 *rho, lre_stream stream) {

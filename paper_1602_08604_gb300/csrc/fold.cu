@@ -620,7 +620,14 @@ std::vector<PassPlan> make_plan(int n, lre_count_kind kind, bool weighted, bool 
   }
   while (r > 0) {
     const int jmax = weighted ? 2 : 3;
-    const int J = r < jmax ? r : jmax;
+    int J = r < jmax ? r : jmax;
+    // After the six-qubit first pass of an estimate the last pass takes two
+    // qubits (one at n = 7 and 10): three would hold its 64 sums, quotients and T
+    // in a thread (n = 12: 418 us), and the qubits it takes are ones the assembly
+    // does not have to (assemble_top.cu).  The second pass takes three from
+    // n = 10 on, for its split-plane input.
+    if (!weighted && !parity && t > 0 && plan[0].J == 6 && r > 2)
+      J = (r == 4 && t == 6) || r > 5 ? 3 : r - 2;
     const bool last = (J == r);
     t += J;
     PassPlan p{};
@@ -738,7 +745,7 @@ bool tensor_first_pass(lre_ctx *ctx, const PassPlan &pp, const FoldArgs &a) {
 bool use_planes(lre_ctx *ctx, const std::vector<PassPlan> &plan, const FoldArgs &a) {
   return !plan.empty() && !plan[0].fused9 && tensor_first_pass(ctx, plan[0], a) && plan.size() > 1 &&
          a.shots_uniform * (plan[0].J == 7 ? 2187 : 729) < (1ll << 23) && plan[1].mode == M_STORE &&
-         plan[1].in_t == T_I32 && ctx->generic_tma && plan[1].C % 32 == 0;
+         plan[1].J == 3 && plan[1].in_t == T_I32 && ctx->generic_tma && plan[1].C % 32 == 0;
 }
 
 // The schedule of a fold: the seven-qubit first pass where the raw
@@ -757,6 +764,21 @@ std::vector<PassPlan> fold_plan(lre_ctx *ctx, const FoldArgs &a, bool weighted, 
 }
 
 }  // namespace
+
+// Whether the last pass hands over top-assembled blocks (assemble_top.cu): its
+// qubits, or 0 for plain T.
+int plan_top_qubits(const std::vector<PassPlan> &plan, int n) {
+  if (plan.size() < 2 || plan[0].J == 7) return 0;
+  const PassPlan &l = plan.back();
+  if (l.mode != M_FINAL_U || l.J > 2 || n - l.J < 6) return 0;
+  return (l.in_t == T_I32 || l.in_t == T_I64) && (l.acc_t == T_I32 || l.acc_t == T_I64) ? l.J : 0;
+}
+
+int fold_top_qubits(lre_ctx *ctx, const FoldArgs &a) {
+  if (!a.T || a.shots || a.S) return 0;
+  const bool aligned16 = (reinterpret_cast<uintptr_t>(a.counts) & 15) == 0;
+  return plan_top_qubits(fold_plan(ctx, a, false, false, a.shots_uniform, aligned16), a.n);
+}
 
 int64_t fold_split_rows(lre_ctx *ctx, const FoldArgs &a) {
   if (a.shots) return 0;
@@ -939,6 +961,11 @@ lre_status fold_run(lre_ctx *ctx, const FoldArgs &a, void *ws, size_t ws_bytes, 
       gp.hi_from = planes_hi_from(a.shots_uniform);
       gp.hi_letters = plan[0].J == 7 ? 7 : 6;
       gp.top7 = plan[0].J == 7 ? 1 : 0;  // the seven-qubit first pass folded qubit n
+      if (gp.T && k + 1 == plan.size() && plan_top_qubits(plan, a.n) > 0) {
+        const lre_status st = fold_final_top_run(ctx, gp, pp.J, pp.in_t, pp.acc_t, s);
+        if (st != LRE_OK) return st;
+        break;
+      }
       const int in_t = (planes && k == 1) ? (int)T_I24P : pp.in_t;
       lre_status tst = ctx->generic_tma ? tma_pass(ctx, gp, pp.J, in_t, pp.acc_t, pp.mode, pp.weight, s)
                                         : LRE_ERR_UNSUPPORTED;

@@ -144,7 +144,11 @@ lre_status estimate_host_run(lre_ctx *ctx, const void *host_in, int host_kind, i
   if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, ctx->ev_theta, 0);
   if (e == cudaSuccess) e = cudaMemcpyAsync(theta_host, theta, theta_bytes, cudaMemcpyDeviceToHost, cs);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "theta copy-back");
-  if (rho_host && (st = assemble_int_run(ctx, T, n, shots, rho, ws, s)) != LRE_OK) return st;
+  if (rho_host) {
+    const int top = fold_top_qubits(ctx, rest);
+    st = top ? assemble_top_run(ctx, T, n, top, shots, rho, ws, s) : assemble_int_run(ctx, T, n, shots, rho, ws, s);
+    if (st != LRE_OK) return st;
+  }
   if (rho_host) e = cudaMemcpyAsync(rho_host, rho, rho_bytes, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(cs);

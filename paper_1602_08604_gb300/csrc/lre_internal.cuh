@@ -164,6 +164,12 @@ const char *noalloc_last_error();
 // Exact-integer variant for uniform shots: T_i = S_i 3^(n-k_i) (= t_i N 3^n).
 lre_status assemble_int_run(lre_ctx *ctx, const int64_t *T, int n, int64_t shots, lre_c64 *rho,
                             void *ws, cudaStream_t s);
+// The same from the blocks the last fold pass hands over (assemble_top.cu):
+// fold_top_qubits says how many qubits that pass assembles for these arguments
+// (0: a.T is plain T, for assemble_int_run).
+int fold_top_qubits(lre_ctx *ctx, const FoldArgs &a);
+lre_status assemble_top_run(lre_ctx *ctx, const int64_t *T, int n, int J, int64_t shots, lre_c64 *rho, void *ws,
+                            cudaStream_t s);
 struct LastScaleArgs {
   float sh, sl;  // 1/(2^n N 3^n) = sh + sl
 };

@@ -291,21 +291,21 @@ __device__ __forceinline__ void fold_emit(const GenParams &P, const AccT (&acc)[
   }
 }
 
-// One output column (ah, oh, c) of a fold pass.  VEC: first pass (C == 1),
-// the row's 2^J outcomes loaded as one vector.
-template <int J, typename InT, typename AccT, int MODE, bool WEIGHT, bool COHERENT = false, bool VEC = false>
-__device__ __forceinline__ void fold_item(const GenParams &P, int64_t item, const DivTables *tab = nullptr) {
+// The 4^J sums of one output column (ah, oh, c) of a fold pass.  VEC: first pass
+// (C == 1), the row's 2^J outcomes loaded as one vector.
+template <int J, typename InT, typename AccT, bool WEIGHT, bool COHERENT = false, bool VEC = false>
+__device__ __forceinline__ void fold_sums(const GenParams &P, int64_t item, AccT (&acc)[1 << (2 * J)], int64_t &ahoh,
+                                          int64_t &c) {
   constexpr int NA = (J == 1) ? 3 : (J == 2) ? 9 : 27;
   constexpr int NO = 1 << J;
   constexpr int NP = 1 << (2 * J);
   const InT *__restrict__ in = static_cast<const InT *>(P.in);
   const int64_t row_stride = (1ll << P.r) * P.C;  // al stride
-  const int64_t c = item % P.C;
-  const int64_t ahoh = item / P.C;
+  c = item % P.C;
+  ahoh = item / P.C;
   const int64_t oh = ahoh % P.n_oh;
   const int64_t ah = ahoh / P.n_oh;
   const int64_t base = ((ah * NA) << P.r) * P.C + (oh * NO) * P.C + c;
-  AccT acc[NP];
 #pragma unroll
   for (int p = 0; p < NP; ++p) acc[p] = 0;
 #pragma unroll
@@ -331,6 +331,14 @@ __device__ __forceinline__ void fold_item(const GenParams &P, int64_t item, cons
       for (int m = 0; m < NO; ++m) acc[block_pauli(al, m, J)] += v[m];
     }
   }
+}
+
+// One output column of a fold pass.
+template <int J, typename InT, typename AccT, int MODE, bool WEIGHT, bool COHERENT = false, bool VEC = false>
+__device__ __forceinline__ void fold_item(const GenParams &P, int64_t item, const DivTables *tab = nullptr) {
+  AccT acc[1 << (2 * J)];
+  int64_t ahoh, c;
+  fold_sums<J, InT, AccT, WEIGHT, COHERENT, VEC>(P, item, acc, ahoh, c);
   fold_emit<J, AccT, MODE>(P, acc, ahoh, c, tab);
 }
 
@@ -338,6 +346,14 @@ __device__ __forceinline__ void fold_item(const GenParams &P, int64_t item, cons
 // multiple of 32; LRE_ERR_UNSUPPORTED (nothing launched) for other passes.
 lre_status tma_pass(lre_ctx *ctx, const GenParams &P, int J, int in_t, int acc_t, int mode, bool weight,
                     cudaStream_t s);
+
+}  // namespace passes
+
+// The last fold pass with its qubits assembled (assemble_top.cu): theta, and in
+// P.T the 2^J x 2^J blocks for assemble_top_run.
+lre_status fold_final_top_run(lre_ctx *ctx, const passes::GenParams &P, int J, int in_t, int acc_t, cudaStream_t s);
+
+namespace passes {
 
 // ---- step (ii) ----------------------------------------------------------------
 struct NumF64 {
@@ -516,10 +532,9 @@ __device__ __forceinline__ void m2(V (&v)[16]) {
 // complex64 with the final scale.
 // asm_low6_finish: the same after S holds the block's coefficients (and the
 // CTA has synchronised): the butterflies and the writes.
-template <class Num, bool LAST, bool HERM = false>
-__device__ __forceinline__ void asm_low6_finish(void *__restrict__ out, int64_t blk, typename Num::V *S,
-                                                const LastScale &scale) {
-  using V = typename Num::V;
+// asm_low6_rounds: the butterflies alone.
+template <typename V>
+__device__ __forceinline__ void asm_low6_rounds(V *S) {
   const int tid = threadIdx.x;
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
@@ -533,14 +548,27 @@ __device__ __forceinline__ void asm_low6_finish(void *__restrict__ out, int64_t 
     for (int u = 0; u < 16; ++u) S[pad16(lo | (u << sh) | (hi << (sh + 4)))] = v[u];
     __syncthreads();
   }
-  // S[pos], pos digit q = 2 r_q + c_q  ->  out[R_lo * 64 + C_lo]
+}
+// Place of entry (R, C) of the 64 x 64 block in the tile: digit q = 2 r_q + c_q.
+__device__ __forceinline__ int low6_place(int R, int C) {
+  int pos = 0;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) pos |= ((((R >> q) & 1) << 1) | ((C >> q) & 1)) << (2 * q);
+  return pos;
+}
+
+template <class Num, bool LAST, bool HERM = false>
+__device__ __forceinline__ void asm_low6_finish(void *__restrict__ out, int64_t blk, typename Num::V *S,
+                                                const LastScale &scale) {
+  using V = typename Num::V;
+  const int tid = threadIdx.x;
+  asm_low6_rounds(S);
+  // the tile -> out[R_lo * 64 + C_lo]
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     const int o = tid + 256 * k;
     const int R = o >> 6, C = o & 63;
-    int pos = 0;
-#pragma unroll
-    for (int q = 0; q < 6; ++q) pos |= ((((R >> q) & 1) << 1) | ((C >> q) & 1)) << (2 * q);
+    const int pos = low6_place(R, C);
     if constexpr (LAST)
       static_cast<float2 *>(out)[blk * 4096 + o] = to_c64(S[pad16(pos)], scale);
     else if (!HERM || herm_stored(R, C))  // HERM: the stored part of the 64 x 64 block

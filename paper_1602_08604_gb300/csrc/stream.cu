@@ -109,7 +109,9 @@ extern "C" lre_status lre_stream_end(lre_ctx *ctx, double *theta, lre_c64 *rho, 
   ctx->stream_active = 0;
   lre_status st = fold_run(ctx, rest, ctx->ws, shared, s);
   if (st != LRE_OK || !rho) return st;
-  return assemble_int_run(ctx, T, ctx->stream_n, ctx->stream_shots, rho, ctx->ws, s);
+  const int top = fold_top_qubits(ctx, rest);
+  return top ? assemble_top_run(ctx, T, ctx->stream_n, top, ctx->stream_shots, rho, ctx->ws, s)
+             : assemble_int_run(ctx, T, ctx->stream_n, ctx->stream_shots, rho, ctx->ws, s);
 }
 
 extern "C" lre_status lre_stream_checkpoint(lre_ctx *ctx, void *host, size_t bytes, size_t *needed,
