@@ -3,14 +3,14 @@
 //
 // Per qubit the map from the Pauli letter coefficients (I, X, Y, Z) to the
 // 2x2 block entries (row bit r, column bit c) is
-//     (0,0) = I + Z   (0,1) = X - iY   (1,0) = X + iY   (1,1) = I - Z
-// (times 1/2), so rho = 2^-n M^{(x)n} t.  The paper instead sums, for each
+//     (0,0) = I + Z   (0,1) = X - iY   (1,0) = X + iY   (1,1) = I - Z,
+// so rho = 2^-n M^{(x)n} t.  The paper instead sums, for each
 // output element, the 2^n strings sharing its nonzero pattern (Sec. IV, the
 // 2^n x-mask groups); the butterfly reaches the same sums in O(n 4^n).
 //
 // Two number types run the same passes:
-//   * FP64 (lre_assemble on an arbitrary theta): FP64 butterflies with the
-//     1/2 per qubit, rounded once to complex64 at the end;
+//   * FP64 (lre_assemble on an arbitrary theta): FP64 butterflies, scaled by
+//     2^-n (exact) and rounded once to complex64 at the end;
 //   * exact int64 (lre_estimate with uniform shots): the fold hands over
 //     T_i = S_i 3^(n-k_i) = t_i N 3^n, integers; the butterflies are exact
 //     integer adds and the last pass scales by 1/(2^n N 3^n) once.  GB300's
@@ -315,7 +315,7 @@ lre_status assemble_preload() {
 
 lre_status assemble_run(lre_ctx *ctx, const double *theta, int n, lre_c64 *rho, void *ws,
                         cudaStream_t s) {
-  return run_passes<NumF64>(ctx, theta, n, rho, ws, LastScale{0.f, 0.f}, s);
+  return run_passes<NumF64>(ctx, theta, n, rho, ws, LastScale{(float)(1.0 / (double)(1ll << n)), 0.f}, s);
 }
 
 lre_status assemble_int_run(lre_ctx *ctx, const int64_t *T, int n, int64_t shots, lre_c64 *rho,

@@ -150,7 +150,8 @@ __global__ void __launch_bounds__(256) top_low6(TopArgs P) {
       S[pad16(i)] = load_block(P.in, C, B, b, Pp * 4096 + i);
     }
     __syncthreads();
-    asm_low6_rounds(S);
+    if (b < B) asm_low6_rounds<true>(S);
+    else asm_low6_rounds<false>(S);
     const Block bl = block_of(b, B);
 #pragma unroll
     for (int k = 0; k < 16; ++k) {

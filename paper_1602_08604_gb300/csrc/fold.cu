@@ -132,6 +132,182 @@ __global__ void __launch_bounds__(P1_THREADS, 2)
 }
 
 // ---------------------------------------------------------------------------
+// Per-basis shots: the first six qubits of the FP64-weighted fold in one pass (in
+// the place of three two-qubit passes).
+//
+// The weight 1/N_b multiplies a basis' parity sums, so the parity transform of all
+// six outcome bits can stay in integers (int32 up to four counts as in the
+// two-qubit pass, int64 beyond), and then every (basis, mask) value is added to
+// exactly one letter: one FP64 multiply-add per count, and for the upper three
+// digits 27 additions per 27 values -- 1.3 FP64 operations a count, where the three
+// passes needed 2.9 and moved their FP64 intermediates through HBM.  The FP64 pipe
+// (about 1.75 operations a cycle and SM) bounds it: 154 us of the 201 us it takes at
+// n = 10, where the three passes took 470; one CTA an SM with all 64 sums live and
+// no row loaded ahead took 557.
+//   level A: thread (alB, olB) reads 27 rows of 8 outcomes; three butterflies in
+//     registers, three across the eight lanes of its rows by shuffles, which leave
+//     lane mB with upper mask mB and the eight lower masks; 64 FP64 sums, 32 of
+//     them live at a time, so that two CTAs fit an SM.
+//   level B: warp w takes upper mask w: per lower letter the 27 upper digits.
+// ---------------------------------------------------------------------------
+// |v| < 2^53 to FP64 in integer operations (the conversions of the FP64 pipe would
+// double its load).
+__device__ __forceinline__ double int_to_double(int64_t v) {
+  const uint64_t a = v < 0 ? (uint64_t)(-v) : (uint64_t)v;
+  const int lz = __clzll((long long)a) & 63;
+  const uint64_t m = (a << lz) << 1;  // the leading one shifted out
+  const uint64_t bits = ((uint64_t)(1023 + 63 - lz) << 52) | (m >> 12);
+  return a == 0 ? 0.0 : __longlong_as_double((long long)(bits | ((uint64_t)v & (1ull << 63))));
+}
+__device__ __forceinline__ double int_to_double(int32_t v) {
+  const uint32_t a = v < 0 ? 0u - (uint32_t)v : (uint32_t)v;
+  const int lz = __clz((int)a) & 31;
+  const uint32_t m = (a << lz) << 1;
+  const uint32_t hi = ((uint32_t)(1023 + 31 - lz) << 20) | (m >> 12) | ((uint32_t)v & 0x80000000u);
+  return a == 0 ? 0.0 : __hiloint2double((int)hi, (int)(m << 20));
+}
+
+// Parity transform over the lanes' three bits: lane L of each eight ends with mask L.
+template <typename V>
+__device__ __forceinline__ void lane_wht(V (&v)[8], int olB) {
+#pragma unroll
+  for (int h = 1; h < 8; h <<= 1) {
+    const V s = (olB & h) ? (V)-1 : (V)0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      V o;
+      if constexpr (sizeof(V) == 8) o = __shfl_xor_sync(0xffffffffu, (long long)v[q], h);
+      else o = __shfl_xor_sync(0xffffffffu, v[q], h);
+      v[q] = o + ((v[q] ^ s) - s);  // o - v on the lanes with the bit, o + v on the others
+    }
+  }
+}
+
+// Upper three digits of mask MB for one lower letter: z[alB * 8] -> the 3^|MB| letters of mask MB.
+template <int MB>
+__device__ __forceinline__ void weighted_upper(const double *z, double *out) {
+  double acc[64];
+#pragma unroll
+  for (int p = 0; p < 64; ++p) acc[p] = 0.0;
+#pragma unroll
+  for (int al = 0; al < 27; ++al) acc[block_pauli(al, MB, 3)] += z[al * 8 + MB];
+#pragma unroll
+  for (int p = 0; p < 64; ++p) {
+    const int m = ((p & 3) ? 1 : 0) | ((p & 12) ? 2 : 0) | ((p & 48) ? 4 : 0);
+    if (m == MB) out[p * 64] = acc[p];
+  }
+}
+
+template <typename InT>
+__global__ void __launch_bounds__(P1_THREADS, 2)
+    fold_first6_weighted(const InT *__restrict__ counts, const double *__restrict__ wgt, double *__restrict__ out, int n,
+                         int64_t num_tiles) {
+  extern __shared__ double Zw[];  // [64][P1_ZSTRIDE]
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int64_t d = 1ll << n;
+  const int64_t n_oh = d >> 6;
+  const int alB = t < 216 ? t >> 3 : 26, olB = t & 7;  // the last warp's spare lanes repeat a row
+  for (int64_t tile = blockIdx.x; tile < num_tiles; tile += gridDim.x) {
+    const int64_t ah = tile / n_oh, oh = tile - ah * n_oh;
+    if (warp < 7) {
+      const InT *row = counts + (ah * 729 + alB * 27) * d + oh * 64 + olB * 8;
+      const double *w = wgt + ah * 729 + alB * 27;
+      // letters of the lower two digits: s0 with the third letter I, over all its
+      // axes; s1 with the third letter the axis at hand, done after nine rows
+      double s0[16], s1[16];
+#pragma unroll
+      for (int p = 0; p < 16; ++p) s0[p] = 0.0;
+      int32_t next[8];
+      load_row8<InT>(row, next);
+      double wn = __ldg(w);
+#pragma unroll 1
+      for (int a2 = 0; a2 < 3; ++a2) {
+#pragma unroll
+        for (int p = 0; p < 16; ++p) s1[p] = 0.0;
+#pragma unroll
+        for (int a01 = 0; a01 < 9; ++a01) {
+          int32_t c[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) c[q] = next[q];
+          const double wb = wn;
+          if (a01 < 8 || a2 < 2) {  // the next row, in flight during this one
+            row += d;
+            load_row8<InT>(row, next);
+            wn = __ldg(++w);
+          }
+          uint32_t any = 0;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) any |= (uint32_t)c[q];
+          // two bits in int32, as the two-qubit pass; the other four too while 64
+          // counts below 2^25 cannot pass 2^31, else in int64
+#pragma unroll
+          for (int q = 0; q < 8; q += 4) {
+            const int32_t a = c[q] + c[q + 1], b = c[q] - c[q + 1], e = c[q + 2] + c[q + 3], f = c[q + 2] - c[q + 3];
+            c[q] = a + e;
+            c[q + 1] = b + f;
+            c[q + 2] = a - e;
+            c[q + 3] = b - f;
+          }
+          double x[8];
+          if (__all_sync(0xffffffffu, any < (1u << 25))) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const int32_t a = c[q], b = c[q + 4];
+              c[q] = a + b;
+              c[q + 4] = a - b;
+            }
+            lane_wht(c, olB);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) x[q] = int_to_double(c[q]);
+          } else {
+            int64_t v[8];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              v[q] = (int64_t)c[q] + c[q + 4];
+              v[q + 4] = (int64_t)c[q] - c[q + 4];
+            }
+            lane_wht(v, olB);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) x[q] = int_to_double(v[q]);
+          }
+#pragma unroll
+          for (int m = 0; m < 8; ++m) {
+            double &s = (m & 4) ? s1[block_pauli(a01, m & 3, 2)] : s0[block_pauli(a01, m & 3, 2)];
+            s = fma(x[m], wb, s);
+          }
+        }
+        if (t < 216) {
+#pragma unroll
+          for (int p = 0; p < 16; ++p) Zw[(p + 16 * (a2 + 1)) * P1_ZSTRIDE + t] = s1[p];
+        }
+      }
+      if (t < 216) {
+#pragma unroll
+        for (int p = 0; p < 16; ++p) Zw[p * P1_ZSTRIDE + t] = s0[p];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int tl = lane + 32 * h;  // lower letter
+      const double *z = Zw + tl * P1_ZSTRIDE;
+      double *o = out + tile * 4096 + tl;
+      switch (warp) {
+        case 0: weighted_upper<0>(z, o); break;
+        case 1: weighted_upper<1>(z, o); break;
+        case 2: weighted_upper<2>(z, o); break;
+        case 3: weighted_upper<3>(z, o); break;
+        case 4: weighted_upper<4>(z, o); break;
+        case 5: weighted_upper<5>(z, o); break;
+        case 6: weighted_upper<6>(z, o); break;
+        default: weighted_upper<7>(z, o); break;
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------------------
 // The same first pass as a warp-specialised TMA pipeline (the ALU first pass
 // wherever the tensor-core one, fold_mma.cu, does not apply).
 //   warp 0      producer: one 2D TMA load per sub-tile (81 rows x 64
@@ -831,6 +1007,25 @@ lre_status fold_run(lre_ctx *ctx, const FoldArgs &a, void *ws, size_t ws_bytes, 
   const bool planes = use_planes(ctx, plan, a);
   const void *in = a.counts;
   size_t k_begin = 0, k_end = plan.size();
+  // per-basis shots, n >= 7: the plan's first three passes (two qubits each) as one
+  if (weighted && aligned16 && plan.size() >= 4 && plan[0].J + plan[1].J + plan[2].J == 6) {
+    const int64_t tiles = ipow(3, a.n - 6) << (a.n - 6);
+    const int smem = 64 * P1_ZSTRIDE * (int)sizeof(double);
+    const int grid = (int)(tiles < 2 * ctx->num_sms ? tiles : 2 * ctx->num_sms);
+    double *out = static_cast<double *>(bufA);  // where the third pass writes
+    Launch L(ctx, "fold_first6_weighted", s);
+    if (a.kind == LRE_COUNTS_I16) {
+      cudaFuncSetAttribute(fold_first6_weighted<int16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      fold_first6_weighted<int16_t><<<grid, P1_THREADS, smem, s>>>(static_cast<const int16_t *>(in), wgt, out, a.n, tiles);
+    } else {
+      cudaFuncSetAttribute(fold_first6_weighted<int32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      fold_first6_weighted<int32_t><<<grid, P1_THREADS, smem, s>>>(static_cast<const int32_t *>(in), wgt, out, a.n, tiles);
+    }
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "weighted first pass launch");
+    in = out;
+    k_begin = 3;
+  }
   if (a.stage != 0) {
     if (fold_split_rows(ctx, a) == 0) return LRE_ERR_UNSUPPORTED;
     if (a.stage == 1) {

@@ -8,8 +8,9 @@
 // of the three axes, X/Y/Z = the matching axis); the last pass divides by
 // N 3^k (k identity letters) and can also emit T_i = S_i 3^(n-k).
 // Step (ii) (Eq. 4): a pass applies the per-qubit map (I,X,Y,Z) ->
-// (I+Z, X-iY, X+iY, I-Z) (times 1/2 in FP64; unscaled on exact integers) to
-// J qubits of [P_hi][R_lo][C_lo].
+// (I+Z, X-iY, X+iY, I-Z) to J qubits of [P_hi][R_lo][C_lo]; the last pass scales
+// (by 2^-n in FP64: exact, as the 1/2 of each qubit would be, at a tenth of its
+// multiplications).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -366,7 +367,7 @@ struct NumI64 {
 };
 
 struct LastScale {
-  float sh, sl;  // 1/(2^n N 3^n) = sh + sl (integer path only)
+  float sh, sl;  // integer path: 1/(2^n N 3^n) = sh + sl; FP64 path: sh = 2^-n
 };
 
 __device__ __forceinline__ double2 mk(double a, double b) { return make_double2(a, b); }
@@ -376,10 +377,10 @@ __device__ __forceinline__ longlong2 mk(long long a, long long b) { return make_
 //   -i*Y = (Y.y, -Y.x);  +i*Y = (-Y.y, Y.x)
 __device__ __forceinline__ void m_qubit(double2 vI, double2 vX, double2 vY, double2 vZ, double2 &o00,
                                         double2 &o01, double2 &o10, double2 &o11) {
-  o00 = mk(0.5 * (vI.x + vZ.x), 0.5 * (vI.y + vZ.y));
-  o11 = mk(0.5 * (vI.x - vZ.x), 0.5 * (vI.y - vZ.y));
-  o01 = mk(0.5 * (vX.x + vY.y), 0.5 * (vX.y - vY.x));
-  o10 = mk(0.5 * (vX.x - vY.y), 0.5 * (vX.y + vY.x));
+  o00 = mk(vI.x + vZ.x, vI.y + vZ.y);
+  o11 = mk(vI.x - vZ.x, vI.y - vZ.y);
+  o01 = mk(vX.x + vY.y, vX.y - vY.x);
+  o10 = mk(vX.x - vY.y, vX.y + vY.x);
 }
 __device__ __forceinline__ void m_qubit(longlong2 vI, longlong2 vX, longlong2 vY, longlong2 vZ,
                                         longlong2 &o00, longlong2 &o01, longlong2 &o10, longlong2 &o11) {
@@ -414,8 +415,8 @@ __device__ __forceinline__ float scaled(long long v, const LastScale &s) {
   const float vl = __fadd_rn(__fsub_rn(X, __fsub_rn(vh, bv)), __fsub_rn(fc, bv));
   return __fmaf_rn(vh, s.sh, __fmaf_rn(vh, s.sl, vl * s.sh));
 }
-__device__ __forceinline__ float2 to_c64(double2 v, const LastScale &) {
-  return make_float2((float)v.x, (float)v.y);
+__device__ __forceinline__ float2 to_c64(double2 v, const LastScale &s) {
+  return make_float2((float)(v.x * (double)s.sh), (float)(v.y * (double)s.sh));
 }
 __device__ __forceinline__ float2 to_c64(longlong2 v, const LastScale &s) {
   return make_float2(scaled(v.x, s), scaled(v.y, s));
@@ -525,6 +526,36 @@ __device__ __forceinline__ void m2(V (&v)[16]) {
   }
 }
 
+__device__ __forceinline__ double zero_of(double) { return 0.0; }
+__device__ __forceinline__ long long zero_of(long long) { return 0; }
+// m2 on values that are still real (the first two qubits): digit 0 needs two
+// additions instead of eight, and half of digit 1's four instead of eight.
+template <typename V>
+__device__ __forceinline__ void m2_real(V (&v)[16]) {
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    const auto i = v[4 * h].x, x = v[4 * h + 1].x, y = v[4 * h + 2].x, z = v[4 * h + 3].x;
+    v[4 * h] = mk(i + z, zero_of(i));
+    v[4 * h + 1] = mk(x, -y);
+    v[4 * h + 2] = mk(x, y);
+    v[4 * h + 3] = mk(i - z, zero_of(i));
+  }
+#pragma unroll
+  for (int u0 = 0; u0 < 4; ++u0) {
+    V a, b, c, d;
+    if (u0 == 0 || u0 == 3) {
+      const auto i = v[u0].x, x = v[4 + u0].x, y = v[8 + u0].x, z = v[12 + u0].x;
+      a = mk(i + z, zero_of(i));
+      b = mk(x, -y);
+      c = mk(x, y);
+      d = mk(i - z, zero_of(i));
+    } else {
+      m_qubit(v[u0], v[4 + u0], v[8 + u0], v[12 + u0], a, b, c, d);
+    }
+    v[u0] = a; v[4 + u0] = b; v[8 + u0] = c; v[12 + u0] = d;
+  }
+}
+
 // Qubits 0..5 of block `blk` (4096 consecutive coefficients of the first
 // pass's input) -> [R_lo 64][C_lo 64] at out + blk * 4096, through the padded
 // shared tile S (4096 + 256 entries).  All 256 threads of the CTA call it
@@ -532,8 +563,8 @@ __device__ __forceinline__ void m2(V (&v)[16]) {
 // complex64 with the final scale.
 // asm_low6_finish: the same after S holds the block's coefficients (and the
 // CTA has synchronised): the butterflies and the writes.
-// asm_low6_rounds: the butterflies alone.
-template <typename V>
+// asm_low6_rounds: the butterflies alone (REAL: the tile holds real values).
+template <bool REAL, typename V>
 __device__ __forceinline__ void asm_low6_rounds(V *S) {
   const int tid = threadIdx.x;
 #pragma unroll
@@ -543,7 +574,8 @@ __device__ __forceinline__ void asm_low6_rounds(V *S) {
     V v[16];
 #pragma unroll
     for (int u = 0; u < 16; ++u) v[u] = S[pad16(lo | (u << sh) | (hi << (sh + 4)))];
-    m2(v);
+    if (REAL && r == 0) m2_real(v);
+    else m2(v);
 #pragma unroll
     for (int u = 0; u < 16; ++u) S[pad16(lo | (u << sh) | (hi << (sh + 4)))] = v[u];
     __syncthreads();
@@ -562,7 +594,7 @@ __device__ __forceinline__ void asm_low6_finish(void *__restrict__ out, int64_t 
                                                 const LastScale &scale) {
   using V = typename Num::V;
   const int tid = threadIdx.x;
-  asm_low6_rounds(S);
+  asm_low6_rounds<true>(S);
   // the tile -> out[R_lo * 64 + C_lo]
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
