@@ -139,5 +139,49 @@ __device__ __forceinline__ float2 split1(double v) {
   return make_float2(h, __double2float_rn(v - (double)h));
 }
 
+// ---- real double-float values -------------------------------------------------
+struct D1 {
+  float h, l;
+};
+__device__ __forceinline__ D1 fast_norm(float h, float l) {  // |h| >= |l|
+  const float t = __fadd_rn(h, l);
+  return {t, __fsub_rn(l, __fsub_rn(t, h))};
+}
+__device__ __forceinline__ D1 operator-(D1 a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ D1 operator+(D1 a, D1 b) {
+  const float t = __fadd_rn(a.h, b.h), bp = __fsub_rn(t, a.h);
+  const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(t, bp)), __fsub_rn(b.h, bp));
+  return fast_norm(t, __fadd_rn(e, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ D1 operator-(D1 a, D1 b) { return a + (-b); }
+__device__ __forceinline__ D1 operator*(D1 a, D1 b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return fast_norm(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
+}
+__device__ __forceinline__ D1 d1(double v) {
+  const float2 s = split1(v);
+  return {s.x, s.y};
+}
+__device__ __forceinline__ double value(D1 a) { return (double)a.h + (double)a.l; }
+// 1 / a and 1 / sqrt(a): the FP32 value and one Newton step on its residual
+__device__ __forceinline__ D1 reciprocal(D1 a) {
+  const float y = 1.0f / a.h;
+  const D1 r = D1{1.f, 0.f} - a * D1{y, 0.f};
+  return fast_norm(y, y * r.h);
+}
+__device__ __forceinline__ D1 inv_sqrt(D1 a) {
+  const float y = rsqrtf(a.h);
+  const D1 q = D1{y, 0.f} * D1{y, 0.f};
+  const D1 r = D1{1.f, 0.f} - a * q;
+  return fast_norm(y, 0.5f * y * r.h);
+}
+template <int W>
+__device__ __forceinline__ D1 lane_sum(D1 v) {  // over W consecutive lanes
+#pragma unroll
+  for (int o = W / 2; o > 0; o >>= 1)
+    v = v + D1{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
+  return v;
+}
+
 }  // namespace df
 }  // namespace lre

@@ -5,29 +5,35 @@
 // microseconds whatever the size.  Here the whole matrix stays in shared
 // memory:
 //   1. Householder reduction of mu to a real tridiagonal T = Q^dag mu Q (Golub
-//      and Van Loan, Matrix Computations, Sec. 8.3; each reflector scaled so
-//      that the off-diagonal comes out real);
+//      and Van Loan, Matrix Computations, Sec. 8.3), the reflectors
+//      I - g u u^dag with u = x - b e_1 unnormalised, so that the reciprocal in g
+//      is off the critical path (a warp of its own forms it during the product);
 //   2. every eigenvalue of T by multisection on Sturm counts, 128 / d points a
-//      round (tri_minor.cuh), to 4 eps ||T||;
+//      round (tri_minor.cuh): FP32, then double-float, then FP64 to 4 eps ||T||;
 //   3. Smolin's walk, and the spectra where they are asked for;
 //   4. inverse iteration on T for the smaller of the kept and dropped sets,
-//      Gram-Schmidt within clusters, the reflectors applied to those vectors;
+//      Gram-Schmidt within clusters, the reflectors applied to those vectors, all
+//      in double-float;
 //   5. the kept or dropped form of the rebuild (project.cu).
-// All in FP64: one SM does about 1.75 FP64 multiply-adds a cycle and a
-// dependent one waits some 64 cycles, which is what bounds it; hence the few
-// points a round and the vectors of one set only.
-// d = 16: 175 us, against 705 us for the library route (d = 4: 50 against 400).
+// Latency bounds it: an FP64 operation's result takes about 110 cycles, and a
+// reduction step was 85 of them in a row (10,000 cycles whatever d); it is now
+// about 50.  Double-float operations take 40 to 80 cycles and do not queue on the
+// narrow FP64 pipe, so everything after the eigenvalues, whose 2^-47 is far inside
+// the complex64 result, uses them.  The eigenvalues are FP64 throughout.
+// d = 16: 111 us, against 705 us for the library route (and 175 with every step in
+// FP64); d = 4: 33 against 400, d = 32: 280.
 #include <cuda_runtime.h>
 
 #include <cfloat>
 
+#include "dfloat.cuh"
 #include "lre_internal.cuh"
 #include "tri_minor.cuh"
 
 namespace lre {
 namespace {
 
-constexpr int PS_THREADS = 256;
+constexpr int PS_THREADS = 256, PS_ALL = PS_THREADS + 32;  // the last warp: reciprocals of the reduction
 constexpr int PS_ROUNDS = 2;  // inverse iterations (from eigenvalues at rounding level)
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
@@ -46,25 +52,31 @@ __device__ __forceinline__ double lane_sum(double v) {  // over W consecutive la
 }
 
 template <int D>
-__global__ void __launch_bounds__(PS_THREADS) project_small(const float2 *mu, float2 *out, double *eig_mu,
-                                                            double *eig_rho) {
+__global__ void __launch_bounds__(PS_ALL) project_small(const float2 *mu, float2 *out, double *eig_mu,
+                                                        double *eig_rho) {
+  using df::D1;
   constexpr int LD = D + 1;                 // padded row
   constexpr int M = D / 2;                  // most vectors formed
   constexpr int TPR = PS_THREADS / D < 32 ? PS_THREADS / D : 32;  // threads per row of the reduction
-  __shared__ double2 A[D * LD];             // the matrix; reflector k below its diagonal in column k
-  __shared__ double2 v[D], w[D], tau[D];
+  // the matrix; reflector k below its diagonal in column k, from step 4 on in
+  // double-float (the same 16 bytes)
+  __shared__ __align__(16) double2 A[D * LD];
+  __shared__ double2 v[D], w[D], gam[D];
   __shared__ double ta[D], tb[D], nb2[D], W[D];
   __shared__ float fa[D], fb[D];
-  __shared__ double X[M][D];
-  __shared__ double2 lu_z[(5 * D * M + 1) / 2 > M * LD ? (5 * D * M + 1) / 2 : M * LD];
-  auto lu = reinterpret_cast<double(*)[D][M]>(lu_z);  // the factors of T - l_j I ...
-  auto Z = reinterpret_cast<double2(*)[LD]>(lu_z);    // ... then the vectors
-  __shared__ double g[M];
-  __shared__ double s_tn, s_lo, s_hi, s_shift;
-  __shared__ int s_kept;
+  __shared__ D1 da[D], db[D], dn[D];        // scaled T: diagonal, off-diagonal, minus its square
+  __shared__ __align__(16) unsigned char lu_z[(5 * D * M * sizeof(D1)) > M * LD * sizeof(float4)
+                                                  ? 5 * D * M * sizeof(D1)
+                                                  : M * LD * sizeof(float4)];
+  auto lu = reinterpret_cast<D1(*)[D][M]>(lu_z);     // the factors of T - l_j I ...
+  auto Z = reinterpret_cast<float4(*)[LD]>(lu_z);    // ... then the vectors
+  __shared__ D1 X[M][D];
+  __shared__ D1 g[M];
+  __shared__ double s_tn, s_lo, s_hi, s_shift, s_beta;
+  __shared__ int s_kept, s_skip;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-  for (int e = tid; e < D * D; e += PS_THREADS) {
+  for (int e = tid; e < D * D; e += PS_ALL) {
     const int r = e / D, c = e % D;
     float2 x = r <= c ? mu[e] : mu[c * D + r];
     if (r > c) x.y = -x.y;
@@ -73,71 +85,69 @@ __global__ void __launch_bounds__(PS_THREADS) project_small(const float2 *mu, fl
   }
   __syncthreads();
 
-  // ---- 1. reduction
+  // ---- 1. reduction: H = I - g u u^dag, g = 1 / (b (b - conj(x_0))), H^dag x = b e_1
   for (int k = 0; k + 1 < D; ++k) {
     const int m = D - 1 - k;  // length of the reflector: rows k + 1 ..
     if (warp == 0) {
       const int i = k + 1 + lane;
       double2 x = lane < m ? A[i * LD + k] : make_double2(0.0, 0.0);
-      const double below = lane_sum<32>(lane > 0 ? x.x * x.x + x.y * x.y : 0.0);
-      const double2 x0 = make_double2(__shfl_sync(0xffffffffu, x.x, 0), __shfl_sync(0xffffffffu, x.y, 0));
-      double beta = x0.x;
-      double2 t = make_double2(0.0, 0.0);
-      if (below != 0.0 || x0.y != 0.0) {
-        beta = -copysign(sqrt(below + x0.x * x0.x + x0.y * x0.y), x0.x);
-        t = make_double2((beta - x0.x) / beta, -x0.y / beta);
-        const double2 den = make_double2(x0.x - beta, x0.y);  // v = x / (x0 - beta), v_0 = 1
-        const double inv = 1.0 / (den.x * den.x + den.y * den.y);
-        const double2 q = make_double2(den.x * inv, -den.y * inv);
-        x = lane == 0 ? make_double2(1.0, 0.0) : cmul(x, q);
-      } else {
-        x = make_double2(lane == 0 ? 1.0 : 0.0, 0.0);
+      const double sq = x.x * x.x + x.y * x.y;
+      const double below = lane_sum<32>(lane > 0 ? sq : 0.0);
+      if (lane == 0) {
+        const double n2 = below + sq;
+        const bool skip = below == 0.0 && x.y == 0.0;
+        const double beta = skip ? x.x : -copysign(n2 * rsqrt(n2), x.x);
+        s_skip = skip;
+        s_beta = beta;
+        tb[k] = beta;
+        if (skip) gam[k] = make_double2(0.0, 0.0);
+        x.x -= beta;
       }
       if (lane < m) {
         v[i] = x;
         A[i * LD + k] = x;
       }
-      if (lane == 0) {
-        tau[k] = t;
-        tb[k] = beta;
-      }
     }
     __syncthreads();
-    const double2 t = tau[k];
-    if (t.x == 0.0 && t.y == 0.0) continue;  // no reflection (uniform)
-    // w = tau B v over the trailing block B
-    {
+    if (s_skip) {  // no reflection (uniform); s_skip is next written after a barrier
+      __syncthreads();
+      continue;
+    }
+    if (warp == PS_THREADS / 32) {
+      if (lane == 0) {  // u_0 = x_0 - b, b - conj(x_0) = -conj(u_0): g = -u_0 / (b |u_0|^2)
+        const double2 u0 = v[k + 1];
+        const double f = -1.0 / (s_beta * (u0.x * u0.x + u0.y * u0.y));
+        gam[k] = make_double2(f * u0.x, f * u0.y);
+      }
+    } else {  // w = B u over the trailing block B
       const int i = tid / TPR, l = tid % TPR;
       double2 s = make_double2(0.0, 0.0);
       if (i < D && i > k)
         for (int j = k + 1 + l; j < D; j += TPR) cfma(s, A[i * LD + j], v[j]);
       s.x = lane_sum<TPR>(s.x);
       s.y = lane_sum<TPR>(s.y);
-      if (i < D && i > k && l == 0) w[i] = cmul(t, s);
+      if (i < D && i > k && l == 0) w[i] = s;
     }
     __syncthreads();
-    // w -= 1/2 tau (w^dag v) v
+    // q = g w - 1/2 |g|^2 (u^dag w) u (u^dag w is real)
     if (warp == 0) {
       const int i = k + 1 + lane;
+      const double2 t = gam[k];
       const double2 a = lane < m ? w[i] : make_double2(0.0, 0.0), b = lane < m ? v[i] : make_double2(0.0, 0.0);
-      double2 s = cmul(conjd(a), b);
-      s.x = lane_sum<32>(s.x);
-      s.y = lane_sum<32>(s.y);
-      const double2 c = cmul(t, s);
-      if (lane < m) {
-        const double2 q = cmul(make_double2(0.5 * c.x, 0.5 * c.y), b);
-        w[i] = make_double2(a.x - q.x, a.y - q.y);
-      }
+      const double s = lane_sum<32>(b.x * a.x + b.y * a.y);
+      const double c = 0.5 * (t.x * t.x + t.y * t.y) * s;
+      const double2 q = cmul(t, a);
+      if (lane < m) w[i] = make_double2(q.x - c * b.x, q.y - c * b.y);
     }
     __syncthreads();
-    // B -= v w^dag + w v^dag
-    for (int e = tid; e < m * m; e += PS_THREADS) {
+    // B -= u q^dag + q u^dag
+    for (int e = tid; e < m * m; e += PS_ALL) {
       const int i = k + 1 + e / m, j = k + 1 + e % m;
-      double2 s = make_double2(0.0, 0.0);
+      double2 s = make_double2(0.0, 0.0), r = s;
       cfma(s, v[i], conjd(w[j]));
-      cfma(s, w[i], conjd(v[j]));
-      A[i * LD + j].x -= s.x;
-      A[i * LD + j].y -= s.y;
+      cfma(r, w[i], conjd(v[j]));
+      A[i * LD + j].x -= s.x + r.x;
+      A[i * LD + j].y -= s.y + r.y;
     }
     __syncthreads();
   }
@@ -164,6 +174,9 @@ __global__ void __launch_bounds__(PS_THREADS) project_small(const float2 *mu, fl
       W[lane] = ta[lane] * sc;  // the scaled diagonal until the values are known
       fa[lane] = (float)W[lane];
       fb[lane] = (float)nb2[lane];
+      da[lane] = df::d1(W[lane]);
+      db[lane] = df::d1(o);
+      dn[lane] = df::d1(nb2[lane]);
     }
     if (lane == 0) {
       s_tn = tn;
@@ -172,9 +185,9 @@ __global__ void __launch_bounds__(PS_THREADS) project_small(const float2 *mu, fl
     }
   }
   __syncthreads();
+  const double sc = Minor<double>::scale(s_tn), tn = s_tn * sc;
   {
     constexpr int P = 128 / D < 32 ? 128 / D : 32;  // points per value and round
-    const double sc = Minor<double>::scale(s_tn), tn = s_tn * sc;
     const int j = tid / P, l = tid % P;
     double val = 0.0;
     if (tid < ((D * P + 31) & ~31)) {  // whole warps
@@ -183,19 +196,30 @@ __global__ void __launch_bounds__(PS_THREADS) project_small(const float2 *mu, fl
       double lo = s_lo, hi = s_hi;  // count(lo) <= jj < count(hi)
       // points whose count is <= jj, a prefix
       auto below = [&](bool b) { return __popc(__ballot_sync(0xffffffffu, b) & group); };
-      int it32 = 0;
-      for (double wd = 1.0; wd > 1e-6; wd /= P + 1) ++it32;
-      for (int it = 0; it < it32; ++it) {
-        const double h = (hi - lo) / (P + 1);
-        const int k = below(minor_count<float>(fa, fb, D, (float)(lo + h * (l + 1))) <= jj);
+      auto narrow = [&](int k, double h) {
         hi = k == P ? hi : lo + h * (k + 1);
         lo = lo + h * k;
+      };
+      constexpr double inv_p1 = 1.0 / (P + 1);
+      int it32 = 0, it48 = 0;
+      for (double wd = 1.0; wd > 1e-6; wd *= inv_p1) ++it32;
+      for (double wd = 8e-6; wd > 1.2e-13; wd *= inv_p1) ++it48;
+      for (int it = 0; it < it32; ++it) {
+        const double h = (hi - lo) * inv_p1;
+        narrow(below(minor_count<float>(fa, fb, D, (float)(lo + h * (l + 1))) <= jj), h);
       }
       const double w32 = 16.0 * 5.9604644775390625e-08 * tn;  // 16 units of FP32 rounding of T
       lo = fmax(s_lo, lo - w32);
       hi = fmin(s_hi, hi + w32);
+      for (int it = 0; it < it48; ++it) {
+        const double h = (hi - lo) * inv_p1;
+        narrow(below(minor_count_df(da, dn, D, df::d1(lo + h * (l + 1))) <= jj), h);
+      }
+      const double w48 = 16.0 * 7.105427357601002e-15 * tn;  // 16 units of 2^-47
+      lo = fmax(s_lo, lo - w48);
+      hi = fmin(s_hi, hi + w48);
       // the ends in FP64 (two counts, P >= 2 points): back to the whole bracket if
-      // FP32 misplaced it
+      // the rounds before misplaced it
       {
         const bool b = minor_count<double>(W, nb2, D, l == 0 ? lo : hi) <= jj;
         const unsigned vt = __ballot_sync(0xffffffffu, b) & group;
@@ -208,23 +232,25 @@ __global__ void __launch_bounds__(PS_THREADS) project_small(const float2 *mu, fl
       const double tol = 4.0 * DBL_EPSILON * tn;
       for (int it = 0; it < 64; ++it) {
         if (__all_sync(0xffffffffu, !(hi - lo > tol))) break;
-        const double h = (hi - lo) / (P + 1);
-        const int k = below(minor_count<double>(W, nb2, D, lo + h * (l + 1)) <= jj);
-        const double nhi = k == P ? hi : lo + h * (k + 1), nlo = lo + h * k;
-        hi = nhi;
-        lo = nlo;
+        const double h = (hi - lo) * inv_p1;
+        narrow(below(minor_count<double>(W, nb2, D, lo + h * (l + 1)) <= jj), h);
       }
       val = 0.5 * (lo + hi) / sc;
     }
     __syncthreads();
     if (j < D && l == 0) W[j] = val;
   }
+  // the reflectors in double-float, in place
+  for (int e = tid; e < D * D; e += PS_ALL) {
+    const int i = e / D, k = e % D;
+    if (i > k) reinterpret_cast<float4 *>(A)[i * LD + k] = df::split(A[i * LD + k]);
+  }
   __syncthreads();
   // ---- 3. Smolin's walk: drop the smallest l_j while l_j + a / kept < 0
   if (tid == 0) {
     int dropped = 0, kept = D;
     double a = 0.0;
-    while (kept > 0 && W[dropped] + a / (double)kept < 0.0) {
+    while (kept > 0 && fma(W[dropped], (double)kept, a) < 0.0) {
       a += W[dropped];
       ++dropped;
       --kept;
@@ -242,72 +268,73 @@ __global__ void __launch_bounds__(PS_THREADS) project_small(const float2 *mu, fl
   }
   const bool kept_form = kept <= D - kept;
   const int m = kept_form ? kept : D - kept, off = kept_form ? D - kept : 0;
-  // ---- 4. vectors: inverse iteration, one lane per vector
+  // ---- 4. vectors: inverse iteration on the scaled T, one lane per vector
   if (warp == 0) {
-    const double tn = s_tn, small = DBL_EPSILON * tn > DBL_MIN ? DBL_EPSILON * tn : DBL_MIN;
+    const float small = (float)(DBL_EPSILON * tn);
     if (lane < m) {
-      const double x = W[off + lane];
-      double p = ta[0] - x, q = D > 1 ? tb[0] : 0.0;
+      const D1 x = df::d1(W[off + lane] * sc);
+      D1 p = da[0] - x, q = db[0];
       for (int k = 0; k + 1 < D; ++k) {
-        const double lo = tb[k], dk = ta[k + 1] - x, up = k + 2 < D ? tb[k + 1] : 0.0;
-        const bool swap = fabs(lo) > fabs(p);
-        double piv = swap ? lo : p;
-        if (!swap && fabs(piv) < small) piv = small;
-        const double r = 1.0 / piv, f = (swap ? p : lo) * r;
+        const D1 lo = db[k], dk = da[k + 1] - x, up = k + 2 < D ? db[k + 1] : D1{0.f, 0.f};
+        const bool swap = fabsf(lo.h) > fabsf(p.h);
+        D1 piv = swap ? lo : p;
+        if (!swap && fabsf(piv.h) < small) piv = {small, 0.f};
+        const D1 r = df::reciprocal(piv), f = (swap ? p : lo) * r;
         lu[0][k][lane] = r;
         lu[1][k][lane] = swap ? dk : q;
-        lu[2][k][lane] = swap ? up : 0.0;
+        lu[2][k][lane] = swap ? up : D1{0.f, 0.f};
         lu[3][k][lane] = f;
-        lu[4][k][lane] = swap ? 1.0 : 0.0;
+        lu[4][k][lane] = {swap ? 1.f : 0.f, 0.f};
         p = swap ? q - f * dk : dk - f * q;
-        q = swap ? -f * up : up;
+        q = swap ? -(f * up) : up;
       }
-      if (fabs(p) < small) p = small;
-      lu[0][D - 1][lane] = 1.0 / p;
-      lu[1][D - 1][lane] = lu[2][D - 1][lane] = 0.0;
+      if (fabsf(p.h) < small) p = {small, 0.f};
+      lu[0][D - 1][lane] = df::reciprocal(p);
+      lu[1][D - 1][lane] = lu[2][D - 1][lane] = {0.f, 0.f};
       for (int k = 0; k < D; ++k) {  // a fixed, spread-out start
         const unsigned h = (unsigned)(k * 32 + lane + 1) * 2654435761u;
-        X[lane][k] = 0.5 + (double)(h >> 8) * (1.0 / 16777216.0);
+        X[lane][k] = {0.5f + (float)(h >> 8) * (1.0f / 16777216.0f), 0.f};
       }
     }
     for (int it = 0; it < PS_ROUNDS; ++it) {
       if (lane < m) {
-        double pend = X[lane][0];
+        D1 pend = X[lane][0];
         for (int k = 0; k + 1 < D; ++k) {
-          const double nxt = X[lane][k + 1], f = lu[3][k][lane];
-          const bool swap = lu[4][k][lane] != 0.0;
+          const D1 nxt = X[lane][k + 1], f = lu[3][k][lane];
+          const bool swap = lu[4][k][lane].h != 0.f;
           X[lane][k] = swap ? nxt : pend;
           pend = swap ? pend - f * nxt : nxt - f * pend;
         }
         X[lane][D - 1] = pend;
-        double x1 = 0.0, x2 = 0.0;
+        D1 x1{0.f, 0.f}, x2 = x1;
         for (int k = D - 1; k >= 0; --k) {
-          const double xk = (X[lane][k] - lu[1][k][lane] * x1 - lu[2][k][lane] * x2) * lu[0][k][lane];
+          const D1 xk = (X[lane][k] - lu[1][k][lane] * x1 - lu[2][k][lane] * x2) * lu[0][k][lane];
           X[lane][k] = xk;
           x2 = x1;
           x1 = xk;
         }
       }
       __syncwarp();
-      // unit norm (scaled first: a solve grows by up to 1 / eps), Gram-Schmidt
-      // against the cluster's earlier vectors, unit norm again
+      // unit norm (scaled by a power of two first: a solve grows by up to 1 / eps),
+      // Gram-Schmidt against the cluster's earlier vectors, unit norm again
       int c0 = 0;
       for (int j = 0; j < m; ++j) {
-        if (j > 0 && W[off + j] - W[off + j - 1] > 1e-3 * tn) c0 = j;
-        double x = lane < D ? X[j][lane] : 0.0;
-        double mx = fabs(x);
+        if (j > 0 && (W[off + j] - W[off + j - 1]) * sc > 1e-3 * tn) c0 = j;
+        D1 x = lane < D ? X[j][lane] : D1{0.f, 0.f};
+        float mx = fabsf(x.h);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        x *= mx > 0.0 ? 1.0 / mx : 0.0;
-        double n2 = lane_sum<32>(x * x);
-        x *= n2 > 0.0 ? rsqrt(n2) : 0.0;
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        const float f = Minor<float>::scale(mx);
+        x = {x.h * f, x.l * f};
+        D1 n2 = df::lane_sum<32>(x * x);
+        if (n2.h > 0.f) x = x * df::inv_sqrt(n2);
         if (c0 < j) {
           for (int i = c0; i < j; ++i) {
-            const double y = lane < D ? X[i][lane] : 0.0;
-            x -= lane_sum<32>(x * y) * y;
+            const D1 y = lane < D ? X[i][lane] : D1{0.f, 0.f};
+            x = x - df::lane_sum<32>(x * y) * y;
           }
-          n2 = lane_sum<32>(x * x);
-          x *= n2 > 0.0 ? rsqrt(n2) : 0.0;
+          n2 = df::lane_sum<32>(x * x);
+          if (n2.h > 0.f) x = x * df::inv_sqrt(n2);
         }
         if (lane < D) X[j][lane] = x;
         __syncwarp();
@@ -316,46 +343,61 @@ __global__ void __launch_bounds__(PS_THREADS) project_small(const float2 *mu, fl
   }
   __syncthreads();
   // z = H_0 H_1 .. x: the last reflector first, D lanes per vector
-  {
+  if (warp < PS_THREADS / 32) {
     constexpr int VPW = 32 / D;  // vectors per warp
     const int sub = lane / D, i = lane % D;
+    const float4 *U = reinterpret_cast<const float4 *>(A);
     for (int j0 = warp * VPW; j0 < ((m + VPW - 1) / VPW) * VPW; j0 += PS_THREADS / 32 * VPW) {
       const int j = j0 + sub;
-      double2 z = make_double2(j < m ? X[j][i] : 0.0, 0.0);
+      const D1 x = j < m ? X[j][i] : D1{0.f, 0.f};
+      float4 z = make_float4(x.h, 0.f, x.l, 0.f);
       for (int k = D - 2; k >= 0; --k) {
-        const double2 t = tau[k];
+        const double2 t = gam[k];
         if (t.x == 0.0 && t.y == 0.0) continue;
-        const double2 vi = i > k ? A[i * LD + k] : make_double2(0.0, 0.0);
-        double2 s = cmul(conjd(vi), z);
-        s.x = lane_sum<D>(s.x);
-        s.y = lane_sum<D>(s.y);
-        const double2 c = cmul(t, s);
-        z.x -= c.x * vi.x - c.y * vi.y;
-        z.y -= c.x * vi.y + c.y * vi.x;
+        const float4 u = i > k ? U[i * LD + k] : make_float4(0.f, 0.f, 0.f, 0.f);
+        df::Sum S;
+        df::mac_df(S, u, df::hi(z), df::lo(z));
+        float4 s = df::df_conj_ab(S);
+#pragma unroll
+        for (int o = D / 2; o > 0; o >>= 1) s = df::add(s, df::shfl_xor(s, o));
+        df::Sum C, R;
+        df::mac_df(C, df::split(t), df::hi(s), df::lo(s));
+        const float4 c = df::df_ab(C);
+        df::mac_df(R, c, df::hi(u), df::lo(u));
+        const float4 r = df::df_ab(R);
+        z = df::add(z, make_float4(-r.x, -r.y, -r.z, -r.w));
       }
       if (j < m) Z[j][i] = z;
     }
     if (tid < m) {
       const double x = (kept_form ? 1.0 : -1.0) * (W[off + tid] + shift);
-      g[tid] = x > 0.0 ? x : 0.0;
+      g[tid] = df::d1(x > 0.0 ? x : 0.0);
     }
   }
   __syncthreads();
   // ---- 5. rebuild: the upper triangle and its mirror
-  for (int e = tid; e < D * D; e += PS_THREADS) {
+  for (int e = tid; e < D * D; e += PS_ALL) {
     const int r = e / D, c = e % D;
     if (r > c) continue;
-    double2 s = make_double2(0.0, 0.0);
+    df::Sum S;
+    for (int j = 0; j < m; ++j) {
+      const float4 a = Z[j][r], b = Z[j][c];
+      df::f2 h = 0, l = 0;
+      df::mac2(h, l, df::pk(g[j].h, g[j].h), df::pk(g[j].l, g[j].l), df::hi(a), df::lo(a));
+      df::mac_df(S, df::norm4(h, l), df::hi(b), df::lo(b));
+    }
+    float4 s = df::df_conj_ab(S);  // a conj(b) is its conjugate
+    s.y = -s.y;
+    s.w = -s.w;
     if (!kept_form) {
       const float2 x = mu[e];  // out may be mu: only this thread reads or writes this place and its mirror
-      s = make_double2((double)x.x, r == c ? 0.0 : (double)x.y);
-      if (r == c) s.x += shift;
+      s = df::add(s, make_float4(x.x, r == c ? 0.f : x.y, 0.f, 0.f));
+      if (r == c) {
+        const float2 q = df::split1(shift);
+        s = df::add(s, make_float4(q.x, 0.f, q.y, 0.f));
+      }
     }
-    for (int j = 0; j < m; ++j) {
-      const double2 a = Z[j][r];
-      cfma(s, make_double2(g[j] * a.x, g[j] * a.y), conjd(Z[j][c]));
-    }
-    const float2 o = make_float2((float)s.x, r == c ? 0.f : (float)s.y);
+    const float2 o = make_float2(s.x, r == c ? 0.f : s.y);
     out[e] = o;
     if (r < c) out[c * D + r] = make_float2(o.x, -o.y);
   }
@@ -370,11 +412,11 @@ lre_status project_small_run(lre_ctx *ctx, const lre_c64 *rho_in, int n, lre_c64
   {
     Launch L(ctx, "project_small", s);
     switch (n) {
-      case 1: project_small<2><<<1, PS_THREADS, 0, s>>>(in, out, eig_mu, eig_rho); break;
-      case 2: project_small<4><<<1, PS_THREADS, 0, s>>>(in, out, eig_mu, eig_rho); break;
-      case 3: project_small<8><<<1, PS_THREADS, 0, s>>>(in, out, eig_mu, eig_rho); break;
-      case 4: project_small<16><<<1, PS_THREADS, 0, s>>>(in, out, eig_mu, eig_rho); break;
-      case 5: project_small<32><<<1, PS_THREADS, 0, s>>>(in, out, eig_mu, eig_rho); break;
+      case 1: project_small<2><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho); break;
+      case 2: project_small<4><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho); break;
+      case 3: project_small<8><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho); break;
+      case 4: project_small<16><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho); break;
+      case 5: project_small<32><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho); break;
       default: return LRE_ERR_UNSUPPORTED;
     }
   }

@@ -3,6 +3,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "dfloat.cuh"
+
 namespace lre {
 
 // Sturm count by the three-term recurrence of the leading principal minors
@@ -53,6 +55,29 @@ __device__ __forceinline__ int minor_count(const R *a, const R *nb2, int n, R x)
     const R f = Minor<R>::scale(ap > am ? ap : am);
     p *= f;
     pm *= f;
+  }
+  return cnt;
+}
+
+// The same in double-float (FP32 pipes), |a|, |nb2|, |x| of order one.
+__device__ __forceinline__ int minor_count_df(const df::D1 *a, const df::D1 *nb2, int n, df::D1 x) {
+  df::D1 pm{1.f, 0.f}, p = a[0] - x;
+  unsigned sg = p.h == 0.f ? 1u : Minor<float>::sign(p.h);
+  int cnt = (int)sg;
+  int k = 1;
+  while (k < n) {
+    const int e = k + 4 < n ? k + 4 : n;
+    for (; k < e; ++k) {
+      const df::D1 t = nb2[k - 1] * pm;
+      pm = p;
+      p = (a[k] - x) * p + t;
+      const unsigned ns = p.h == 0.f ? sg ^ 1u : Minor<float>::sign(p.h);
+      cnt += (int)(ns ^ sg);
+      sg = ns;
+    }
+    const float ap = fabsf(p.h), am = fabsf(pm.h), f = Minor<float>::scale(ap > am ? ap : am);
+    p = {p.h * f, p.l * f};
+    pm = {pm.h * f, pm.l * f};
   }
   return cnt;
 }
