@@ -267,6 +267,7 @@ struct KryBuffers {
   double *alpha, *beta, *b2, *stats, *Wr, *Xr, *lu, *last, *nrm;
   int *cl, *nclust, *breakdown;
   int64_t rows, ct_max;
+  bool persistent;  // steps in one launch (krylov_steps.cu)
 };
 
 // The J x J Lanczos matrix's CB smallest and CT largest eigenvalues
@@ -280,7 +281,7 @@ struct RitzEnds {
 // Convergence check.  The residual of a Ritz pair is beta_J |s_J|, s_J the last
 // component of its eigenvector, which one inverse-iteration solve from the
 // eigenvalue (computed to 4 eps ||T||) gives to far below the tolerance; the
-// vectors that are used get all rounds (ritz_vectors) and are looked at again.
+// vectors that are used get two rounds (ritz_vectors) and are looked at again.
 // Values placed less exactly will not do: an unconverged neighbour's last
 // component comes through with the value's error over their gap.
 lre_status ritz_values(lre_ctx *ctx, const KryBuffers &B, const double *alpha, const double *beta, int J, int CB,
@@ -336,9 +337,12 @@ lre_status ritz_vectors(lre_ctx *ctx, const KryBuffers &B, const double *alpha, 
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "Ritz clusters");
   {
-    Launch L(ctx, "kry_inverse_iteration", s, 2 + 2 * TRI_ROUNDS);
+    // two rounds: the eigenvalues are at rounding level, and the last components
+    // are looked at below
+    constexpr int rounds = 2;
+    Launch L(ctx, "kry_inverse_iteration", s, 2 + 2 * rounds);
     tri_factor<<<(m + 31) / 32, 32, 0, s>>>(alpha, beta, J, w, m, tnorm, B.lu);
-    for (int it = 0; it < TRI_ROUNDS; ++it) {
+    for (int it = 0; it < rounds; ++it) {
       tri_solve<<<(m + 31) / 32, 32, 0, s>>>(B.lu, J, m, B.Xr, it == 0);
       tri_orthonormalise<<<hk, TRI_THREADS, 0, s>>>(B.Xr, J, B.cl);
     }
@@ -355,7 +359,7 @@ lre_status ritz_vectors(lre_ctx *ctx, const KryBuffers &B, const double *alpha, 
 // Gram-Schmidt, twice) and writes alpha[j], beta[j] and row base + j + 1.
 lre_status lanczos_steps(lre_ctx *ctx, const KryBuffers &B, int64_t d, int64_t base, int j0, int j1, double *alpha,
                          double *beta, double tiny, cudaStream_t s) {
-  if (d <= KRY_STEPS_MAX_D) {
+  if (B.persistent) {
     const KryStepBuffers K{B.A, B.Q, B.Ws, B.Wn, B.Hs, B.sync, B.breakdown, B.rows};
     return kry_steps_run(ctx, K, d, base, j0, j1, alpha, beta, tiny, s);
   }
@@ -477,6 +481,11 @@ lre_status project_krylov(lre_ctx *ctx, const lre_c64 *rho_in, int64_t d, lre_c6
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "Krylov set-up");
   const double tiny = 1e-14 * sqrt(fro_tr[0]);
+  // the persistent steps hold squared norms in FP32 pairs, down to tiny^2: a density
+  // matrix has a norm in [1/64, 1] there; anything far from that takes the FP64 work
+  // vector of the multi-launch form, or the reduction where d is too small for it
+  B.persistent = copy && fro_tr[0] >= 0x1p-20 && fro_tr[0] <= 0x1p60;
+  if (copy && !B.persistent && d < 2048) return LRE_OK;
   const double trace = fro_tr[1];  // Tr mu (1 up to the complex64 rounding of the diagonal)
   if ((st = start_vector(ctx, B, d, 0, 0x5EED0001ull, s)) != LRE_OK) return st;
 

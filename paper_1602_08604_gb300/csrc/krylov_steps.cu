@@ -27,9 +27,9 @@
 // FP64; every CTA adds the shares in the same order, so all have the same
 // scalars and a run repeats bit for bit.
 // What bounds it: at d = 4096 the product's FP32 instructions (22 packed ones of
-// two cycles per entry of mu: 21 us of its 34 us a step; the rest is waiting for
-// the 134 MB that do not stay in L2), below that the barriers and dependent
-// trips to L2 (22 us a step at d = 1024).
+// two cycles per entry of mu: 21 us of a step's 46; with mu's next batch loaded
+// during the products of the one before, 46 against 67 us a step), below that the
+// barriers and dependent trips to L2 (16 us a step at d = 1024).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -56,7 +56,7 @@ struct StepArgs {
   float2 *shares;       // [2][G] the CTAs' shares of alpha and of the norm
   unsigned *bar;        // arrivals, then the abort flag; zeroed before the launch
   int *breakdown, *status;
-  double tiny;
+  float tiny;
   int d, base, j0, j1, rows;
 };
 
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(THREADS, 1) kry_steps(StepArgs P) {
   // marked evict-first, so that the basis stays (n = 12: dots and update 49k
   // against 37k cycles a step)
   const uint64_t policy = (int64_t)d * d * 8 > (64ll << 20) ? sm103::l2_evict_first() : sm103::l2_evict_normal();
-  double alpha_1 = 0.0, yscale = 1.0;  // warp 0: alpha before the corrections; y = yscale (mu xs)
+  df::D1 alpha_1{0.f, 0.f}, yscale{1.f, 0.f};  // warp 0: alpha before the corrections; y = yscale (mu xs)
 
   // x = the basis row of the first step
   {
@@ -207,29 +207,51 @@ __global__ void __launch_bounds__(THREADS, 1) kry_steps(StepArgs P) {
     // ---- product
     for (int rb = 0; rb < nr; rb += rroom) {
       const int nrow = nr - rb < rroom ? nr - rb : rroom;
-      for (int u = warp; u < nrow * nseg; u += WARPS) {
-        const int r = u / nseg, sg = u - r * nseg;
-        const float2 *a = P.A + (int64_t)(r0 + rb + r) * d + sg * seg + lane;
-        const float4 *x = xs + sg * seg + lane;
+      const int units = nrow * nseg;
+      if (seg >= 512) {
+        // batches of sixteen entries per lane; the next batch (of this unit or of the
+        // warp's next one) is in flight during the products of the current one, 64 KB an SM
+        const int per = seg >> 9, nb = units > warp ? ((units - warp + WARPS - 1) / WARPS) * per : 0;
+        auto load = [&](int bt, float2 (&v)[16]) {
+          const int u = warp + bt / per * WARPS, r = u / nseg;
+          const float2 *a = P.A + (int64_t)(r0 + rb + r) * d + (u - r * nseg) * seg + (bt % per) * 512 + lane;
+#pragma unroll
+          for (int q = 0; q < 16; ++q) v[q] = ld_mu(a + 32 * q, policy);
+        };
+        float2 next[16];
+        if (nb > 0) load(0, next);
         df::Sum S;
-        int k = 0;
-        for (; k + 512 <= seg; k += 512) {  // sixteen loads in flight per lane: 64 KB an SM
+        for (int bt = 0; bt < nb; ++bt) {
           float2 v[16];
 #pragma unroll
-          for (int q = 0; q < 16; ++q) v[q] = ld_mu(a + k + 32 * q, policy);
+          for (int q = 0; q < 16; ++q) v[q] = next[q];
+          if (bt + 1 < nb) load(bt + 1, next);
+          const int u = warp + bt / per * WARPS, r = u / nseg;
+          const float4 *x = xs + (u - r * nseg) * seg + (bt % per) * 512 + lane;
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
-            const float4 w = x[k + 32 * q];
+            const float4 w = x[32 * q];
             df::mac_c64(S, v[q], df::hi(w), df::lo(w));
           }
+          if (bt % per == per - 1) {
+            part[u * 32 + lane] = df::df_ab(S);
+            S = df::Sum();
+          }
         }
-        for (; k + 64 <= seg; k += 64) {
-          const float2 v0 = ld_mu(a + k, policy), v1 = ld_mu(a + k + 32, policy);
-          const float4 w0 = x[k], w1 = x[k + 32];
-          df::mac_c64(S, v0, df::hi(w0), df::lo(w0));
-          df::mac_c64(S, v1, df::hi(w1), df::lo(w1));
+      } else {
+        for (int u = warp; u < units; u += WARPS) {
+          const int r = u / nseg, sg = u - r * nseg;
+          const float2 *a = P.A + (int64_t)(r0 + rb + r) * d + sg * seg + lane;
+          const float4 *x = xs + sg * seg + lane;
+          df::Sum S;
+          for (int k = 0; k < seg; k += 64) {
+            const float2 v0 = ld_mu(a + k, policy), v1 = ld_mu(a + k + 32, policy);
+            const float4 w0 = x[k], w1 = x[k + 32];
+            df::mac_c64(S, v0, df::hi(w0), df::lo(w0));
+            df::mac_c64(S, v1, df::hi(w1), df::lo(w1));
+          }
+          part[u * 32 + lane] = df::df_ab(S);
         }
-        part[u * 32 + lane] = df::df_ab(S);
       }
       __syncthreads();
       for (int r = warp; r < nrow; r += WARPS) {
@@ -251,33 +273,35 @@ __global__ void __launch_bounds__(THREADS, 1) kry_steps(StepArgs P) {
       real_mac(sh, sl, q.y, q.w, y.y, y.w);
     }
     block_real_sum(sh, sl, red, wide);
-    // q_prev of the entries this thread forms below, in flight over the barrier
     const bool prev = j > 0;
-    constexpr int PER = (int)(KRY_STEPS_MAX_D / THREADS);
-    float4 qp[PER];
-#pragma unroll
-    for (int m = 0; m < PER; ++m)
-      if (prev && tid + m * THREADS < d) qp[m] = ldcg4(P.Q + (int64_t)(c - 1) * d + tid + m * THREADS);
+    constexpr int PER = (int)(KRY_STEPS_MAX_D / THREADS), HALF = PER / 2;
     if (tid == 0) P.shares[g] = make_float2(sh, sl);
     if (!grid_barrier(P, target, &s_ok)) return;
     // ---- w' = y - alpha q - beta q_prev, whole; q = xs yscale
-    float4 yv[PER];
-#pragma unroll
-    for (int m = 0; m < PER; ++m)
-      if (tid + m * THREADS < d) yv[m] = ldcg4(P.Y + tid + m * THREADS);
     if (warp == 0) {
       if (G > 1) sum_shares(P.shares, sh, sl);
       if (lane == 0) {
-        alpha_1 = (double)sh + (double)sl;
-        s_alpha_x = df::split1(alpha_1 * yscale);
+        alpha_1 = df::fast_norm(sh, sl);
+        const df::D1 ax = alpha_1 * yscale;
+        s_alpha_x = make_float2(ax.h, ax.l);
       }
     }
-    __syncthreads();
-    {
+#pragma unroll
+    for (int m0 = 0; m0 < PER; m0 += HALF) {
+      float4 yv[HALF], qp[HALF];
+#pragma unroll
+      for (int m = 0; m < HALF; ++m) {
+        const int i = tid + (m0 + m) * THREADS;
+        if (i < d) {
+          yv[m] = ldcg4(P.Y + i);
+          if (prev) qp[m] = ldcg4(P.Q + (int64_t)(c - 1) * d + i);
+        }
+      }
+      if (m0 == 0) __syncthreads();  // alpha
       const float2 ca = s_alpha_x, cb = s_beta;
 #pragma unroll
-      for (int m = 0; m < PER; ++m) {
-        const int i = tid + m * THREADS;
+      for (int m = 0; m < HALF; ++m) {
+        const int i = tid + (m0 + m) * THREADS;
         if (i < d) {
           float4 v = sub_scaled(yv[m], ca, xs[i]);
           if (prev) v = sub_scaled(v, cb, qp[m]);
@@ -388,43 +412,38 @@ __global__ void __launch_bounds__(THREADS, 1) kry_steps(StepArgs P) {
     if (tid == 0) P.shares[G + g] = make_float2(sh, sl);
     if (!grid_barrier(P, target, &s_ok)) return;
     // ---- close the step
-    float4 wv[PER];
-    if (j + 1 < P.j1) {
-#pragma unroll
-      for (int m = 0; m < PER; ++m)
-        if (tid + m * THREADS < d) wv[m] = ldcg4(P.W + tid + m * THREADS);
-    }
     if (warp == 0) {
       if (G > 1) sum_shares(P.shares + G, sh, sl);  // every lane has the sum
       else {
         sh = __shfl_sync(0xffffffffu, sh, 0);
         sl = __shfl_sync(0xffffffffu, sl, 0);
       }
-      const double b2 = (double)sh + (double)sl;
-      const double inv0 = b2 > 0.0 ? rsqrt(b2) : 0.0, b = b2 * inv0;
-      const bool dead = !(b > P.tiny);  // an invariant subspace: q_next = 0, as the host expects
-      const double inv = dead ? 0.0 : inv0;
+      // what the next phase waits for in double-float (an FP64 square root and its
+      // splits are twenty dependent operations of 110 cycles)
+      const df::D1 b2 = df::fast_norm(sh, sl);
+      const df::D1 inv0 = b2.h > 0.f ? df::inv_sqrt(b2) : df::D1{0.f, 0.f}, b = b2 * inv0;
+      const bool dead = !(b.h > P.tiny);  // an invariant subspace: q_next = 0, as the host expects
+      const df::D1 inv = dead ? df::D1{0.f, 0.f} : inv0;
       // xs = w'' 2^-e with beta 2^-e in [1, 2): exact, and y's factor is 2^e / beta
-      int ex = 0;
-      if (!dead) ex = (int)((__double_as_longlong(b) >> 52) & 0x7FF) - 1023;
+      int ex = dead ? 0 : (int)((__float_as_uint(b.h) >> 23) & 0xFF) - 127;
       ex = ex > 120 ? 120 : ex < -120 ? -120 : ex;
-      yscale = inv * __longlong_as_double((long long)(1023 + ex) << 52);
-      const float2 v = df::split1(lane == 0 ? yscale : lane == 1 ? inv : dead ? 0.0 : b);
+      const float up = __int_as_float((127 + ex) << 23);
+      yscale = {inv.h * up, inv.l * up};
       if (lane == 0) {
-        s_ysc = v;
+        s_ysc = make_float2(yscale.h, yscale.l);
         s_pow = dead ? 0.f : __int_as_float((127 - ex) << 23);
-      } else if (lane == 1) {
-        s_inv = v;
-      } else if (lane == 2) {
-        s_beta = v;
-      }
-      if (g == 0 && lane == 0) {
-        P.alpha[j] = alpha_1 + ((double)hs[c].x + (double)hs[c].z);
-        P.beta[j] = dead ? 0.0 : b;
-        if (dead && *P.breakdown == 0) *P.breakdown = j + 1;
+        s_inv = make_float2(inv.h, inv.l);
+        s_beta = dead ? make_float2(0.f, 0.f) : make_float2(b.h, b.l);
       }
     }
     __syncthreads();
+    if (g == 0 && tid == 0) {  // the Lanczos matrix, in FP64
+      const double b2 = (double)sh + (double)sl, b = b2 > 0.0 ? sqrt(b2) : 0.0;
+      const bool dead = s_pow == 0.f;
+      P.alpha[j] = df::value(alpha_1) + ((double)hs[c].x + (double)hs[c].z);
+      P.beta[j] = dead ? 0.0 : b;
+      if (dead && *P.breakdown == 0) *P.breakdown = j + 1;
+    }
     const float2 inv = s_inv;
     const bool store = c + 1 < P.rows;
     for (int e = tid; e < nr; e += THREADS) {
@@ -435,9 +454,16 @@ __global__ void __launch_bounds__(THREADS, 1) kry_steps(StepArgs P) {
     if (j + 1 < P.j1) {
       const float pw = s_pow;
 #pragma unroll
-      for (int m = 0; m < PER; ++m) {
-        const int i = tid + m * THREADS;
-        if (i < d) xs[i] = make_float4(wv[m].x * pw, wv[m].y * pw, wv[m].z * pw, wv[m].w * pw);
+      for (int m0 = 0; m0 < PER; m0 += HALF) {
+        float4 wv[HALF];
+#pragma unroll
+        for (int m = 0; m < HALF; ++m)
+          if (tid + (m0 + m) * THREADS < d) wv[m] = ldcg4(P.W + tid + (m0 + m) * THREADS);
+#pragma unroll
+        for (int m = 0; m < HALF; ++m) {
+          const int i = tid + (m0 + m) * THREADS;
+          if (i < d) xs[i] = make_float4(wv[m].x * pw, wv[m].y * pw, wv[m].z * pw, wv[m].w * pw);
+        }
       }
     }
     __syncthreads();
@@ -456,8 +482,8 @@ size_t steps_smem(int64_t d, int64_t rows, int G) {
 // below that (d = 256: 3.6 ms a run on 32 CTAs, 4.0 on 16, 15.8 on one;
 // d = 1024: 7.7 on 128, 9.0 on 64; d = 64: 0.8 on 8, 0.9 on one).
 // Whole projections, before (the reduction path below d = 2048, one launch per
-// operation above) and now: d = 64 4.9 -> 1.3 ms, 256 16 -> 5.2, 512 34 -> 8.2,
-// 1024 82.7 -> 13.1 (51 vectors kept), 4096 176 -> 77 (100 kept).
+// operation above) and now: d = 64 4.9 -> 1.1 ms, 256 16 -> 4.7, 512 34 -> 7.5,
+// 1024 82.7 -> 12.7 (51 vectors kept), 4096 176 -> 58 (100 kept).
 int kry_steps_grid(lre_ctx *ctx, int64_t d) {
   const int64_t g = d / 8;
   return (int)std::min<int64_t>(g, ctx->num_sms);
@@ -480,7 +506,7 @@ lre_status kry_steps_run(lre_ctx *ctx, const KryStepBuffers &B, int64_t d, int64
   P.shares = reinterpret_cast<float2 *>(P.bar + 4);
   P.breakdown = B.breakdown;
   P.status = ctx->d_status;
-  P.tiny = tiny;
+  P.tiny = (float)tiny;
   P.d = (int)d;
   P.base = (int)base;
   P.j0 = j0;

@@ -119,3 +119,24 @@ def test_only_the_upper_triangle_is_read(env, n):
         outs.append(out.cpu().numpy())
     np.testing.assert_array_equal(outs[0], outs[1])
 
+
+
+@pytest.mark.parametrize("n,scale", [(7, 1e-9), (8, 1e12), (11, 1e-9), (11, 1e12)])
+def test_scaled_inputs(env, n, scale):
+    """Norms far from a density matrix' leave the persistent steps, whose squared
+    norms are FP32 pairs; the projection scales with its input (trace kept)."""
+    torch, lre, ctx = env
+    d = 2 ** n
+    rng = np.random.default_rng(n)
+    lam = -rng.uniform(0, 2e-4, d)
+    lam[-4:] = (0.1, 0.2, 0.3, 0.4)
+    m = _hermitian_with_spectrum(lam / lam.sum(), 5 + n)
+    scaled = (m * np.float32(scale)).astype(np.complex64)
+    outs = []
+    for x in (m, scaled):
+        mu = torch.from_numpy(x).cuda()
+        out = torch.full_like(mu, float("nan"))
+        lre.lre_project(ctx, mu, n, out)
+        lre.lre_sync(ctx)
+        outs.append(out.cpu().numpy().astype(np.complex128))
+    assert rel_fro(outs[1] / float(np.float32(scale)), outs[0]) <= 1e-6
