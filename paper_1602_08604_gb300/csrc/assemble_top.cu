@@ -29,6 +29,7 @@
 
 #include "lre_internal.cuh"
 #include "passes.cuh"
+#include "sm103.cuh"
 
 namespace lre {
 namespace {
@@ -44,7 +45,9 @@ __global__ void __launch_bounds__(256) fold_final_top(GenParams P) {
   constexpr int NP = 1 << (2 * J), B = 1 << J;
   __shared__ DivTables tab;
   load_div_tables(P, tab);
+  sm103::pdl_wait();
   __syncthreads();
+  sm103::pdl_trigger();
   double *theta = static_cast<double *>(P.out);
   long long *diag = reinterpret_cast<long long *>(P.T);
   V *off = reinterpret_cast<V *>(diag + B * P.C);
@@ -141,6 +144,8 @@ __global__ void __launch_bounds__(256) top_low6(TopArgs P) {
   V *S = reinterpret_cast<V *>(smem_raw);
   const int B = 1 << P.J, m = P.n - P.J, tid = threadIdx.x;
   const int64_t C = 1ll << (2 * m), per = C >> 12;
+  sm103::pdl_wait();
+  sm103::pdl_trigger();
   for (int64_t u = blockIdx.x; u < P.units; u += gridDim.x) {
     const int b = (int)(u / per);
     const int64_t Pp = u - b * per;
@@ -184,6 +189,8 @@ __global__ void __launch_bounds__(256) top_high(TopArgs P) {
   const int64_t side = 1ll << t, L4 = side * side, tiles = side / TD;
   const int64_t per_b = (1ll << (2 * (m - t - Q))) * tiles * tiles;
   const int64_t C = 1ll << (2 * m), W = side << Q;
+  sm103::pdl_wait();
+  sm103::pdl_trigger();
   for (int64_t u = blockIdx.x; u < P.units; u += gridDim.x) {
     const int b = (int)(u / per_b);
     const int64_t x = u - b * per_b, Pp = x / (tiles * tiles), y = x - Pp * tiles * tiles;
@@ -274,7 +281,7 @@ template <int Q>
 void launch_high(bool last, const TopArgs &a, int grid, cudaStream_t s) {
   auto k = last ? top_high<Q, true> : top_high<Q, false>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, ASM_TILE_SMEM);
-  k<<<grid, 256, ASM_TILE_SMEM, s>>>(a);
+  launch_pdl(overlaps(a.n), k, grid, 256, ASM_TILE_SMEM, s, a);
 }
 
 }  // namespace
@@ -293,7 +300,7 @@ lre_status fold_final_top_run(lre_ctx *ctx, const passes::GenParams &P, int J, i
   if (!k) return LRE_ERR_UNSUPPORTED;
   {
     Launch L(ctx, "fold_final", s);
-    k<<<(unsigned)blocks, threads, 0, s>>>(P);
+    launch_pdl(overlaps(P.n), k, blocks, threads, 0, s, P);
   }
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? LRE_OK : cuda_fail(ctx, e, "last fold pass launch");
@@ -323,7 +330,7 @@ lre_status assemble_top_run(lre_ctx *ctx, const int64_t *T, int n, int J, int64_
     Launch L(ctx, "assemble_low6", s);
     auto k = m == 6 ? top_low6<true> : top_low6<false>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, ASM_TILE_SMEM);
-    k<<<grid(a.units), 256, ASM_TILE_SMEM, s>>>(a);
+    launch_pdl(overlaps(n), k, grid(a.units), 256, ASM_TILE_SMEM, s, a);
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "assembly launch");

@@ -9,11 +9,12 @@
 // same division and same final scale as the passes (passes.cuh), so the results
 // are the same bits.  One CTA: an n = 6 instance reads 187 KB, about 2 us of one
 // SM's share of the bandwidth, less than a grid-wide barrier per pass would
-// cost.  n = 4: 18.4 -> 8.8 us a call, most of it the host's launch.
+// cost.  n = 4: 18.4 us a call as passes; 3.1 us on the device, the host's 5 us hide it.
 #include <cuda_runtime.h>
 
 #include "lre_internal.cuh"
 #include "passes.cuh"
+#include "sm103.cuh"
 
 namespace lre {
 namespace {
@@ -53,8 +54,8 @@ __host__ __device__ constexpr int es_first_bytes() {
   return ((tile > a ? tile : a) + 15) / 16 * 16;
 }
 template <int N>
-__host__ __device__ constexpr int es_smem() {
-  return es_first_bytes<N>() + es_buf_b<N>() * 4;
+__host__ __device__ constexpr int es_smem() {  // then the parity sums
+  return es_first_bytes<N>() + es_buf_b<N>() * 4 + pw(4, N) * 4;
 }
 
 // Sums of one item of a pass over J qubits, R of them left before it: the
@@ -105,22 +106,6 @@ struct SmallTab {
   int ld[7];
 };
 
-template <int N, int J, bool FIRST, typename InT>
-__device__ __forceinline__ void es_final(const SmallArgs &P, const SmallTab &tab, const InT *in, longlong2 *tile) {
-  constexpr int C = pw(4, N - J), NP = 1 << (2 * J);
-  for (int c = threadIdx.x; c < C; c += es_threads<N>()) {
-    int32_t acc[NP];
-    es_item<N, J, J, FIRST>(in, c, acc);
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-      const int i = q * C + c, k = identity_letters((uint64_t)i, N);
-      if (i == 0 && acc[q] != P.total) latch(P.status, LRE_ERR_SHOTS_MISMATCH);
-      P.theta[i] = div_int_rn((int64_t)acc[q], tab.dint[k], tab.recip[k], tab.ld[k], tab.dn[k]);
-      if (P.rho) tile[pad16(i)] = mk((long long)acc[q] * tab.up3[k], 0ll);
-    }
-  }
-}
-
 template <int N, typename InT>
 __global__ void __launch_bounds__(es_threads<N>()) estimate_small(const __grid_constant__ SmallArgs P) {
   constexpr int T = es_threads<N>();
@@ -139,31 +124,29 @@ __global__ void __launch_bounds__(es_threads<N>()) estimate_small(const __grid_c
     tab.ld[t] = 63 - __clzll(d);
     tab.dn[t] = (uint64_t)d << (63 - tab.ld[t]);
   }
-  // ---- fold; the tile shares A, which the last pass must not read while it
-  // writes T: N = 3 and 4 read A, and keep their sums in registers over a barrier
+  sm103::pdl_wait();
+  __syncthreads();
+  sm103::pdl_trigger();
+  // ---- fold
+  int32_t *S = B + es_buf_b<N>();
   if constexpr (N <= 2) {
-    __syncthreads();
-    es_final<N, N, true>(P, tab, counts, tile);
+    es_pass<N, N, N, true>(counts, S);
+  } else if constexpr (N <= 4) {
+    es_pass<N, N, 2, true>(counts, A);
+    es_pass<N, N - 2, N - 2, false>(A, S);
   } else {
     es_pass<N, N, 2, true>(counts, A);
-    if constexpr (N <= 4) {
-      constexpr int J = N - 2, C = 16, NP = 1 << (2 * J);
-      int32_t acc[NP];
-      if (t < C) es_item<N, J, J, false>(A, t, acc);
-      __syncthreads();
-      if (t < C) {
-#pragma unroll
-        for (int q = 0; q < NP; ++q) {
-          const int i = q * C + t, k = identity_letters((uint64_t)i, N);
-          if (i == 0 && acc[q] != P.total) latch(P.status, LRE_ERR_SHOTS_MISMATCH);
-          P.theta[i] = div_int_rn((int64_t)acc[q], tab.dint[k], tab.recip[k], tab.ld[k], tab.dn[k]);
-          if (P.rho) tile[pad16(i)] = mk((long long)acc[q] * tab.up3[k], 0ll);
-        }
-      }
-    } else {
-      es_pass<N, N - 2, 2, false>(A, B);
-      es_final<N, N - 4, false>(P, tab, B, tile);
-    }
+    es_pass<N, N - 2, 2, false>(A, B);
+    es_pass<N, N - 4, N - 4, false>(B, S);
+  }
+  // ---- theta, and T into the tile: a division is a hundred instructions, so its
+  // outputs are dealt out over all threads and not left with the few that summed them
+  for (int i = t; i < pw(4, N); i += T) {
+    const int32_t s = S[i];
+    const int k = identity_letters((uint64_t)i, N);
+    if (i == 0 && s != P.total) latch(P.status, LRE_ERR_SHOTS_MISMATCH);
+    P.theta[i] = div_int_rn((int64_t)s, tab.dint[k], tab.recip[k], tab.ld[k], tab.dn[k]);
+    if (P.rho) tile[pad16(i)] = mk((long long)s * tab.up3[k], 0ll);
   }
   if (!P.rho) return;
   __syncthreads();
@@ -213,8 +196,7 @@ lre_status launch_small(lre_ctx *ctx, const SmallArgs &a, bool i16, cudaStream_t
     if (e != cudaSuccess) return cuda_fail(ctx, e, "small estimate");
   }
   Launch L(ctx, "estimate_small", s);
-  k<<<1, es_threads<N>(), smem, s>>>(a);
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_pdl(true, k, 1, es_threads<N>(), smem, s, a);
   return e == cudaSuccess ? LRE_OK : cuda_fail(ctx, e, "small estimate launch");
 }
 

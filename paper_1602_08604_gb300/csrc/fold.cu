@@ -448,7 +448,9 @@ __global__ void __launch_bounds__(FUSE ? FUSE_THREADS : PIPE_THREADS, 1)
     *abort_flag = 0;
     sm103::fence_barrier_init();
   }
+  sm103::pdl_wait();
   __syncthreads();
+  sm103::pdl_trigger();
   auto give_up = [&]() {
     *abort_flag = 1;
     latch(status, LRE_ERR_TIMEOUT);
@@ -737,9 +739,10 @@ struct PassPlan {
 
 // Build the pass schedule.  shots_bound: an upper bound on every basis' total
 // count (decides int32 vs int64 partial sums); weighted: FP64 path; first7:
-// the caller runs the raw tensor-core first pass, which may fold seven qubits.
+// the caller runs the raw tensor-core first pass, which may fold seven qubits;
+// top: rho is wanted (the last pass hands its letters to the assembly).
 std::vector<PassPlan> make_plan(int n, lre_count_kind kind, bool weighted, bool parity,
-                                int64_t shots_bound, bool aligned16, int variant, bool first7 = false) {
+                                int64_t shots_bound, bool aligned16, int variant, bool first7 = false, bool top = false) {
   std::vector<PassPlan> plan;
   int r = n, t = 0;
   int64_t C = 1;
@@ -801,8 +804,9 @@ std::vector<PassPlan> make_plan(int n, lre_count_kind kind, bool weighted, bool 
     // qubits (one at n = 7 and 10): three would hold its 64 sums, quotients and T
     // in a thread (n = 12: 418 us), and the qubits it takes are ones the assembly
     // does not have to (assemble_top.cu).  The second pass takes three from
-    // n = 10 on, for its split-plane input.
-    if (!weighted && !parity && t > 0 && plan[0].J == 6 && r > 2)
+    // n = 10 on, for its split-plane input; n = 9 without rho keeps two passes, one
+    // buffer less.
+    if (!weighted && !parity && t > 0 && plan[0].J == 6 && r > 2 && (top || n != 9))
       J = (r == 4 && t == 6) || r > 5 ? 3 : r - 2;
     const bool last = (J == r);
     t += J;
@@ -930,7 +934,7 @@ bool use_planes(lre_ctx *ctx, const std::vector<PassPlan> &plan, const FoldArgs 
 // rows of the six-qubit pass).
 std::vector<PassPlan> fold_plan(lre_ctx *ctx, const FoldArgs &a, bool weighted, bool parity, int64_t bound,
                                 bool aligned16) {
-  auto plan = make_plan(a.n, a.kind, weighted, parity, bound, aligned16, ctx->first_variant);
+  auto plan = make_plan(a.n, a.kind, weighted, parity, bound, aligned16, ctx->first_variant, false, a.T != nullptr);
   if (ctx->first7 && a.stage == 0 && !a.rec_entries && !plan.empty() && plan[0].first6 && !plan[0].fused9 &&
       tensor_variant(ctx, plan[0], a) == 0) {
     auto p7 = make_plan(a.n, a.kind, weighted, parity, bound, aligned16, ctx->first_variant, true);
@@ -1108,12 +1112,12 @@ lre_status fold_run(lre_ctx *ctx, const FoldArgs &a, void *ws, size_t ws_bytes, 
         constexpr int sm = PipeCfg<int16_t>::SMEM;
         auto k = pp.fused9 ? fold_first6_pipe<int16_t, true> : fold_first6_pipe<int16_t, false>;
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-        k<<<grid, threads, sm, s>>>(tmap, A);
+        launch_pdl(overlaps(a.n), k, grid, threads, sm, s, tmap, A);
       } else {
         constexpr int sm = PipeCfg<int32_t>::SMEM;
         auto k = pp.fused9 ? fold_first6_pipe<int32_t, true> : fold_first6_pipe<int32_t, false>;
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-        k<<<grid, threads, sm, s>>>(tmap, A);
+        launch_pdl(overlaps(a.n), k, grid, threads, sm, s, tmap, A);
       }
     } else if (pp.first6 && !pp.fused9) {
       const int64_t tiles = ipow(3, pp.r - 6) << (pp.r - 6);

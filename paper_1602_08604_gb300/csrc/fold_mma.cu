@@ -232,7 +232,9 @@ __global__ void __launch_bounds__(MmaCfg<V>::THREADS, 1)
   sm103::fence_proxy_async_smem();  // A is read by the tensor cores
   if (warp == 1 && !consumer) sm103::tmem_alloc(tmem_slot, TMEM_COLS);
   sm103::tc_fence_before();
+  if constexpr (!F9) sm103::pdl_wait();  // the operand above is written once, with the context
   __syncthreads();
+  if constexpr (!F9) sm103::pdl_trigger();
   sm103::tc_fence_after();
   const uint32_t tmem = consumer ? 0u : *tmem_slot;
   auto give_up = [&]() {
@@ -759,10 +761,10 @@ lre_status mma_first_pass(lre_ctx *ctx, const CUtensorMap &map_big, const CUtens
                                            : (seven ? fold_first6_mma<V_RAW7> : fold_first6_mma<V_RAW>));
   const int threads = variant == 3 ? MmaCfg<V_SPLIT>::THREADS : MMA_THREADS;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, MMA_SMEM);
-  kern<<<grid, threads, MMA_SMEM, s>>>(map_big, map_tail, map_tail, grid, 0, static_cast<const uint4 *>(a_dev), out,
-                                       out_hi, n, tile_begin, tile_end, nullptr, nullptr, shots, row_base, nullptr,
-                                       nullptr, ctx->d_status);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(overlaps(n), kern, grid, threads, MMA_SMEM, s, map_big, map_tail, map_tail, grid, 0,
+                             static_cast<const uint4 *>(a_dev), out, out_hi, n, tile_begin, tile_end,
+                             (const uint16_t *)nullptr, (const int32_t *)nullptr, shots, row_base, (int32_t *)nullptr,
+                             (unsigned *)nullptr, ctx->d_status);
   return e == cudaSuccess ? LRE_OK : cuda_fail(ctx, e, "tensor-core first pass launch");
 }
 

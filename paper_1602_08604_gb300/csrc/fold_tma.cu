@@ -68,7 +68,9 @@ __global__ void __launch_bounds__(tma_warps<J>() * 32, 1) fold_tma(const __grid_
     sm103::mbar_init(&bar[1], 1);
     sm103::fence_barrier_init();
   }
+  sm103::pdl_wait();
   __syncthreads();
+  sm103::pdl_trigger();
 
   const int64_t cblocks = P.C / TC;
   const int64_t tasks = P.items / TC;  // items = 3^(r-J) 2^(r-J) C
@@ -155,8 +157,7 @@ lre_status launch(lre_ctx *ctx, const CUtensorMap &map, const CUtensorMap &map_h
   int64_t grid = (tasks + TMA_WARPS - 1) / TMA_WARPS;
   const int64_t cap = (int64_t)ctx->num_sms * (smem <= 110 * 1024 ? 2 : 1);
   if (grid > cap) grid = cap;
-  k<<<(unsigned)grid, TMA_WARPS * 32, smem, s>>>(map, map_hi, P);
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_pdl(overlaps(P.n), k, grid, TMA_WARPS * 32, smem, s, map, map_hi, P);
   return e == cudaSuccess ? LRE_OK : cuda_fail(ctx, e, "TMA fold pass launch");
 }
 

@@ -6,6 +6,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/lre.h"
@@ -106,6 +107,32 @@ class Launch {
   cudaStream_t s_;
   long idx_ = -1;  // index into ctx->prof_pool (the pool may grow)
 };
+
+// Launch a kernel of the estimate's chain so that its set-up (launch, shared-memory
+// barriers, tables, the tensor cores' operand) overlaps the end of the kernel before
+// it in the stream; the kernel calls sm103::pdl_wait before its first access to
+// memory that any other kernel writes or reads.  overlap false: a plain launch.
+// overlaps(n): up to n = 10 the chain is mostly launches and drains (n = 7: 22.9 ->
+// 15.2 us on the device, n = 8: 24.9 -> 20.4, n = 9: 40 -> 30, n = 10: 91 -> 82).
+// Beyond, the early CTAs meet an SM whose shared memory is carved for the kernel
+// that is ending and stay at one or two where three fit (n = 12: 1907 -> 2002 us,
+// n = 13: 6293 -> 6915).
+inline bool overlaps(int n) { return n <= 10; }
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(bool overlap, void (*k)(KArgs...), int64_t grid, int threads, size_t smem, cudaStream_t s,
+                       Args &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
+}
 
 inline int64_t ipow(int64_t b, int e) {
   int64_t r = 1;

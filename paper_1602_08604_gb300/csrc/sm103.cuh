@@ -80,6 +80,14 @@ __device__ __forceinline__ bool poll_geq(const unsigned *p, unsigned target, vol
   }
 }
 
+// Programmatic dependent launch (launch_pdl): wait until every kernel before this
+// one in the stream is complete and its writes are visible -- nothing another
+// kernel writes may be read, and nothing it reads written, before -- and let the
+// next kernel's CTAs be set up from here on (they wait in turn).  Both do nothing
+// in a kernel launched without the attribute.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // 5D TMA tile load global -> shared (coordinates innermost first),
 // completion counted on `bar` (bytes).
 __device__ __forceinline__ void tma_load_5d(void *dst, const CUtensorMap *map, int c0, int c1, int c2, int c3,
