@@ -110,10 +110,27 @@ def _ptr(t):
     return t.data_ptr()
 
 
+def _current_stream():
+    """A function for the calling thread's current stream on the current device, as
+    a raw handle: the lookup torch's own launchers use, where this torch has it.
+    Building a Stream object for its handle cost 4 of a call's 9 us of host time,
+    three times the device time of the smallest estimates."""
+    import torch
+    if hasattr(torch._C, "_cuda_getCurrentRawStream"):
+        raw, device = torch._C._cuda_getCurrentRawStream, torch.cuda.current_device
+        return lambda: raw(device())
+    return lambda: torch.cuda.current_stream().cuda_stream
+
+
+_current = None
+
+
 def _stream(s):
+    global _current
     if s is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        if _current is None:
+            _current = _current_stream()
+        return _current()
     if isinstance(s, int):
         return s
     return s.cuda_stream
