@@ -56,25 +56,26 @@ struct BatchState {
   int abort;
 };
 
+// tab: the divisor tables of a final pass in shared memory.
 template <int JMAX>
-__device__ __forceinline__ void run_item(const BPhase &P, int64_t item) {
+__device__ __forceinline__ void run_item(const BPhase &P, int64_t item, const DivTables *tab) {
   switch (P.code) {
     case C_FOLD + 0: fold_item<1, int16_t, int32_t, M_STORE, false, true, false>(P.g, item); break;
-    case C_FOLD + 1: fold_item<1, int16_t, int64_t, M_FINAL_U, false, true, false>(P.g, item); break;
+    case C_FOLD + 1: fold_item<1, int16_t, int64_t, M_FINAL_U, false, true, false>(P.g, item, tab); break;
     case C_FOLD + 2: fold_item<1, int32_t, int32_t, M_STORE, false, true, false>(P.g, item); break;
-    case C_FOLD + 3: fold_item<1, int32_t, int64_t, M_FINAL_U, false, true, false>(P.g, item); break;
+    case C_FOLD + 3: fold_item<1, int32_t, int64_t, M_FINAL_U, false, true, false>(P.g, item, tab); break;
     case C_FOLD + 4: fold_item<1, int16_t, int32_t, M_STORE, false, false, true>(P.g, item); break;
-    case C_FOLD + 5: fold_item<1, int16_t, int64_t, M_FINAL_U, false, false, true>(P.g, item); break;
+    case C_FOLD + 5: fold_item<1, int16_t, int64_t, M_FINAL_U, false, false, true>(P.g, item, tab); break;
     case C_FOLD + 6: fold_item<1, int32_t, int32_t, M_STORE, false, false, true>(P.g, item); break;
-    case C_FOLD + 7: fold_item<1, int32_t, int64_t, M_FINAL_U, false, false, true>(P.g, item); break;
+    case C_FOLD + 7: fold_item<1, int32_t, int64_t, M_FINAL_U, false, false, true>(P.g, item, tab); break;
     case C_FOLD + 8: fold_item<2, int16_t, int32_t, M_STORE, false, true, false>(P.g, item); break;
-    case C_FOLD + 9: fold_item<2, int16_t, int64_t, M_FINAL_U, false, true, false>(P.g, item); break;
+    case C_FOLD + 9: fold_item<2, int16_t, int64_t, M_FINAL_U, false, true, false>(P.g, item, tab); break;
     case C_FOLD + 10: fold_item<2, int32_t, int32_t, M_STORE, false, true, false>(P.g, item); break;
-    case C_FOLD + 11: fold_item<2, int32_t, int64_t, M_FINAL_U, false, true, false>(P.g, item); break;
+    case C_FOLD + 11: fold_item<2, int32_t, int64_t, M_FINAL_U, false, true, false>(P.g, item, tab); break;
     case C_FOLD + 12: fold_item<2, int16_t, int32_t, M_STORE, false, false, true>(P.g, item); break;
-    case C_FOLD + 13: fold_item<2, int16_t, int64_t, M_FINAL_U, false, false, true>(P.g, item); break;
+    case C_FOLD + 13: fold_item<2, int16_t, int64_t, M_FINAL_U, false, false, true>(P.g, item, tab); break;
     case C_FOLD + 14: fold_item<2, int32_t, int32_t, M_STORE, false, false, true>(P.g, item); break;
-    case C_FOLD + 15: fold_item<2, int32_t, int64_t, M_FINAL_U, false, false, true>(P.g, item); break;
+    case C_FOLD + 15: fold_item<2, int32_t, int64_t, M_FINAL_U, false, false, true>(P.g, item, tab); break;
     case C_FOLD + 16:
       if constexpr (JMAX >= 3) fold_item<3, int16_t, int32_t, M_STORE, false, true, false>(P.g, item);
       break;
@@ -227,6 +228,7 @@ __global__ void __launch_bounds__(256, 2) batch_kernel(const BPhase *__restrict_
   NumI64::V *tile = reinterpret_cast<NumI64::V *>(bsmem);
   __shared__ int64_t s_unit;
   __shared__ int s_phase, s_ok;
+  __shared__ DivTables tab;  // of the final pass at hand
   volatile int *abort = &st->abort;
   const bool cached = nph <= BATCH_SMEM_PHASES;
   if (cached)
@@ -305,9 +307,13 @@ __global__ void __launch_bounds__(256, 2) batch_kernel(const BPhase *__restrict_
       }
     } else {
       const int64_t first = (s_unit - P.unit_begin) * P.per_unit + threadIdx.x;
+      if (P.code < C_ASM && (P.code & 1)) {  // a final pass (uniform across the CTA): it divides
+        load_div_tables(P.g, tab);
+        __syncthreads();
+      }
       for (int k = 0; k < P.per_unit; k += 256) {
         const int64_t item = first + k;
-        if (item < P.items) run_item<JMAX>(P, item);
+        if (item < P.items) run_item<JMAX>(P, item, &tab);
       }
     }
     // publish the unit: the CTA barrier orders every thread's writes before
