@@ -296,17 +296,24 @@ lre_status lre_estimate(lre_ctx *ctx, const void *counts, lre_count_kind kind, c
   if ((st = ensure_workspace(ctx, shared + tbytes + dense)) != LRE_OK) return st;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   int64_t *T = int_asm ? reinterpret_cast<int64_t *>(static_cast<char *>(ctx->ws) + shared) : nullptr;
-  if (records) {
+  FoldArgs fa{counts, kind, n, shots, shots_uniform, theta, nullptr};
+  fa.T = T;
+  if (records && records_fold_takes(ctx, counts, n, shots_uniform, dense)) {
+    st = records_fold_run(ctx, static_cast<const uint16_t *>(counts), shots_uniform, n,
+                          static_cast<char *>(ctx->ws) + shared + tbytes, ctx->ws, s);
+    if (st != LRE_OK && st != LRE_ERR_UNSUPPORTED) return st;  // no tensor map here: dense counts below
+    fa.kind = ck;
+    fa.first_done = st == LRE_OK;
+  }
+  if (records && !fa.first_done) {
     void *dc = static_cast<char *>(ctx->ws) + shared + tbytes;
     st = histogram_run(ctx, static_cast<const uint16_t *>(counts), ipow(3, n), shots_uniform, n, dc, ck, s);
     if (st != LRE_OK) return st;
-    counts = dc;
-    kind = ck;
+    fa.counts = dc;
+    fa.kind = ck;
   }
-  if (!shots && estimate_small_takes(counts, n, shots_uniform))
-    return estimate_small_run(ctx, counts, kind, n, shots_uniform, theta, rho, s);
-  FoldArgs fa{counts, kind, n, shots, shots_uniform, theta, nullptr};
-  fa.T = T;
+  if (!shots && estimate_small_takes(fa.counts, n, shots_uniform))
+    return estimate_small_run(ctx, fa.counts, fa.kind, n, shots_uniform, theta, rho, s);
   if ((st = fold_run(ctx, fa, ctx->ws, shared, s)) != LRE_OK) return st;
   if (!rho) return LRE_OK;
   if (!int_asm) return assemble_run(ctx, theta, n, rho, ctx->ws, s);

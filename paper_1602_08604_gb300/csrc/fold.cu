@@ -934,6 +934,7 @@ bool use_planes(lre_ctx *ctx, const std::vector<PassPlan> &plan, const FoldArgs 
 // rows of the six-qubit pass).
 std::vector<PassPlan> fold_plan(lre_ctx *ctx, const FoldArgs &a, bool weighted, bool parity, int64_t bound,
                                 bool aligned16) {
+  if (a.first_done) return make_plan(a.n, a.kind, false, parity, bound, true, 1, false, a.T != nullptr);
   auto plan = make_plan(a.n, a.kind, weighted, parity, bound, aligned16, ctx->first_variant, false, a.T != nullptr);
   if (ctx->first7 && a.stage == 0 && !a.rec_entries && !plan.empty() && plan[0].first6 && !plan[0].fused9 &&
       tensor_variant(ctx, plan[0], a) == 0) {
@@ -1008,9 +1009,14 @@ lre_status fold_run(lre_ctx *ctx, const FoldArgs &a, void *ws, size_t ws_bytes, 
     Launch L(ctx, "inv_shots", s);
     inv_shots_kernel<<<256, 256, 0, s>>>(a.shots, wgt, B, ctx->d_status);
   }
-  const bool planes = use_planes(ctx, plan, a);
+  const bool planes = !a.first_done && use_planes(ctx, plan, a);
   const void *in = a.counts;
   size_t k_begin = 0, k_end = plan.size();
+  if (a.first_done) {  // the six-qubit pass's output is in the workspace already, as int32
+    if (plan.size() < 2 || plan[0].J != 6) return LRE_ERR_UNSUPPORTED;
+    k_begin = 1;
+    in = bufA;
+  }
   // per-basis shots, n >= 7: the plan's first three passes (two qubits each) as one
   if (weighted && aligned16 && plan.size() >= 4 && plan[0].J + plan[1].J + plan[2].J == 6) {
     const int64_t tiles = ipow(3, a.n - 6) << (a.n - 6);

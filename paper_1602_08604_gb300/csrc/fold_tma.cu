@@ -35,15 +35,16 @@ __host__ __device__ constexpr int tma_warps() {
   return J == 3 ? 4 : 16;
 }
 
-// box bytes per task: int32 values, or split planes (2 + 1 bytes per value)
-template <int J, bool PLANES = false>
+// box bytes per task: int32 or int16 values, or split planes (2 + 1 bytes per value)
+template <int J, int IN>
 __host__ __device__ constexpr int box_bytes() {
-  return (J == 1 ? 3 : J == 2 ? 9 : 27) * (1 << J) * TC * (PLANES ? 3 : 4);
+  return (J == 1 ? 3 : J == 2 ? 9 : 27) * (1 << J) * TC * (IN == T_I24P ? 3 : IN == T_I16 ? 2 : 4);
 }
 
-// PLANES: the input is split planes (map: the uint16 low halves, map_hi: the
-// int8 high parts, one box of each per task on the same barrier).
-template <int J, typename AccT, int MODE, bool PLANES>
+// IN: the input's type, int32, int16 (the records' three-qubit sums) or split planes
+// (PLANES; map: the uint16 low halves, map_hi: the int8 high parts, one box of each
+// per task on the same barrier).
+template <int J, typename AccT, int MODE, int IN>
 __global__ void __launch_bounds__(tma_warps<J>() * 32, 1) fold_tma(const __grid_constant__ CUtensorMap map,
                                                                     const __grid_constant__ CUtensorMap map_hi,
                                                                     GenParams P) {
@@ -51,7 +52,8 @@ __global__ void __launch_bounds__(tma_warps<J>() * 32, 1) fold_tma(const __grid_
   constexpr int NA = (J == 1) ? 3 : (J == 2) ? 9 : 27;
   constexpr int NO = 1 << J;
   constexpr int NP = 1 << (2 * J);
-  constexpr int BOX = box_bytes<J, PLANES>();
+  constexpr bool PLANES = IN == T_I24P;
+  constexpr int BOX = box_bytes<J, IN>();
   constexpr int BOX_LO = NA * NO * TC * 2;  // PLANES: the uint16 box, then the int8 box
   static_assert(!PLANES || BOX_LO % 128 == 0, "TMA destinations stay 128-byte aligned");
   extern __shared__ __align__(128) uint8_t smem_raw[];
@@ -123,6 +125,8 @@ __global__ void __launch_bounds__(tma_warps<J>() * 32, 1) fold_tma(const __grid_
         if constexpr (PLANES)
           v[ol] = hi ? (AccT)(int32_t)(((uint32_t)(int32_t)SH[idx] << 16) | (uint32_t)SL[idx])
                      : (AccT)(int16_t)SL[idx];
+        else if constexpr (IN == T_I16)
+          v[ol] = (AccT)(int16_t)SL[idx];
         else
           v[ol] = (AccT)S[idx];
       }
@@ -146,12 +150,12 @@ __global__ void __launch_bounds__(tma_warps<J>() * 32, 1) fold_tma(const __grid_
   __syncwarp();
 }
 
-template <int J, typename AccT, int MODE, bool PLANES = false>
+template <int J, typename AccT, int MODE, int IN = T_I32>
 lre_status launch(lre_ctx *ctx, const CUtensorMap &map, const CUtensorMap &map_hi, const GenParams &P,
                   cudaStream_t s) {
   constexpr int TMA_WARPS = tma_warps<J>();
-  constexpr int smem = TMA_WARPS * 2 * box_bytes<J, PLANES>() + TMA_WARPS * 16 + 16 + 128;
-  auto k = fold_tma<J, AccT, MODE, PLANES>;
+  constexpr int smem = TMA_WARPS * 2 * box_bytes<J, IN>() + TMA_WARPS * 16 + 16 + 128;
+  auto k = fold_tma<J, AccT, MODE, IN>;
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   const int64_t tasks = P.items / TC;
   int64_t grid = (tasks + TMA_WARPS - 1) / TMA_WARPS;
@@ -165,14 +169,14 @@ lre_status launch(lre_ctx *ctx, const CUtensorMap &map, const CUtensorMap &map_h
 
 lre_status passes::tma_pass(lre_ctx *ctx, const GenParams &P, int J, int in_t, int acc_t, int mode, bool weight,
                             cudaStream_t s) {
-  if ((in_t != T_I32 && in_t != T_I24P) || J < 1 || J > 3 || P.C % TC != 0 || weight) return LRE_ERR_UNSUPPORTED;
+  if ((in_t != T_I32 && in_t != T_I24P && in_t != T_I16) || J < 1 || J > 3 || P.C % TC != 0 || weight) return LRE_ERR_UNSUPPORTED;
   // final passes (the correctly rounded division of every coefficient) are
   // ALU-bound and run faster in the register-load kernel at full occupancy
   if (mode != M_STORE && mode != M_PARITY) return LRE_ERR_UNSUPPORTED;
   if (acc_t != T_I32 && acc_t != T_I64) return LRE_ERR_UNSUPPORTED;
   if ((reinterpret_cast<uintptr_t>(P.in) & 15) != 0) return LRE_ERR_UNSUPPORTED;
   const bool planes = in_t == T_I24P;
-  if (planes && (J != 3 || mode != M_STORE || acc_t != T_I32)) return LRE_ERR_UNSUPPORTED;
+  if (in_t != T_I32 && (J != 3 || mode != M_STORE || acc_t != T_I32)) return LRE_ERR_UNSUPPORTED;
   const int NA = J == 1 ? 3 : J == 2 ? 9 : 27, NO = 1 << J;
   const int64_t n_ah = ipow(3, P.r - J);
   // X[ah][al][oh][ol][c], innermost first
@@ -196,7 +200,14 @@ lre_status passes::tma_pass(lre_ctx *ctx, const GenParams &P, int J, int in_t, i
                            dims, strides, box))
       return LRE_ERR_UNSUPPORTED;
     Launch L(ctx, "fold_tma", s);
-    return launch<3, int32_t, M_STORE, true>(ctx, map, map_hi, P, s);
+    return launch<3, int32_t, M_STORE, T_I24P>(ctx, map, map_hi, P, s);
+  }
+  if (in_t == T_I16) {
+    strides_of(2, strides);
+    if (!encode_tensor_map(&map, CU_TENSOR_MAP_DATA_TYPE_UINT16, P.in, 5, dims, strides, box))
+      return LRE_ERR_UNSUPPORTED;
+    Launch L(ctx, "fold_tma", s);
+    return launch<3, int32_t, M_STORE, T_I16>(ctx, map, map, P, s);
   }
   strides_of(4, strides);
   if (!encode_tensor_map_i32(&map, P.in, 5, dims, strides, box)) return LRE_ERR_UNSUPPORTED;

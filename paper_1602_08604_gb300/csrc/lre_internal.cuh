@@ -162,6 +162,9 @@ struct FoldArgs {
   // stage 1 only: `counts` holds rows [row_base, row_base + rows_in) of the
   // count matrix (rows_in = 0: all 3^n rows from row 0)
   int64_t row_base = 0, rows_in = 0;
+  // stage 0 only: the output of the six-qubit first pass is at the start of the
+  // workspace, int32 (records_fold_run); counts is not read
+  bool first_done = false;
 };
 size_t fold_workspace_bytes(int n, lre_count_kind kind, bool weighted, int64_t shots_bound,
                             int variant = 2);
@@ -277,6 +280,12 @@ size_t mma_fused9_counter_bytes();
 // records grouped by count tile (records.cu) and the first pass over them
 lre_status tile_bucket_run(lre_ctx *ctx, const uint16_t *records, int64_t tile_rows, int64_t shots, int n,
                            uint16_t *entries, int32_t *offs, cudaStream_t s);
+// Shot records -> the six-qubit pass's int32 output, without dense counts, for n <= 12
+// and at most 32767 shots (records.cu).  sums: room for the three-qubit sums; out: the
+// start of the fold workspace.
+bool records_fold_takes(lre_ctx *ctx, const void *records, int n, int64_t shots, size_t dense_bytes);
+lre_status records_fold_run(lre_ctx *ctx, const uint16_t *records, int64_t shots, int n, void *sums, void *out,
+                            cudaStream_t s);
 lre_status mma_first_pass_records(lre_ctx *ctx, const void *a_dev, const uint16_t *entries, const int32_t *offs,
                                   int64_t shots, int32_t *out, int8_t *out_hi, int n, int64_t tile_begin,
                                   int64_t tile_end, cudaStream_t s);
