@@ -279,9 +279,9 @@ struct RitzEnds {
 };
 
 // Convergence check.  The residual of a Ritz pair is beta_J |s_J|, s_J the last
-// component of its eigenvector, which one inverse-iteration solve from the
-// eigenvalue (computed to 4 eps ||T||) gives to far below the tolerance; the
-// vectors that are used get two rounds (ritz_vectors) and are looked at again.
+// component of its eigenvector, which the minors at the eigenvalue (computed to
+// 4 eps ||T||) give to far below the tolerance (tri_residual); the vectors that are
+// used come from two rounds of inverse iteration (ritz_vectors) and are looked at again.
 // Values placed less exactly will not do: an unconverged neighbour's last
 // component comes through with the value's error over their gap.
 lre_status ritz_values(lre_ctx *ctx, const KryBuffers &B, const double *alpha, const double *beta, int J, int CB,
@@ -299,8 +299,9 @@ lre_status ritz_values(lre_ctx *ctx, const KryBuffers &B, const double *alpha, c
   const double tnorm = fmax(fabs(hst[0]), fabs(hst[1]));
   const double pad = 2.0 * DBL_EPSILON * tnorm + 2.0 * DBL_MIN;
   const int m = CB + CT;
-  const size_t smem = (size_t)24 * J;
+  const size_t smem = (size_t)40 * J, rsmem = (size_t)41 * J + 48;
   e = cudaFuncSetAttribute(tri_ends_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(tri_residual, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "Ritz values");
   {
     Launch L(ctx, "kry_bisect", s);
@@ -308,7 +309,7 @@ lre_status ritz_values(lre_ctx *ctx, const KryBuffers &B, const double *alpha, c
   }
   if (want_last) {
     Launch L(ctx, "kry_residuals", s);
-    tri_residual<<<(m + 31) / 32, 32, 0, s>>>(alpha, beta, J, B.Wr, m, tnorm, B.lu, B.last);
+    tri_residual<<<m, 128, rsmem, s>>>(alpha, B.b2, J, B.Wr, tnorm, B.last);
   }
   out.w.resize(m);
   out.last.assign(m, 0.0);

@@ -224,8 +224,7 @@ __global__ void tri_bisect_kernel(const double *a, const double *b2, int64_t n, 
                                   double pivmin, double *W, int64_t j0, int64_t cnt);
 __global__ void tri_ends_kernel(const double *a, const double *b2, int n, double lo0, double hi0, double tnorm,
                                 double *W, int cb, int ct);
-__global__ void tri_residual(const double *a, const double *b, int n, const double *lam, int m, double tnorm,
-                             double *work, double *out);
+__global__ void tri_residual(const double *a, const double *b2, int n, const double *lam, double tnorm, double *out);
 __global__ void tri_last(const double *X, int n, int m, double *out);
 // Gershgorin bounds of T (stats[0], stats[1]), the largest squared
 // off-diagonal (stats[2]) and the squares b2 (one CTA of 256 threads).

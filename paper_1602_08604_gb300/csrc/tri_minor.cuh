@@ -19,6 +19,14 @@ struct Minor;
 template <>
 struct Minor<double> {
   static __device__ __forceinline__ unsigned sign(double v) { return (unsigned)(__double2hiint(v)) >> 31; }
+  static __device__ __forceinline__ bool zero(double v) {  // by the integer units: FP64 compares cost FP64 time
+    return ((__double2hiint(v) & 0x7FFFFFFF) | __double2loint(v)) == 0;
+  }
+  // 2^-exponent of the larger of the two
+  static __device__ __forceinline__ double scale(double u, double v) {
+    const int a = __double2hiint(u) & 0x7FFFFFFF, b = __double2hiint(v) & 0x7FFFFFFF;
+    return scale(__hiloint2double(a > b ? a : b, 0));
+  }
   static __device__ __forceinline__ double scale(double m) {  // 2^-exponent(m)
     int e = (__double2hiint(m) >> 20) & 0x7FF;
     e = e < 1 ? 1 : e > 2045 ? 2045 : e;
@@ -28,34 +36,45 @@ struct Minor<double> {
 template <>
 struct Minor<float> {
   static __device__ __forceinline__ unsigned sign(float v) { return __float_as_uint(v) >> 31; }
+  static __device__ __forceinline__ bool zero(float v) { return v == 0.f; }
+  static __device__ __forceinline__ float scale(float u, float v) { return scale(fmaxf(fabsf(u), fabsf(v))); }
   static __device__ __forceinline__ float scale(float m) {
     int e = (int)(__float_as_uint(m) >> 23) & 0xFF;
     e = e < 1 ? 1 : e > 253 ? 253 : e;
     return __uint_as_float((unsigned)(254 - e) << 23);
   }
 };
-// a: diagonal, nb2: minus the squared off-diagonal (nb2[k] couples k and k + 1)
+// a: diagonal, nb2: minus the squared off-diagonal (nb2[k] couples k and k + 1).
+// The entries of a whole stretch between two scalings are loaded before its steps:
+// loaded one by one, their latency is on every step's path.
 template <typename R>
 __device__ __forceinline__ int minor_count(const R *a, const R *nb2, int n, R x) {
   R pm = (R)1, p = a[0] - x;
-  unsigned sg = p == (R)0 ? 1u : Minor<R>::sign(p);
+  unsigned sg = Minor<R>::zero(p) ? 1u : Minor<R>::sign(p);
   int cnt = (int)sg;
+  auto step = [&](R ak, R bk) {
+    const R t = bk * pm;
+    pm = p;
+    p = fma(ak - x, p, t);
+    const unsigned ns = Minor<R>::zero(p) ? sg ^ 1u : Minor<R>::sign(p);
+    cnt += (int)(ns ^ sg);
+    sg = ns;
+  };
   int k = 1;
-  while (k < n) {
-    const int e = k + 8 < n ? k + 8 : n;
-    for (; k < e; ++k) {
-      const R t = nb2[k - 1] * pm;
-      pm = p;
-      p = fma(a[k] - x, p, t);
-      const unsigned ns = p == (R)0 ? sg ^ 1u : Minor<R>::sign(p);
-      cnt += (int)(ns ^ sg);
-      sg = ns;
+  for (; k + 8 <= n; k += 8) {
+    R ak[8], bk[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      ak[i] = a[k + i];
+      bk[i] = nb2[k - 1 + i];
     }
-    const R ap = fabs(p), am = fabs(pm);
-    const R f = Minor<R>::scale(ap > am ? ap : am);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) step(ak[i], bk[i]);
+    const R f = Minor<R>::scale(p, pm);
     p *= f;
     pm *= f;
   }
+  for (; k < n; ++k) step(a[k], nb2[k - 1]);
   return cnt;
 }
 
@@ -64,21 +83,29 @@ __device__ __forceinline__ int minor_count_df(const df::D1 *a, const df::D1 *nb2
   df::D1 pm{1.f, 0.f}, p = a[0] - x;
   unsigned sg = p.h == 0.f ? 1u : Minor<float>::sign(p.h);
   int cnt = (int)sg;
+  auto step = [&](df::D1 ak, df::D1 bk) {
+    const df::D1 t = bk * pm;
+    pm = p;
+    p = (ak - x) * p + t;
+    const unsigned ns = p.h == 0.f ? sg ^ 1u : Minor<float>::sign(p.h);
+    cnt += (int)(ns ^ sg);
+    sg = ns;
+  };
   int k = 1;
-  while (k < n) {
-    const int e = k + 4 < n ? k + 4 : n;
-    for (; k < e; ++k) {
-      const df::D1 t = nb2[k - 1] * pm;
-      pm = p;
-      p = (a[k] - x) * p + t;
-      const unsigned ns = p.h == 0.f ? sg ^ 1u : Minor<float>::sign(p.h);
-      cnt += (int)(ns ^ sg);
-      sg = ns;
+  for (; k + 4 <= n; k += 4) {
+    df::D1 ak[4], bk[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      ak[i] = a[k + i];
+      bk[i] = nb2[k - 1 + i];
     }
-    const float ap = fabsf(p.h), am = fabsf(pm.h), f = Minor<float>::scale(ap > am ? ap : am);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) step(ak[i], bk[i]);
+    const float f = Minor<float>::scale(p.h, pm.h);
     p = {p.h * f, p.l * f};
     pm = {pm.h * f, pm.l * f};
   }
+  for (; k < n; ++k) step(a[k], nb2[k - 1]);
   return cnt;
 }
 

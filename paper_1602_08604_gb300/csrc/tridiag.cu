@@ -5,7 +5,8 @@
 // computed only for the eigenvalues the projection needs, by inverse
 // iteration with re-orthogonalisation inside clusters of close eigenvalues
 // (the classical scheme of Wilkinson and Peters; see also Demmel, Applied
-// Numerical Linear Algebra, Sec. 5.3).  Everything is FP64.
+// Numerical Linear Algebra, Sec. 5.3).  FP64, but for the first rounds of the Krylov
+// checks' bisection.
 #include <cuda_runtime.h>
 
 #include <cfloat>
@@ -204,18 +205,25 @@ __global__ void tri_clusters(const double *lam, int m, double gap_tol, int *cl, 
 // ---- the extreme eigenvalues a Krylov check needs ----------------------------
 
 // The cb smallest and ct largest eigenvalues of T (ascending: W[0 .. cb + ct)),
-// one CTA of 128 threads each: a round evaluates the count at 128 points over
-// the bracket, both ends included, so the bracket shrinks 127-fold.  The first
-// rounds run in FP32 on the rounded T and end with the bracket widened by that
-// rounding; the FP64 rounds (five, to 4 eps ||T||) check its ends and start over
-// from [lo0, hi0] if the FP32 rounds misplaced it.  Dynamic shared memory 24 n
-// bytes.  96 values at n = 450 on average: 0.7 ms (one warp per value on the
-// pivot form: 4.1 ms).
+// one CTA of 128 threads each: a round evaluates the count at several points over
+// the bracket, both ends included.  Three rounds of 128 points run in FP32 on the
+// rounded T and three in double-float, each kind ending with the bracket widened by
+// its rounding; the last 12 bits (to 4 eps ||T||) are FP64 rounds, which check the
+// bracket's ends and start over from [lo0, hi0] if an earlier round misplaced it.
+// The FP64 pipe bounds those (three operations a step and point, 1.75 a cycle and
+// SM), so they evaluate 64 points, as many as the chain of dependent operations
+// hides.  Dynamic shared memory 40 n bytes.
+// n = 12 projection, ten checks: 6.26 -> 2.18 ms (five FP64 rounds of 128 points, the
+// entries loaded one by one, before; with 32 FP64 points a third round is needed: 3.3
+// against 2.7 ms at the time).
+constexpr int TRI_FP64_POINTS = 64;
+
 __global__ void __launch_bounds__(128) tri_ends_kernel(const double *a, const double *b2, int n, double lo0, double hi0,
                                                        double tnorm, double *W, int cb, int ct) {
   extern __shared__ __align__(16) unsigned char tri_smem[];
   double *sa = reinterpret_cast<double *>(tri_smem), *sb = sa + n;
-  float *fa = reinterpret_cast<float *>(sb + n), *fb = fa + n;
+  df::D1 *da = reinterpret_cast<df::D1 *>(sb + n), *db = da + n;
+  float *fa = reinterpret_cast<float *>(db + n), *fb = fa + n;
   __shared__ unsigned votes[4];
   // scale by a power of two near 1 / ||T||: exact
   const double sc = Minor<double>::scale(tnorm);
@@ -223,12 +231,14 @@ __global__ void __launch_bounds__(128) tri_ends_kernel(const double *a, const do
     const double d = a[k] * sc, o = k + 1 < n ? -(b2[k] * sc * sc) : 0.0;
     sa[k] = d;
     sb[k] = o;
+    da[k] = df::d1(d);
+    db[k] = df::d1(o);
     fa[k] = (float)d;
     fb[k] = (float)o;
   }
   __syncthreads();
   const int idx = blockIdx.x, j = idx < cb ? idx : n - (cb + ct) + idx;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const double L0 = lo0 * sc, H0 = hi0 * sc, tn = tnorm * sc;
   double lo = L0, hi = H0;  // count(lo) <= j < count(hi)
   // last point whose count is <= j, -1 if none
@@ -242,82 +252,184 @@ __global__ void __launch_bounds__(128) tri_ends_kernel(const double *a, const do
       if (votes[w]) k = 32 * w + 31 - __clz(votes[w]);
     return k;
   };
-  for (int it = 0; it < 3; ++it) {
-    const double h = (hi - lo) / 127.0;
-    const float x = (float)(lo + h * threadIdx.x);
-    const int k = last_below(minor_count<float>(fa, fb, n, x) <= j);
+  auto narrow = [&](int k, double h) {
     const int kk = k < 0 ? 0 : k > 126 ? 126 : k;
     hi = lo + h * (kk + 1);
     lo = lo + h * kk;
+  };
+  auto widen = [&](double by) {
+    lo = fmax(L0, lo - by);
+    hi = fmin(H0, hi + by);
+  };
+  for (int it = 0; it < 3; ++it) {
+    const double h = (hi - lo) / 127.0;
+    narrow(last_below(minor_count<float>(fa, fb, n, (float)(lo + h * t)) <= j), h);
   }
-  const double w32 = 16.0 * 5.9604644775390625e-08 * tn;  // 16 units of FP32 rounding of T
-  lo = fmax(L0, lo - w32);
-  hi = fmin(H0, hi + w32);
+  widen(0x1p-20 * tn);  // 16 units of FP32 rounding of T
+  for (int it = 0; it < 3; ++it) {
+    const double h = (hi - lo) / 127.0;
+    narrow(last_below(minor_count_df(da, db, n, df::d1(lo + h * t)) <= j), h);
+  }
+  widen(0x1p-41 * tn);  // the same of double-float, 2^-45
+  constexpr int P = TRI_FP64_POINTS;
   const double tol = 4.0 * DBL_EPSILON * tn;
   bool restarted = false;
   for (int it = 0; it < 24 && hi - lo > tol; ++it) {
-    const double h = (hi - lo) / 127.0;
-    const double x = threadIdx.x == 127 ? hi : lo + h * threadIdx.x;
-    const int k = last_below(minor_count<double>(sa, sb, n, x) <= j);
-    if ((k < 0 || k > 126) && !restarted) {
+    const double h = (hi - lo) / (P - 1.0);
+    const double x = t == P - 1 ? hi : lo + h * t;
+    const int k = last_below(t < P && minor_count<double>(sa, sb, n, x) <= j);
+    if ((k < 0 || k > P - 2) && !restarted) {
       restarted = true;
       lo = L0;
       hi = H0;
       continue;
     }
-    const int kk = k < 0 ? 0 : k > 126 ? 126 : k;
-    const double nlo = lo + h * kk, nhi = kk == 126 ? hi : lo + h * (kk + 1);
+    const int kk = k < 0 ? 0 : k > P - 2 ? P - 2 : k;
+    const double nlo = lo + h * kk, nhi = kk == P - 2 ? hi : lo + h * (kk + 1);
     if (!(nhi - nlo < hi - lo)) break;
     lo = nlo;
     hi = nhi;
   }
-  if (threadIdx.x == 0) W[idx] = 0.5 * (lo + hi) / sc;
+  if (t == 0) W[idx] = 0.5 * (lo + hi) / sc;
 }
 
-// |last component| of the unit eigenvector for each of the m eigenvalues lam,
-// one thread each: one inverse-iteration solve from start_entry, the
-// factorisation of tri_factor and the forward substitution in one pass and the
-// norm taken during the back substitution, so that nothing but the factors
-// goes through memory, lane-interleaved (work: 4 n m doubles; n = 450 on
-// average at n = 12: 0.64 ms as tri_factor, tri_solve and a norm).
-__global__ void tri_residual(const double *__restrict__ a, const double *__restrict__ b, int n,
-                             const double *__restrict__ lam, int m, double tnorm, double *work, double *out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= m) return;
-  const double x = lam[j];
-  double *ui = work + j, *u1 = ui + (size_t)n * m, *u2 = u1 + (size_t)n * m, *v = u2 + (size_t)n * m;
-  const double small = DBL_EPSILON * tnorm > DBL_MIN ? DBL_EPSILON * tnorm : DBL_MIN;
-  double p = a[0] - x, q = n > 1 ? b[0] : 0.0, pend = start_entry(0, j);
-#pragma unroll 4
-  for (int k = 0; k + 1 < n; ++k) {
-    const double lo = b[k], dk = a[k + 1] - x, up = (k + 2 < n) ? b[k + 1] : 0.0;
-    const double nxt = start_entry(k + 1, j);
-    const bool swap = fabs(lo) > fabs(p);
-    double piv = swap ? lo : p;
-    if (!swap && fabs(piv) < small) piv = small;
-    const double r = 1.0 / piv, f = (swap ? p : lo) * r;
-    const size_t at = (size_t)k * m;
-    ui[at] = r;
-    u1[at] = swap ? dk : q;
-    u2[at] = swap ? up : 0.0;
-    v[at] = swap ? nxt : pend;
-    pend = swap ? pend - f * nxt : nxt - f * pend;
-    p = swap ? q - f * dk : dk - f * q;
-    q = swap ? -f * up : up;
+// log2 |v|, and LOG_ZERO for 0
+constexpr double LOG_ZERO = -1e30;
+__device__ __forceinline__ double log2_abs(double v) {
+  const int hi = __double2hiint(v), E = (hi >> 20) & 0x7FF;
+  if (E == 0) return LOG_ZERO;
+  const float f = __uint_as_float(0x3F800000u | (((unsigned)hi & 0xFFFFFu) << 3) | ((unsigned)__double2loint(v) >> 29));
+  return (double)(E - 1023) + (double)__log2f(f);
+}
+
+// |last component| of the unit eigenvector of T for each of the eigenvalues lam, one
+// CTA each.  Column r of (T - lam)^-1 is the eigenvector to rounding where its
+// diagonal entry is largest (r is then where the vector is), and its entries are
+// products of leading and trailing principal minors F_k, P_k and off-diagonals:
+//   u_k / u_r = F_k b_k .. b_(r-1) / F_r  (k < r),   P_(k+1) b_r .. b_(k-1) / P_(r+1)  (k > r),
+// with the diagonal proportional to F_r P_(r+1) (the inverse of a Jacobi matrix,
+// Gantmacher and Krein; choosing r so: Fernando, SIAM J. Matrix Anal. Appl. 18
+// (1997) 1013).  Warp 0 runs the leading, warp 1 the trailing minors, three FP64
+// operations a step as in minor_count; warp 2 sums the off-diagonals' logarithms;
+// the rest is done in logarithms by all threads.
+// Bounded by the FP64 operations a warp issues one after the other (about 105 cycles
+// each, dependent or not).  Against the values in extended precision the residuals
+// are right to 1e-11 relative; an inverse-iteration solve, whose vector holds its
+// neighbours to eps / gap, was to 1e-4.
+// n = 12 projection, nine checks: 3.60 -> 0.67 ms (n = 10, four: 1.00 -> 0.19).
+__global__ void __launch_bounds__(128) tri_residual(const double *a, const double *b2, int n, const double *lam,
+                                                    double tnorm, double *out) {
+  extern __shared__ double tri_rs[];
+  double *sa = tri_rs, *sb = sa + n, *LB = sb + n;  // diagonal, -b^2, prefix sums of log2 |b|
+  double *G[2] = {LB + n, LB + n + (n + 1)};        // F_0 .. F_n; P_n .. P_0
+  int *eG[2] = {reinterpret_cast<int *>(G[1] + (n + 1)), reinterpret_cast<int *>(G[1] + (n + 1)) + (n / 8 + 2)};
+  __shared__ double best[4];
+  __shared__ int at[4];
+  __shared__ float part[4];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const double sc = Minor<double>::scale(tnorm), x = lam[blockIdx.x] * sc;
+  for (int k = t; k < n; k += 128) {
+    sa[k] = a[k] * sc;
+    sb[k] = k + 1 < n ? -(b2[k] * sc * sc) : 0.0;
   }
-  if (fabs(p) < small) p = small;
-  double x1 = pend / p, x2 = 0.0;
-  const double last = x1;
-  double s = x1 * x1;
-#pragma unroll 8
-  for (int k = n - 2; k >= 0; --k) {
-    const size_t at = (size_t)k * m;
-    const double xk = (v[at] - u1[at] * x1 - u2[at] * x2) * ui[at];
-    s = fma(xk, xk, s);
-    x2 = x1;
-    x1 = xk;
+  __syncthreads();
+  if (warp < 2) {
+    // entry i of G is scaled by 2^-eG[(i - 2) / 8]
+    double *g = G[warp];
+    int *e = eG[warp];
+    const int s = warp ? -1 : 1, a0 = warp ? n - 1 : 0, c0 = warp ? n - 1 : -1;
+    double pm = 1.0, p = sa[a0] - x;
+    int E = 0;
+    if (lane == 0) {
+      g[0] = 1.0;
+      g[1] = p;
+      e[0] = 0;
+    }
+    auto step = [&](double ak, double bk, int k) {
+      const double u = bk * pm;
+      pm = p;
+      p = fma(ak - x, p, u);
+      if (lane == 0) g[k + 1] = p;
+    };
+    int k = 1;
+    for (; k + 8 <= n; k += 8) {
+      double ak[8], bk[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        ak[i] = sa[a0 + s * (k + i)];
+        bk[i] = sb[c0 + s * (k + i)];
+      }
+      if (lane == 0) e[(k - 1) >> 3] = E;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) step(ak[i], bk[i], k + i);
+      const double f = Minor<double>::scale(p, pm);
+      p *= f;
+      pm *= f;
+      E += 1023 - (__double2hiint(f) >> 20);
+    }
+    if (lane == 0 && k < n) e[(k - 1) >> 3] = E;
+    for (; k < n; ++k) step(sa[a0 + s * k], sb[c0 + s * k], k);
+  } else if (warp == 2) {
+    const int c = (n + 31) / 32, k0 = lane * c < n ? lane * c : n, k1 = k0 + c < n ? k0 + c : n;
+    double sum = 0.0;
+    for (int k = k0; k < k1; ++k) {
+      LB[k] = sum;
+      if (k + 1 < n) sum += 0.5 * log2_abs(sb[k]);
+    }
+    double before = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double v = __shfl_up_sync(0xffffffffu, before, o);
+      if (lane >= o) before += v;
+    }
+    before -= sum;
+    for (int k = k0; k < k1; ++k) LB[k] += before;
   }
-  out[j] = s > 0.0 ? fabs(last) / sqrt(s) : 1.0;
+  __syncthreads();
+  auto lg = [&](int w, int i) { return log2_abs(G[w][i]) + (double)eG[w][i < 2 ? 0 : (i - 2) >> 3]; };
+  // lF(k) = log2 |F_k|, lP(k) = log2 |P_(k+1)|: P_(k+1) is entry n - 1 - k
+  double mx = 4.0 * LOG_ZERO;
+  int r = 0;
+  for (int k = t; k < n; k += 128) {
+    const double v = lg(0, k) + lg(1, n - 1 - k);
+    if (v > mx) {
+      mx = v;
+      r = k;
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double v = __shfl_xor_sync(0xffffffffu, mx, o);
+    const int k = __shfl_xor_sync(0xffffffffu, r, o);
+    if (v > mx || (v == mx && k < r)) {
+      mx = v;
+      r = k;
+    }
+  }
+  if (lane == 0) {
+    best[warp] = mx;
+    at[warp] = r;
+  }
+  __syncthreads();
+  for (int w = 0; w < 4; ++w)
+    if (best[w] > mx || (best[w] == mx && at[w] < r)) {
+      mx = best[w];
+      r = at[w];
+    }
+  const double fr = lg(0, r) - LB[r], pr = lg(1, n - 1 - r) + LB[r];
+  auto lu = [&](int k) { return k < r ? lg(0, k) - LB[k] - fr : lg(1, n - 1 - k) + LB[k] - pr; };
+  float s2 = 0.f;
+  for (int k = t; k < n; k += 128) s2 += exp2f((float)(2.0 * lu(k)));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+  if (lane == 0) part[warp] = s2;
+  __syncthreads();
+  if (t == 0) {
+    const float s = part[0] + part[1] + part[2] + part[3], l = exp2f((float)lu(n - 1));
+    // out of range, or T in pieces (a zero off-diagonal): not taken for converged
+    const bool ok = mx > 0.5 * LOG_ZERO && LB[n - 1] > 0.25 * LOG_ZERO && s >= 0.5f && s < 3.0e38f && l < 3.0e38f;
+    out[blockIdx.x] = ok ? (double)(l / sqrtf(s)) : 1.0;
+  }
 }
 
 // out[k] = |last component| / norm of column k of X (n x m), one warp each.

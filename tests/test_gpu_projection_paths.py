@@ -140,3 +140,19 @@ def test_scaled_inputs(env, n, scale):
         lre.lre_sync(ctx)
         outs.append(out.cpu().numpy().astype(np.complex128))
     assert rel_fro(outs[1] / float(np.float32(scale)), outs[0]) <= 1e-6
+
+
+@pytest.mark.parametrize("n", [7, 9, 10])
+@pytest.mark.parametrize("gap", [1e-2, 1e-5])
+def test_close_neighbours(env, n, gap):
+    """Kept values close together above a dense bulk that does not converge: the
+    residuals must tell the two apart (accepted too early, the eigenvalues are off;
+    never accepted, the reduction would run)."""
+    d = 2 ** n
+    rng = np.random.default_rng(n)
+    lam = -rng.uniform(0.0, 0.25 / d, d)
+    lam[-12:] = 0.05 * (1.0 + gap * np.arange(12))
+    lam[-24:-12] = 0.01 * (1.0 + gap * rng.uniform(0, 12, 12))
+    names, out = _run(env, _hermitian_with_spectrum(lam / lam.sum(), 29 + n), n)
+    assert "kry_residuals" in names and "hetrd(cusolver)" not in names, names
+    assert (out > 0).sum() < d // 2
