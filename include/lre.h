@@ -103,7 +103,7 @@ lre_status lre_set_workspace_limit(lre_ctx *ctx, size_t bytes);
 
 /* Workspace bytes lre_estimate needs for this n and count kind, rho
  * included (per_basis_shots != 0 for the per-basis FP64 weighting; for
- * LRE_SHOTS_U16 the dense int16 counts the records are histogrammed into,
+ * LRE_SHOTS_U16 the dense int16 counts the records may be histogrammed into,
  * i.e. at most 32767 shots per basis). */
 lre_status lre_workspace_size(lre_ctx *ctx, int n, lre_count_kind kind, int per_basis_shots,
                               size_t *bytes);
@@ -127,8 +127,9 @@ lre_status lre_parity_sums(lre_ctx *ctx, const void *counts, lre_count_kind kind
  * Eq. (4): rho = (1/2^n) sum_i theta[i] P_i.
  * counts: device [3^n][2^n] counts (LRE_COUNTS_*), or device uint16 shot
  * records [3^n][shots_uniform] (LRE_SHOTS_U16, which the call histograms into
- * dense counts in its workspace; a record >= 2^n latches
- * LRE_ERR_INVALID_ARG); shots: device int64 [3^n] per-basis totals (counts
+ * dense counts in its workspace or, for 9 <= n <= 12 and rows of 16-byte
+ * multiples with at most 1213 shots, counts and folds in shared memory, with
+ * the same results; a record >= 2^n latches LRE_ERR_INVALID_ARG); shots: device int64 [3^n] per-basis totals (counts
  * only), or NULL to use shots_uniform (> 0) for every basis; theta: device
  * FP64 [4^n]; rho: device complex64 [2^n][2^n] or NULL.  With uniform shots
  * theta is the correctly rounded quotient of two exact integers.  When the
@@ -210,7 +211,8 @@ lre_status lre_assemble_noalloc(const double *theta, int n, lre_c64 *rho, lre_st
 /* Step (iii): rho_out = argmin over density matrices sigma of
  * ||sigma - rho_in||_F (Sec. II, Smolin et al.): the eigenpairs of rho_in
  * on the needed side of the threshold (Lanczos in double-float arithmetic
- * with FP64 scalars, certified; else an FP64
+ * with FP64 scalars, certified, from n = 6 on when eig_mu is NULL; one kernel
+ * with FP64 eigenvalues up to n = 5; else an FP64
  * Hermitian eigendecomposition of rho_in promoted to complex128), the
  * eigenvalue correction onto the probability simplex, and the
  * reconstruction in FP64 rounded once to complex64.  rho_in, rho_out: device complex64

@@ -460,8 +460,8 @@ extern "C" lre_status lre_debug_set_first_grid(lre_ctx *ctx, int ctas) {
 }
 
 // Test hook (not part of include/lre.h): step (iii) through the default
-// choice (1: the Krylov path from d = 2048 on when eig_mu is not asked for,
-// else the eigenvalue-first path for d >= 64), always the eigenvalue-first
+// choice (1: one kernel for n <= 5; above, the Krylov path when eig_mu is not
+// asked for, else the eigenvalue-first path), always the eigenvalue-first
 // path with its tridiagonal reduction (2), or always the full
 // eigendecomposition (0).
 extern "C" lre_status lre_debug_set_project_mode(lre_ctx *ctx, int mode) {

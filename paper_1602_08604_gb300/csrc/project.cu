@@ -9,8 +9,10 @@
 // conj(mu); the projection commutes with conjugation, so the solver works on
 // conj(mu) and the column-major result, read back row-major, is rho_hat.
 //
-// Two ways to the spectrum and the vectors the rebuild needs:
-//   eigenvalue-first (default for d >= 64): cuSOLVER reduces conj(mu) to a
+// By default n <= 5 is one kernel (project_small.cu) and d >= 64 without eig_mu
+// the Krylov path (krylov.cu).  Here, two ways to the spectrum and the vectors the
+// rebuild needs:
+//   eigenvalue-first (d >= 64 with eig_mu, and the Krylov path's fallback): cuSOLVER reduces conj(mu) to a
 //     real tridiagonal T = Q^dag conj(mu) Q (the O(d^3) part), every
 //     eigenvalue of T comes from bisection (tridiag.cu), the Smolin walk runs
 //     on them, and eigenvectors are formed only for the smaller of the kept
@@ -18,7 +20,7 @@
 //     columns).  At n = 14 the estimate keeps a few dozen of 16384 eigenvalues,
 //     so the back-transformation of the full eigenbasis is skipped;
 //   full: cuSOLVER's divide-and-conquer eigendecomposition (Xsyevd), used
-//     for small d and whenever the needed set exceeds PARTIAL_MAX vectors.
+//     whenever the needed set exceeds PARTIAL_MAX vectors.
 //
 // Rebuild with the cheaper of two equal forms (K kept, D dropped, s = a/i):
 //   rho_hat = sum_{j in K} (l_j + s) v_j v_j^dag                       (|K| <= |D|)
