@@ -316,7 +316,7 @@ lre_status lre_estimate(lre_ctx *ctx, const void *counts, lre_count_kind kind, c
     return estimate_small_run(ctx, fa.counts, fa.kind, n, shots_uniform, theta, rho, s);
   if ((st = fold_run(ctx, fa, ctx->ws, shared, s)) != LRE_OK) return st;
   if (!rho) return LRE_OK;
-  if (!int_asm) return assemble_run(ctx, theta, n, rho, ctx->ws, s);
+  if (!int_asm) return assemble_run(ctx, theta, n, rho, ctx->ws, s, overlaps_weighted(n));
   const int top = fold_top_qubits(ctx, fa);
   return top ? assemble_top_run(ctx, T, n, top, shots_uniform, rho, ctx->ws, s)
              : assemble_int_run(ctx, T, n, shots_uniform, rho, ctx->ws, s);
@@ -328,7 +328,7 @@ lre_status lre_assemble(lre_ctx *ctx, const double *theta, int n, lre_c64 *rho, 
   if (st != LRE_OK) return st;
   if ((st = set_device(ctx)) != LRE_OK) return st;
   if ((st = ensure_workspace(ctx, assemble_workspace_bytes(n))) != LRE_OK) return st;
-  return assemble_run(ctx, theta, n, rho, ctx->ws, reinterpret_cast<cudaStream_t>(stream));
+  return assemble_run(ctx, theta, n, rho, ctx->ws, reinterpret_cast<cudaStream_t>(stream), overlaps(n));
 }
 
 lre_status lre_project(lre_ctx *ctx, const lre_c64 *rho_in, int n, lre_c64 *rho_out,

@@ -29,6 +29,7 @@
 
 #include "lre_internal.cuh"
 #include "passes.cuh"
+#include "sm103.cuh"
 
 namespace lre {
 namespace {
@@ -43,6 +44,8 @@ using namespace passes;
 // memory and come out conjugated and transposed.  Blocks (A, B) and (B, A)
 // read and write disjoint entries, so no two CTAs touch the same place.
 __global__ void __launch_bounds__(256) assemble_mirror(float2 *__restrict__ rho, int64_t d) {
+  sm103::pdl_wait();
+  sm103::pdl_trigger();
   __shared__ float2 tile[56][65];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t nb = d >> 6;
@@ -85,6 +88,8 @@ __global__ void __launch_bounds__(256) assemble_mirror(float2 *__restrict__ rho,
 
 template <class Num, int J, bool FIRST, bool LAST, bool HERM>
 __global__ void __launch_bounds__(256) assemble_pass(AsmParams P) {
+  sm103::pdl_wait();
+  sm103::pdl_trigger();
   for (int64_t item = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; item < P.items;
        item += (int64_t)gridDim.x * blockDim.x)
     asm_item<Num, J, FIRST, LAST, HERM>(P, item);
@@ -105,6 +110,8 @@ constexpr int TILE_SMEM = ASM_TILE_SMEM;
 template <class Num>
 __global__ void __launch_bounds__(256) assemble_low6(const typename Num::In *__restrict__ in,
                                                     typename Num::V *__restrict__ out, int64_t blocks) {
+  sm103::pdl_wait();
+  sm103::pdl_trigger();
   using V = typename Num::V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V *S = reinterpret_cast<V *>(smem_raw);  // 4096 + 256 padded entries
@@ -123,6 +130,8 @@ template <class Num, bool LAST>
 __global__ void __launch_bounds__(256) assemble_high4(const typename Num::V *__restrict__ in,
                                                      void *__restrict__ out, int t, int64_t units,
                                                      LastScale scale) {
+  sm103::pdl_wait();
+  sm103::pdl_trigger();
   using V = typename Num::V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V *S = reinterpret_cast<V *>(smem_raw);
@@ -176,18 +185,18 @@ __global__ void __launch_bounds__(256) assemble_high4(const typename Num::V *__r
 
 // herm: the pass runs after the tiled first pass, on the stored half only
 template <class Num, int J>
-void launch_reg(bool first, bool last, bool herm, const AsmParams &p, int grid, cudaStream_t s) {
-  if (first && last) assemble_pass<Num, J, true, true, false><<<grid, 256, 0, s>>>(p);
-  else if (first) assemble_pass<Num, J, true, false, false><<<grid, 256, 0, s>>>(p);
-  else if (last && herm) assemble_pass<Num, J, false, true, true><<<grid, 256, 0, s>>>(p);
-  else if (last) assemble_pass<Num, J, false, true, false><<<grid, 256, 0, s>>>(p);
-  else if (herm) assemble_pass<Num, J, false, false, true><<<grid, 256, 0, s>>>(p);
-  else assemble_pass<Num, J, false, false, false><<<grid, 256, 0, s>>>(p);
+void launch_reg(bool first, bool last, bool herm, const AsmParams &p, int grid, cudaStream_t s, bool overlap) {
+  if (first && last) launch_pdl(overlap, assemble_pass<Num, J, true, true, false>, grid, 256, 0, s, p);
+  else if (first) launch_pdl(overlap, assemble_pass<Num, J, true, false, false>, grid, 256, 0, s, p);
+  else if (last && herm) launch_pdl(overlap, assemble_pass<Num, J, false, true, true>, grid, 256, 0, s, p);
+  else if (last) launch_pdl(overlap, assemble_pass<Num, J, false, true, false>, grid, 256, 0, s, p);
+  else if (herm) launch_pdl(overlap, assemble_pass<Num, J, false, false, true>, grid, 256, 0, s, p);
+  else launch_pdl(overlap, assemble_pass<Num, J, false, false, false>, grid, 256, 0, s, p);
 }
 
 template <class Num>
 lre_status run_passes(lre_ctx *ctx, const typename Num::In *in0, int n, lre_c64 *rho, void *ws,
-                      LastScale scale, cudaStream_t s) {
+                      LastScale scale, cudaStream_t s, bool overlap) {
   using V = typename Num::V;
   const size_t one = (((size_t)1 << (2 * n)) * sizeof(V) + 255) & ~(size_t)255;
   char *bufs[2] = {static_cast<char *>(ws), static_cast<char *>(ws) + one};
@@ -200,7 +209,7 @@ lre_status run_passes(lre_ctx *ctx, const typename Num::In *in0, int n, lre_c64 
     {
       Launch L(ctx, "assemble_low6", s);
       cudaFuncSetAttribute(assemble_low6<Num>, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_SMEM);
-      assemble_low6<Num><<<grid, 256, TILE_SMEM, s>>>(in0, reinterpret_cast<V *>(bufs[0]), blocks);
+      launch_pdl(overlap, assemble_low6<Num>, grid, 256, TILE_SMEM, s, in0, reinterpret_cast<V *>(bufs[0]), blocks);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "assemble_low6 launch");
@@ -217,10 +226,10 @@ lre_status run_passes(lre_ctx *ctx, const typename Num::In *in0, int n, lre_c64 
         Launch L(ctx, last ? "assemble_high4_last" : "assemble_high4", s);
         if (last) {
           cudaFuncSetAttribute(assemble_high4<Num, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_SMEM);
-          assemble_high4<Num, true><<<g, 256, TILE_SMEM, s>>>(static_cast<const V *>(in), out, t, units, scale);
+          launch_pdl(overlap, assemble_high4<Num, true>, g, 256, TILE_SMEM, s, static_cast<const V *>(in), out, t, units, scale);
         } else {
           cudaFuncSetAttribute(assemble_high4<Num, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_SMEM);
-          assemble_high4<Num, false><<<g, 256, TILE_SMEM, s>>>(static_cast<const V *>(in), out, t, units, scale);
+          launch_pdl(overlap, assemble_high4<Num, false>, g, 256, TILE_SMEM, s, static_cast<const V *>(in), out, t, units, scale);
         }
       }
       e = cudaGetLastError();
@@ -246,8 +255,8 @@ lre_status run_passes(lre_ctx *ctx, const typename Num::In *in0, int n, lre_c64 
     {
       Launch L(ctx, last ? "assemble_last" : "assemble_pass", s);
       const bool herm = n >= 10;  // after the tiled first pass: the stored part only
-      if (J == 2) launch_reg<Num, 2>(first, last, herm, p, (int)blocks, s);
-      else launch_reg<Num, 1>(first, last, herm, p, (int)blocks, s);
+      if (J == 2) launch_reg<Num, 2>(first, last, herm, p, (int)blocks, s, overlap);
+      else launch_reg<Num, 1>(first, last, herm, p, (int)blocks, s, overlap);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "assemble pass launch");
@@ -261,7 +270,7 @@ lre_status run_passes(lre_ctx *ctx, const typename Num::In *in0, int n, lre_c64 
     if (g > nb * nb) g = nb * nb;
     {
       Launch L(ctx, "assemble_mirror", s);
-      assemble_mirror<<<(int)g, 256, 0, s>>>(reinterpret_cast<float2 *>(rho), 1ll << n);
+      launch_pdl(overlap, assemble_mirror, g, 256, 0, s, reinterpret_cast<float2 *>(rho), 1ll << n);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "assemble_mirror launch");
@@ -314,14 +323,14 @@ lre_status assemble_preload() {
 }
 
 lre_status assemble_run(lre_ctx *ctx, const double *theta, int n, lre_c64 *rho, void *ws,
-                        cudaStream_t s) {
-  return run_passes<NumF64>(ctx, theta, n, rho, ws, LastScale{(float)(1.0 / (double)(1ll << n)), 0.f}, s);
+                        cudaStream_t s, bool overlap) {
+  return run_passes<NumF64>(ctx, theta, n, rho, ws, LastScale{(float)(1.0 / (double)(1ll << n)), 0.f}, s, overlap);
 }
 
 lre_status assemble_int_run(lre_ctx *ctx, const int64_t *T, int n, int64_t shots, lre_c64 *rho,
                             void *ws, cudaStream_t s) {
   const LastScaleArgs a = int_assembly_scale(n, shots);
-  return run_passes<NumI64>(ctx, reinterpret_cast<const long long *>(T), n, rho, ws, LastScale{a.sh, a.sl}, s);
+  return run_passes<NumI64>(ctx, reinterpret_cast<const long long *>(T), n, rho, ws, LastScale{a.sh, a.sl}, s, overlaps(n));
 }
 
 }  // namespace lre

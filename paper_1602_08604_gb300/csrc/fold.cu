@@ -202,6 +202,8 @@ template <typename InT>
 __global__ void __launch_bounds__(P1_THREADS, 2)
     fold_first6_weighted(const InT *__restrict__ counts, const double *__restrict__ wgt, double *__restrict__ out, int n,
                          int64_t num_tiles) {
+  sm103::pdl_wait();
+  sm103::pdl_trigger();
   extern __shared__ double Zw[];  // [64][P1_ZSTRIDE]
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int64_t d = 1ll << n;
@@ -662,6 +664,8 @@ bool make_count_map(CUtensorMap *map, const void *base, lre_count_kind kind, int
 // Generic pass: one thread per (ah, oh, c) column, J <= 3 qubits in registers.
 template <int J, typename InT, typename AccT, int MODE, bool WEIGHT>
 __global__ void __launch_bounds__(256) fold_generic(GenParams P) {
+  sm103::pdl_wait();
+  sm103::pdl_trigger();
   __shared__ DivTables tab;  // uniform-shot final pass: divisor tables per k
   if constexpr (MODE == M_FINAL_U) {
     load_div_tables(P, tab);
@@ -894,6 +898,8 @@ size_t fold_workspace_bytes(int n, lre_count_kind kind, bool weighted, int64_t s
 }
 
 __global__ void inv_shots_kernel(const int64_t *shots, double *w, int64_t B, int *status) {
+  sm103::pdl_wait();
+  sm103::pdl_trigger();
   for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < B;
        b += (int64_t)gridDim.x * blockDim.x) {
     const int64_t s = shots[b];
@@ -1007,7 +1013,7 @@ lre_status fold_run(lre_ctx *ctx, const FoldArgs &a, void *ws, size_t ws_bytes, 
   const int64_t B = ipow(3, a.n);
   if (weighted) {
     Launch L(ctx, "inv_shots", s);
-    inv_shots_kernel<<<256, 256, 0, s>>>(a.shots, wgt, B, ctx->d_status);
+    launch_pdl(overlaps_weighted(a.n), inv_shots_kernel, 256, 256, 0, s, a.shots, wgt, B, ctx->d_status);
   }
   const bool planes = !a.first_done && use_planes(ctx, plan, a);
   const void *in = a.counts;
@@ -1017,19 +1023,25 @@ lre_status fold_run(lre_ctx *ctx, const FoldArgs &a, void *ws, size_t ws_bytes, 
     k_begin = 1;
     in = bufA;
   }
+  // the weighted first pass and the one after it overlap while a tile per SM is all there
+  // is: beyond, their CTAs meet the carve-out of the kernel before (n = 9: 112 us with
+  // both overlapped, 103 with the first plain, 97 with both plain)
+  const bool overlap = weighted ? overlaps_weighted(a.n) : overlaps(a.n);
+  bool early = overlap;
   // per-basis shots, n >= 7: the plan's first three passes (two qubits each) as one
   if (weighted && aligned16 && plan.size() >= 4 && plan[0].J + plan[1].J + plan[2].J == 6) {
     const int64_t tiles = ipow(3, a.n - 6) << (a.n - 6);
     const int smem = 64 * P1_ZSTRIDE * (int)sizeof(double);
     const int grid = (int)(tiles < 2 * ctx->num_sms ? tiles : 2 * ctx->num_sms);
     double *out = static_cast<double *>(bufA);  // where the third pass writes
+    early = early && tiles <= ctx->num_sms;
     Launch L(ctx, "fold_first6_weighted", s);
     if (a.kind == LRE_COUNTS_I16) {
       cudaFuncSetAttribute(fold_first6_weighted<int16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      fold_first6_weighted<int16_t><<<grid, P1_THREADS, smem, s>>>(static_cast<const int16_t *>(in), wgt, out, a.n, tiles);
+      launch_pdl(early, fold_first6_weighted<int16_t>, grid, P1_THREADS, smem, s, static_cast<const int16_t *>(in), wgt, out, a.n, tiles);
     } else {
       cudaFuncSetAttribute(fold_first6_weighted<int32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      fold_first6_weighted<int32_t><<<grid, P1_THREADS, smem, s>>>(static_cast<const int32_t *>(in), wgt, out, a.n, tiles);
+      launch_pdl(early, fold_first6_weighted<int32_t>, grid, P1_THREADS, smem, s, static_cast<const int32_t *>(in), wgt, out, a.n, tiles);
     }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "weighted first pass launch");
@@ -1183,7 +1195,7 @@ lre_status fold_run(lre_ctx *ctx, const FoldArgs &a, void *ws, size_t ws_bytes, 
         const int64_t cap = (int64_t)ctx->num_sms * 64;
         if (blocks > cap) blocks = cap;
         Launch L(ctx, pp.mode == M_STORE ? "fold_pass" : "fold_final", s);
-        kern<<<(unsigned)blocks, 256, 0, s>>>(gp);
+        launch_pdl(k == k_begin ? early : overlap, kern, blocks, 256, 0, s, gp);
       } else if (tst != LRE_OK) {
         return tst;
       }

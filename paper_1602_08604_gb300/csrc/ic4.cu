@@ -143,5 +143,5 @@ extern "C" lre_status lre_estimate_ic4(lre_ctx *ctx, const void *counts, lre_cou
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(ctx, e, "4^n-operator passes");
-  return rho ? assemble_run(ctx, theta, n, rho, ctx->ws, s) : LRE_OK;
+  return rho ? assemble_run(ctx, theta, n, rho, ctx->ws, s, overlaps(n)) : LRE_OK;
 }

@@ -118,6 +118,9 @@ class Launch {
 // that is ending and stay at one or two where three fit (n = 12: 1907 -> 2002 us,
 // n = 13: 6293 -> 6915).
 inline bool overlaps(int n) { return n <= 10; }
+// The chain of per-basis shots, for the same reason one size less (n = 4: 31 -> 20 us,
+// 7: 70 -> 54, 9: 109 -> 97; n = 10: 331 -> 345).
+inline bool overlaps_weighted(int n) { return n <= 9; }
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(bool overlap, void (*k)(KArgs...), int64_t grid, int threads, size_t smem, cudaStream_t s,
                        Args &&...args) {
@@ -185,8 +188,8 @@ bool encode_tensor_map(CUtensorMap *map, CUtensorMapDataType type, const void *b
 
 // ---- step (ii): theta -> rho -------------------------------------------------
 size_t assemble_workspace_bytes(int n);
-lre_status assemble_run(lre_ctx *ctx, const double *theta, int n, lre_c64 *rho, void *ws,
-                        cudaStream_t s);
+lre_status assemble_run(lre_ctx *ctx, const double *theta, int n, lre_c64 *rho, void *ws, cudaStream_t s,
+                        bool overlap);
 // Load the kernels of assemble_run into the current device (see assemble.cu).
 lre_status assemble_preload();
 // Text of the last failure of lre_assemble_noalloc on the calling thread.

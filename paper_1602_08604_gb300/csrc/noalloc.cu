@@ -109,7 +109,7 @@ extern "C" lre_status lre_assemble_noalloc(const double *theta, int n, lre_c64 *
   local.num_sms = sms;
   if (lre::assemble_workspace_bytes(n) > kNoallocScratchBytes)
     return fail(LRE_ERR_UNSUPPORTED, "scratch above the fixed array", cudaSuccess);
-  st = lre::assemble_run(&local, theta, n, rho, scratch, reinterpret_cast<cudaStream_t>(stream));
+  st = lre::assemble_run(&local, theta, n, rho, scratch, reinterpret_cast<cudaStream_t>(stream), lre::overlaps(n));
   if (st != LRE_OK) std::snprintf(g_error, sizeof g_error, "%s", local.last_error.c_str());
   return st;
 }

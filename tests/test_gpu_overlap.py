@@ -74,3 +74,47 @@ def test_captured_in_a_graph(n):
         assert torch.equal(t, want[0]) and torch.equal(r, want[1])
     finally:
         lre.lre_destroy(ctx)
+
+
+def test_per_basis_chain():
+    """Per-basis shots (FP64 chain, and lre_assemble): the same bits back to back, with
+    counts and totals rewritten around each call, and from a graph."""
+    torch = need_gpu()
+    lre, ctx = ctx_and_lre()
+    try:
+        sizes = (3, 6, 10, 7, 11, 9, 1, 8)
+        data = [_counts(torch, n, torch.int32, 90 + n) for n in sizes]
+        shots = [c.sum(dim=1, dtype=torch.int64) for c in data]
+        want = []
+        for n, c, sh in zip(sizes, data, shots):
+            t, r = _out(torch, n)
+            lre.lre_estimate(ctx, c, sh, n, t, r)
+            lre.lre_sync(ctx)
+            torch.cuda.synchronize()
+            want.append((t, r))
+        for _ in range(3):
+            got = []
+            for n, c, sh in zip(sizes, data, shots):
+                w, ws, (t, r) = c.clone(), sh.clone(), _out(torch, n)
+                lre.lre_estimate(ctx, w, ws, n, t, r)
+                w.zero_()
+                ws.fill_(1)
+                again = torch.empty_like(r)
+                lre.lre_assemble(ctx, t, n, again)
+                got.append((t, r, again, w, ws))
+            lre.lre_sync(ctx)
+            for a, b in zip(got, want):
+                assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1]) and torch.equal(a[2], b[1])
+        n, c, sh = 7, data[3], shots[3]
+        t, r = _out(torch, n)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            lre.lre_estimate(ctx, c, sh, n, t, r, stream=torch.cuda.current_stream())
+        for _ in range(3):
+            t.fill_(float("nan"))
+            r.zero_()
+            graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(t, want[3][0]) and torch.equal(r, want[3][1])
+    finally:
+        lre.lre_destroy(ctx)
