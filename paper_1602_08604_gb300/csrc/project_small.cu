@@ -7,7 +7,11 @@
 //   1. Householder reduction of mu to a real tridiagonal T = Q^dag mu Q (Golub
 //      and Van Loan, Matrix Computations, Sec. 8.3), the reflectors
 //      I - g u u^dag with u = x - b e_1 unnormalised, so that the reciprocal in g
-//      is off the critical path (a warp of its own forms it during the product);
+//      is off the critical path (a warp of its own forms it during the product).
+//      x is first scaled by a power of two to parts of order one (exact, and the
+//      reflector is the same): |g| <= 1 then, whatever the column's size.  Where mu
+//      has few distinct eigenvalues the columns are rounding residue of residue
+//      (1e-16, 1e-32, ...), and g = 1 / |x|^2 of such an x leaves FP32's range;
 //   2. every eigenvalue of T by multisection on Sturm counts, 128 / d points a
 //      round (tri_minor.cuh): FP32, then double-float, then FP64 to 4 eps ||T||;
 //   3. Smolin's walk, and the spectra where they are asked for;
@@ -86,12 +90,17 @@ __global__ void __launch_bounds__(PS_ALL) project_small(const float2 *mu, float2
   }
   __syncthreads();
 
-  // ---- 1. reduction: H = I - g u u^dag, g = 1 / (b (b - conj(x_0))), H^dag x = b e_1
+  // ---- 1. reduction: H = I - g u u^dag, g = 1 / (b (b - conj(x_0))), H^dag x = b e_1,
+  // for the scaled x (x, u, b and s_beta below; tb[k] is b scaled back)
   for (int k = 0; k + 1 < D; ++k) {
     const int m = D - 1 - k;  // length of the reflector: rows k + 1 ..
     if (warp == 0) {
       const int i = k + 1 + lane;
       double2 x = lane < m ? A[i * LD + k] : make_double2(0.0, 0.0);
+      const unsigned px = __double2hiint(x.x) & 0x7FFFFFFF, py = __double2hiint(x.y) & 0x7FFFFFFF;
+      const double f = Minor<double>::scale(__hiloint2double((int)__reduce_max_sync(0xffffffffu, px > py ? px : py), 0));
+      x.x *= f;
+      x.y *= f;
       const double sq = x.x * x.x + x.y * x.y;
       const double below = lane_sum<32>(lane > 0 ? sq : 0.0);
       if (lane == 0) {
@@ -100,7 +109,7 @@ __global__ void __launch_bounds__(PS_ALL) project_small(const float2 *mu, float2
         const double beta = skip ? x.x : -copysign(n2 * rsqrt(n2), x.x);
         s_skip = skip;
         s_beta = beta;
-        tb[k] = beta;
+        tb[k] = beta * Minor<double>::scale(f);
         if (skip) gam[k] = make_double2(0.0, 0.0);
         x.x -= beta;
       }
@@ -371,12 +380,19 @@ __global__ void __launch_bounds__(PS_ALL) project_small(const float2 *mu, float2
       if (j < m) Z[j][i] = z;
     }
     if (tid < m) {
-      const double x = (kept_form ? 1.0 : -1.0) * (W[off + tid] + shift);
+      const double x = (kept_form ? sc : -sc) * (W[off + tid] + shift);
       g[tid] = df::d1(x > 0.0 ? x : 0.0);
     }
   }
   __syncthreads();
-  // ---- 5. rebuild: the upper triangle and its mirror
+  // ---- 5. rebuild: the upper triangle and its mirror, of the matrix scaled as T
+  // (FP32 pairs: no input's weights leave their range), scaled back at the end by
+  // 2^-ex = dn1 dn2
+  int ex = (__double2hiint(sc) >> 20) - 1023;
+  ex = ex > 150 ? 150 : ex < -150 ? -150 : ex;  // beyond: the zero matrix
+  const float up1 = __int_as_float((127 + ex / 2) << 23), up2 = __int_as_float((127 + ex - ex / 2) << 23);
+  const float dn1 = __int_as_float((127 - ex / 2) << 23), dn2 = __int_as_float((127 - ex + ex / 2) << 23);
+  const float2 shift_s = df::split1(shift * sc);
   for (int e = tid; e < D * D; e += PS_ALL) {
     const int r = e / D, c = e % D;
     if (r > c) continue;
@@ -392,13 +408,10 @@ __global__ void __launch_bounds__(PS_ALL) project_small(const float2 *mu, float2
     s.w = -s.w;
     if (!kept_form) {
       const float2 x = mu[e];  // out may be mu: only this thread reads or writes this place and its mirror
-      s = df::add(s, make_float4(x.x, r == c ? 0.f : x.y, 0.f, 0.f));
-      if (r == c) {
-        const float2 q = df::split1(shift);
-        s = df::add(s, make_float4(q.x, 0.f, q.y, 0.f));
-      }
+      s = df::add(s, make_float4(x.x * up1 * up2, r == c ? 0.f : x.y * up1 * up2, 0.f, 0.f));
+      if (r == c) s = df::add(s, make_float4(shift_s.x, 0.f, shift_s.y, 0.f));
     }
-    const float2 o = make_float2(s.x, r == c ? 0.f : s.y);
+    const float2 o = make_float2(s.x * dn1 * dn2, r == c ? 0.f : s.y * dn1 * dn2);
     out[e] = o;
     if (r < c) out[c * D + r] = make_float2(o.x, -o.y);
   }

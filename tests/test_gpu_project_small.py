@@ -1,0 +1,105 @@
+"""lre_project for n <= 5 (one launch) on exact low-rank and structured input, whose
+tridiagonal reduction runs into columns of rounding residue, on scaled input, and on
+input that is not finite, against the oracle's Smolin projection.
+
+Tolerances: eigenvalues at FP64 rounding of the input's norm (the bound of
+test_gpu_projection_paths), the complex64 result within 1e-6 relative Frobenius."""
+import numpy as np
+import pytest
+
+from oracle import project
+from tests.gpu_util import ctx_and_lre, need_gpu, rel_fro
+
+pytestmark = pytest.mark.gpu
+
+EIG_RTOL = 2.5e-13
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = need_gpu()
+    lre, ctx = ctx_and_lre()
+    yield torch, lre, ctx
+    lre.lre_destroy(ctx)
+
+
+def _kron(vs):
+    out = np.ones(1, dtype=np.complex128)
+    for v in vs:
+        out = np.kron(out, np.asarray(v, dtype=np.complex128))
+    return out
+
+
+def _weight_state(n, k):
+    v = np.array([1.0 if bin(i).count("1") == k else 0.0 for i in range(2 ** n)], dtype=np.complex128)
+    return v / np.linalg.norm(v)
+
+
+def _cluster(n):
+    v = np.ones(2 ** n, dtype=np.complex128)
+    for i in range(2 ** n):
+        v[i] = (-1) ** bin(i & (i >> 1)).count("1")
+    return v / np.linalg.norm(v)
+
+
+def _vectors(n):
+    s = np.sqrt(0.5)
+    return {
+        "plus": _kron([[s, s]] * n),
+        "plus i": _kron([[s, 1j * s]] * n),
+        "equal product": _kron([[np.cos(0.3), np.sin(0.3)]] * n),
+        "0.8 0.6 product": _kron([[0.8, 0.6]] * n),
+        "phased product": _kron([[np.cos(0.3), np.exp(0.7j) * np.sin(0.3)]] * n),
+        "unequal product": _kron([[np.cos(0.2 + 0.3 * q), np.exp(0.4j * q) * np.sin(0.2 + 0.3 * q)] for q in range(n)]),
+        "cluster": _cluster(n),
+        "W": _weight_state(n, 1),
+        "Dicke": _weight_state(n, min(2, n)),
+    }
+
+
+def _inputs(n):
+    """Rank-one states, their mixtures with I/d, and (1 + e) P - e I/d."""
+    d = 2 ** n
+    eye = np.eye(d) / d
+    for name, v in _vectors(n).items():
+        p = np.outer(v, v.conj())
+        yield name, p
+        yield name + " + I", 0.9 * p + 0.1 * eye
+        yield name + " - I", 1.05 * p - 0.05 * eye
+
+
+def _check(env, m, n, name, eig=True):
+    torch, lre, ctx = env
+    mu = torch.from_numpy(m).cuda()
+    out = torch.full_like(mu, float("nan"))
+    em, er = [torch.full((2 ** n,), float("nan"), dtype=torch.float64, device="cuda") for _ in range(2)]
+    lre.lre_project(ctx, mu, n, out, em if eig else None, er if eig else None)
+    lre.lre_sync(ctx)
+    ref, lam_mu, lam = project.smolin(m.astype(np.complex128))
+    got = out.cpu().numpy()
+    assert np.isfinite(got.view(np.float32)).all(), name
+    assert rel_fro(got, ref) <= 1e-6, (name, rel_fro(got, ref))
+    assert np.array_equal(got, got.conj().T), name
+    if eig:
+        tol = EIG_RTOL * np.abs(lam_mu).max()
+        np.testing.assert_allclose(em.cpu().numpy(), lam_mu, rtol=0, atol=tol, err_msg=name)
+        np.testing.assert_allclose(er.cpu().numpy(), lam, rtol=0, atol=tol, err_msg=name)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("eig", [True, False])
+def test_structured_states(env, n, eig):
+    for name, m in _inputs(n):
+        _check(env, m.astype(np.complex64), n, name, eig)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("scale", [1e-30, 1e-20, 1e-9, 1e12, 1e30])
+def test_scaled_inputs(env, n, scale):
+    """The projection keeps the input's trace, so it scales with it."""
+    rng = np.random.default_rng(n)
+    g = rng.standard_normal((2 ** n, 2 ** n)) + 1j * rng.standard_normal((2 ** n, 2 ** n))
+    noisy = _vectors(n)["W"]
+    noisy = np.outer(noisy, noisy.conj()) + 0.05 * (g + g.conj().T) / 2 ** n
+    for name, m in list(_inputs(n)) + [("noisy", noisy)]:
+        _check(env, (m * scale).astype(np.complex64), n, "%s x %g" % (name, scale))
