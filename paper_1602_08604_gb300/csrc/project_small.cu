@@ -280,16 +280,20 @@ __global__ void __launch_bounds__(PS_ALL) project_small(const float2 *mu, float2
   const int m = kept_form ? kept : D - kept, off = kept_form ? D - kept : 0;
   // ---- 4. vectors: inverse iteration on the scaled T, one lane per vector
   if (warp == 0) {
-    const float small = (float)(DBL_EPSILON * tn);
+    // a remainder p below double-float's rounding of T is noise, and raised to it
+    // before the pivot is chosen (T changes by as little): where the blocks T falls
+    // into share an eigenvalue (a projector's do), every block's vector then grows
+    // alike in a solve.  With a floor of eps ||T||, or none where the coupling becomes
+    // the pivot, one vector drowned the others beyond what the second round recovers.
+    const float small = (float)(0x1p-47 * tn);
     if (lane < m) {
       const D1 x = df::d1(W[off + lane] * sc);
       D1 p = da[0] - x, q = db[0];
       for (int k = 0; k + 1 < D; ++k) {
         const D1 lo = db[k], dk = da[k + 1] - x, up = k + 2 < D ? db[k + 1] : D1{0.f, 0.f};
+        if (fabsf(p.h) < small) p = {small, 0.f};
         const bool swap = fabsf(lo.h) > fabsf(p.h);
-        D1 piv = swap ? lo : p;
-        if (!swap && fabsf(piv.h) < small) piv = {small, 0.f};
-        const D1 r = df::reciprocal(piv), f = (swap ? p : lo) * r;
+        const D1 r = df::reciprocal(swap ? lo : p), f = (swap ? p : lo) * r;
         lu[0][k][lane] = r;
         lu[1][k][lane] = swap ? dk : q;
         lu[2][k][lane] = swap ? up : D1{0.f, 0.f};

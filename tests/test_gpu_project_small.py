@@ -103,3 +103,38 @@ def test_scaled_inputs(env, n, scale):
     noisy = np.outer(noisy, noisy.conj()) + 0.05 * (g + g.conj().T) / 2 ** n
     for name, m in list(_inputs(n)) + [("noisy", noisy)]:
         _check(env, (m * scale).astype(np.complex64), n, "%s x %g" % (name, scale))
+
+
+_PAULI = [np.eye(2), np.array([[0, 1], [1, 0]]), np.array([[0, -1j], [1j, 0]]), np.diag([1, -1])]
+
+
+def _stabilizer(n, k, rng):
+    """The state of k commuting Pauli strings of value +-1: a projector of rank 2^(n-k), over its rank."""
+    d = 2 ** n
+    rho, done = np.eye(d, dtype=np.complex128), []
+    while len(done) < k:
+        p = np.ones((1, 1), dtype=np.complex128)
+        for _ in range(n):
+            p = np.kron(p, _PAULI[rng.integers(4)])
+        t = rho @ (np.eye(d) + rng.choice([-1, 1]) * p) / 2
+        if all(np.allclose(p @ g, g @ p) for g in done) and 0.4 < np.trace(t).real / np.trace(rho).real < 0.6:
+            rho = t
+            done.append(p)
+    return rho / np.trace(rho).real
+
+
+@pytest.mark.parametrize("n", [2, 3, 4, 5])
+def test_projectors(env, n):
+    """Eigenvalues of high multiplicity, T in many blocks: stabilizer projectors, sums of
+    two, and (1 + e) P - e I/d."""
+    rng = np.random.default_rng(n)
+    eye = np.eye(2 ** n) / 2 ** n
+    plus, minus = _vectors(n)["plus"], _kron([[np.sqrt(0.5), -np.sqrt(0.5)]] * n)
+    _check(env, (0.5 * np.outer(plus, plus) + 0.5 * np.outer(minus, minus)).astype(np.complex64), n, "plus and minus")
+    for it in range(150):
+        m = _stabilizer(n, int(rng.integers(1, n + 1)), rng)
+        if it % 3 == 2:
+            w = rng.choice([0.5, rng.uniform(0.1, 0.9)])
+            m = w * m + (1 - w) * _stabilizer(n, int(rng.integers(1, n + 1)), rng)
+        e = rng.choice([0.0, 0.05, 0.3, -0.2])
+        _check(env, ((1 + e) * m - e * eye).astype(np.complex64), n, "projector %d" % it, eig=it % 2 == 0)
