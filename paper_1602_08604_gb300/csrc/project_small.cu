@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(PS_ALL) project_small(const float2 *mu, float2
     const double sc = Minor<double>::scale(tn);
     if (lane < D) {
       const double o = lane + 1 < D ? tb[lane] * sc : 0.0;
-      nb2[lane] = -(o * o);
+      nb2[lane] = o * o < MIN_COUPLING ? 0.0 : -(o * o);
       W[lane] = ta[lane] * sc;  // the scaled diagonal until the values are known
       fa[lane] = (float)W[lane];
       fb[lane] = (float)nb2[lane];

@@ -14,6 +14,13 @@ namespace lre {
 // form above has a division on the critical path.  T is scaled to norm 1 or so
 // by the caller, and every eighth step both terms are scaled by a power of two
 // (exact); a zero minor counts as a sign change, as the pivot form's -pivmin.
+// Where a coupling is zero T falls into two blocks and the recurrence starts over
+// (p = 1): carried on after a zero minor, p and p_{k-1} would both stay 0 and
+// every further row would count.  Callers set squared couplings below
+// MIN_COUPLING to zero (an eigenvalue moves by 2^-60 ||T|| at most): smaller ones
+// would take the eight steps between scalings below FP64's range, or FP32's.
+constexpr double MIN_COUPLING = 0x1p-120;
+
 template <typename R>
 struct Minor;
 template <>
@@ -53,6 +60,10 @@ __device__ __forceinline__ int minor_count(const R *a, const R *nb2, int n, R x)
   unsigned sg = Minor<R>::zero(p) ? 1u : Minor<R>::sign(p);
   int cnt = (int)sg;
   auto step = [&](R ak, R bk) {
+    if (Minor<R>::zero(bk)) {
+      p = (R)1;
+      sg = 0u;
+    }
     const R t = bk * pm;
     pm = p;
     p = fma(ak - x, p, t);
@@ -84,6 +95,10 @@ __device__ __forceinline__ int minor_count_df(const df::D1 *a, const df::D1 *nb2
   unsigned sg = p.h == 0.f ? 1u : Minor<float>::sign(p.h);
   int cnt = (int)sg;
   auto step = [&](df::D1 ak, df::D1 bk) {
+    if (bk.h == 0.f) {
+      p = {1.f, 0.f};
+      sg = 0u;
+    }
     const df::D1 t = bk * pm;
     pm = p;
     p = (ak - x) * p + t;

@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(128) tri_ends_kernel(const double *a, const do
   // scale by a power of two near 1 / ||T||: exact
   const double sc = Minor<double>::scale(tnorm);
   for (int k = threadIdx.x; k < n; k += 128) {
-    const double d = a[k] * sc, o = k + 1 < n ? -(b2[k] * sc * sc) : 0.0;
+    const double d = a[k] * sc, q = k + 1 < n ? b2[k] * sc * sc : 0.0, o = q < MIN_COUPLING ? 0.0 : -q;
     sa[k] = d;
     sb[k] = o;
     da[k] = df::d1(d);
@@ -452,4 +452,34 @@ __global__ void tri_last(const double *X, int n, int m, double *out) {
   if (lane == 0) out[k] = s > 0.0 ? fabs(v[n - 1]) * inv / sqrt(s) : 1.0;
 }
 
+namespace {
+__global__ void minor_counts(const double *a, const double *nb2, int n, const double *x, int m, int *out) {
+  extern __shared__ __align__(16) unsigned char mc_smem[];
+  df::D1 *da = reinterpret_cast<df::D1 *>(mc_smem), *db = da + n;
+  float *fa = reinterpret_cast<float *>(db + n), *fb = fa + n;
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    da[k] = df::d1(a[k]);
+    db[k] = df::d1(nb2[k]);
+    fa[k] = (float)a[k];
+    fb[k] = (float)nb2[k];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+    out[3 * i] = minor_count<double>(a, nb2, n, x[i]);
+    out[3 * i + 1] = minor_count_df(da, db, n, df::d1(x[i]));
+    out[3 * i + 2] = minor_count<float>(fa, fb, n, (float)x[i]);
+  }
+}
+}  // namespace
+
 }  // namespace lre
+
+// Test hook (not part of include/lre.h): the Sturm counts at m points of T (device
+// arrays; nb2 minus the squared couplings, n <= 1024) in FP64, double-float and FP32.
+extern "C" lre_status lre_debug_minor_counts(lre_ctx *ctx, const double *a, const double *nb2, int n, const double *x,
+                                             int m, int *out) {
+  if (!ctx || !a || !nb2 || !x || !out || n < 1 || n > 1024 || m < 1) return LRE_ERR_INVALID_ARG;
+  lre::minor_counts<<<1, 128, (size_t)n * 24>>>(a, nb2, n, x, m, out);
+  const cudaError_t e = cudaDeviceSynchronize();
+  return e == cudaSuccess ? LRE_OK : lre::cuda_fail(ctx, e, "minor counts");
+}
