@@ -138,3 +138,20 @@ def test_projectors(env, n):
             m = w * m + (1 - w) * _stabilizer(n, int(rng.integers(1, n + 1)), rng)
         e = rng.choice([0.0, 0.05, 0.3, -0.2])
         _check(env, ((1 + e) * m - e * eye).astype(np.complex64), n, "projector %d" % it, eig=it % 2 == 0)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5])
+def test_diagonal_eigenvalues(env, n):
+    """Diagonal input is its own tridiagonal form, and its counts are exact: what is left
+    is half the last bracket, eps ||mu|| wide, and the rounding of its middle."""
+    torch, lre, ctx = env
+    rng = np.random.default_rng(n)
+    for it in range(40):
+        lam = rng.standard_normal(2 ** n).astype(np.float32)
+        mu = torch.from_numpy(np.diag(lam).astype(np.complex64)).cuda()
+        em = torch.empty(2 ** n, dtype=torch.float64, device="cuda")
+        lre.lre_project(ctx, mu, n, torch.empty_like(mu), em)
+        lre.lre_sync(ctx)
+        want = np.sort(lam.astype(np.float64))[::-1]
+        tol = np.finfo(np.float64).eps * np.abs(want).max()
+        np.testing.assert_allclose(em.cpu().numpy(), want, rtol=0, atol=tol)
