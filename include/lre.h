@@ -218,7 +218,11 @@ lre_status lre_assemble_noalloc(const double *theta, int n, lre_c64 *rho, lre_st
  * reconstruction in FP64 rounded once to complex64.  rho_in, rho_out: device complex64
  * [2^n][2^n] (may alias); eig_mu, eig_rho: device FP64 [2^n] or NULL,
  * receiving the spectra of rho_in and rho_out in decreasing order.  The call
- * synchronises `stream` once (to size the reconstruction). */
+ * synchronises `stream`: for n <= 5 once, at its end; above, before the
+ * reconstruction, once or (Lanczos) at every convergence check.  An input that
+ * is not finite, or a failing eigensolver, is LRE_ERR_EIG_FAILED.  For n <= 5
+ * the call may be captured in a CUDA graph; that error is then latched for
+ * lre_sync. */
 lre_status lre_project(lre_ctx *ctx, const lre_c64 *rho_in, int n, lre_c64 *rho_out,
                        double *eig_mu, double *eig_rho, lre_stream stream);
 

@@ -196,8 +196,8 @@ lre_status lre_create(lre_ctx **out, int device) {
   ctx->device = device;
   cudaError_t e = cudaSetDevice(device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device);
-  if (e == cudaSuccess) e = cudaMalloc(&ctx->d_status, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(ctx->d_status, 0, sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&ctx->d_status, 2 * sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(ctx->d_status, 0, 2 * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&ctx->mma_operand, lre::mma_operand_bytes());
   if (e != cudaSuccess) {
     lre_status st = cuda_fail(ctx, e, "lre_create");
@@ -377,7 +377,7 @@ lre_status lre_sync(lre_ctx *ctx, lre_stream stream) {
   int code = 0;
   cudaError_t e = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = cudaMemcpy(&code, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess && code != 0) e = cudaMemset(ctx->d_status, 0, sizeof(int));
+  if (e == cudaSuccess && code != 0) e = cudaMemset(ctx->d_status, 0, 2 * sizeof(int));
   if (e != cudaSuccess) return cuda_fail(ctx, e, "lre_sync");
   return static_cast<lre_status>(code);
 }

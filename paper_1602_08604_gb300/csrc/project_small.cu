@@ -56,9 +56,11 @@ __device__ __forceinline__ double lane_sum(double v) {  // over W consecutive la
   return v;
 }
 
+// *info = 1 where T is not finite (nothing is written to the outputs then), else 0;
+// info NULL: LRE_ERR_EIG_FAILED is latched in status instead.
 template <int D>
 __global__ void __launch_bounds__(PS_ALL) project_small(const float2 *mu, float2 *out, double *eig_mu,
-                                                        double *eig_rho) {
+                                                        double *eig_rho, int *info, int *status) {
   using df::D1;
   constexpr int LD = D + 1;                 // padded row
   constexpr int M = D / 2;                  // most vectors formed
@@ -78,7 +80,7 @@ __global__ void __launch_bounds__(PS_ALL) project_small(const float2 *mu, float2
   __shared__ D1 X[M][D];
   __shared__ D1 g[M];
   __shared__ double s_tn, s_lo, s_hi, s_shift, s_beta;
-  __shared__ int s_kept, s_skip;
+  __shared__ int s_kept, s_skip, s_bad;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
   for (int e = tid; e < D * D; e += PS_ALL) {
@@ -164,8 +166,10 @@ __global__ void __launch_bounds__(PS_ALL) project_small(const float2 *mu, float2
   // ---- 2. eigenvalues of T (scaled by a power of two near 1 / ||T||)
   if (warp == 0) {
     double lo = 1e308, hi = -1e308;
+    bool bad = false;
     if (lane < D) {
       const double d = A[lane * LD + lane].x;
+      bad = !isfinite(d) || (lane + 1 < D && !isfinite(tb[lane]));
       const double l = lane > 0 ? fabs(tb[lane - 1]) : 0.0, r = lane + 1 < D ? fabs(tb[lane]) : 0.0;
       ta[lane] = d;
       lo = d - l - r;
@@ -188,13 +192,20 @@ __global__ void __launch_bounds__(PS_ALL) project_small(const float2 *mu, float2
       db[lane] = df::d1(o);
       dn[lane] = df::d1(nb2[lane]);
     }
+    bad = __any_sync(0xffffffffu, bad);
     if (lane == 0) {
+      s_bad = bad;
       s_tn = tn;
       s_lo = (lo - pad) * sc;
       s_hi = (hi + pad) * sc;
     }
   }
   __syncthreads();
+  if (tid == 0) {
+    if (info) *info = s_bad;
+    else if (s_bad) latch(status, LRE_ERR_EIG_FAILED);
+  }
+  if (s_bad) return;
   const double sc = Minor<double>::scale(s_tn), tn = s_tn * sc;
   {
     constexpr int P = 128 / D < 32 ? 128 / D : 32;  // points per value and round
@@ -435,19 +446,31 @@ lre_status project_small_run(lre_ctx *ctx, const lre_c64 *rho_in, int n, lre_c64
                              double *eig_rho, cudaStream_t s) {
   const float2 *in = reinterpret_cast<const float2 *>(rho_in);
   float2 *out = reinterpret_cast<float2 *>(rho_out);
+  // the status is read back, as after the library's solver; a capture cannot wait for
+  // it, and a replay reports through lre_sync
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(s, &cap);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "projection");
+  int *const info = cap == cudaStreamCaptureStatusNone ? ctx->d_status + 1 : nullptr, *const st = ctx->d_status;
   {
     Launch L(ctx, "project_small", s);
     switch (n) {
-      case 1: project_small<2><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho); break;
-      case 2: project_small<4><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho); break;
-      case 3: project_small<8><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho); break;
-      case 4: project_small<16><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho); break;
-      case 5: project_small<32><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho); break;
+      case 1: project_small<2><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho, info, st); break;
+      case 2: project_small<4><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho, info, st); break;
+      case 3: project_small<8><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho, info, st); break;
+      case 4: project_small<16><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho, info, st); break;
+      case 5: project_small<32><<<1, PS_ALL, 0, s>>>(in, out, eig_mu, eig_rho, info, st); break;
       default: return LRE_ERR_UNSUPPORTED;
     }
   }
-  const cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? LRE_OK : cuda_fail(ctx, e, "projection");
+  e = cudaGetLastError();
+  int bad = 0;
+  if (e == cudaSuccess && info) e = cudaMemcpyAsync(&bad, info, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess && info) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "projection");
+  if (!bad) return LRE_OK;
+  ctx->last_error = "projection: the input's tridiagonal form is not finite";
+  return LRE_ERR_EIG_FAILED;
 }
 
 }  // namespace lre

@@ -155,3 +155,60 @@ def test_diagonal_eigenvalues(env, n):
         want = np.sort(lam.astype(np.float64))[::-1]
         tol = np.finfo(np.float64).eps * np.abs(want).max()
         np.testing.assert_allclose(em.cpu().numpy(), want, rtol=0, atol=tol)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("value", [np.nan, np.inf, complex(0, np.nan)])
+def test_input_that_is_not_finite_is_reported(env, n, value):
+    torch, lre, ctx = env
+    d = 2 ** n
+    for r, c in ((0, 0), (0, d - 1), (d - 2, d - 1), (d - 1, d - 1)):
+        if r == c and np.isfinite(np.real(value)):
+            continue  # the diagonal's imaginary part is not read
+        m = (np.eye(d) / d).astype(np.complex64)
+        m[r, c] = value
+        mu = torch.from_numpy(m).cuda()
+        out = torch.full_like(mu, 3.0)
+        with pytest.raises(lre.LreError) as e:
+            lre.lre_project(ctx, mu, n, out)
+        assert e.value.status == lre.LRE_ERR_EIG_FAILED
+        lre.lre_sync(ctx)
+        assert (out == 3.0).all()
+    _check(env, (np.eye(d) / d).astype(np.complex64), n, "the next call")
+
+
+@pytest.mark.parametrize("n", [1, 4])
+def test_the_call_synchronises(env, n):
+    torch, lre, ctx = env
+    mu = (torch.eye(2 ** n, dtype=torch.complex64) / 2 ** n).cuda()
+    out = torch.empty_like(mu)
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        torch.cuda._sleep(20_000_000)
+        lre.lre_project(ctx, mu, n, out, stream=stream)
+        assert stream.query()
+    assert torch.equal(out, mu)
+
+
+def test_captured_in_a_graph(env):
+    torch, lre, ctx = env
+    n = 4
+    g = torch.Generator().manual_seed(1)
+    a, b = [torch.randn((16, 16), dtype=torch.complex64, generator=g) for _ in range(2)]
+    a, b = [((x + x.conj().T) / 16).cuda() for x in (a, b)]
+    want = torch.empty_like(b)
+    lre.lre_project(ctx, b, n, want)
+    mu, out = a.clone(), torch.empty_like(a)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        lre.lre_project(ctx, mu, n, out, stream=torch.cuda.current_stream())
+    mu.copy_(b)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+    mu[0, 0] = float("nan")
+    graph.replay()
+    with pytest.raises(lre.LreError) as e:
+        lre.lre_sync(ctx)
+    assert e.value.status == lre.LRE_ERR_EIG_FAILED
