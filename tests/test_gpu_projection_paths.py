@@ -156,3 +156,21 @@ def test_close_neighbours(env, n, gap):
     names, out = _run(env, _hermitian_with_spectrum(lam / lam.sum(), 29 + n), n)
     assert "kry_residuals" in names and "hetrd(cusolver)" not in names, names
     assert (out > 0).sum() < d // 2
+
+
+@pytest.mark.parametrize("n", [7, 8, 9])
+def test_missed_copy_close_to_the_threshold(env, n):
+    """A kept eigenvalue with an exact copy (a Krylov space sees one until rounding brings
+    in the other, which the spread of the rest delays) 4e-11 above the threshold: the
+    certification must find the copy and the reduction run."""
+    d = 2 ** n
+    b = 2.0 ** -10 * (1 + 2.0 ** -23)
+    lam = np.empty(d)
+    lam[:4] = 1 + 2.0 ** -10, b, b, 0.93 * b
+    mean = (1.0 - lam[:4].sum()) / (d - 4)
+    lam[4:] = mean + (0.86 * b - mean) * np.linspace(-1.0, 1.0, d - 4)
+    lam[4:] = np.round(lam[4:] * 2.0 ** 33) / 2.0 ** 33
+    lam[4 + (d - 4) // 2] += 1.0 - lam.sum()
+    names, out = _run(env, np.diag(lam).astype(np.complex64), n)
+    assert (out > 0).sum() == 3
+    assert "hetrd(cusolver)" in names, names
