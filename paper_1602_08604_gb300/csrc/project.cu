@@ -49,6 +49,41 @@ __global__ void promote_kernel(const float2 *in, double2 *a, double2 *b, int64_t
   }
 }
 
+// acc = the largest |part| of mu as float bits (an integer maximum; zeroed by the caller).
+__global__ void largest_part(const float2 *in, int64_t N, unsigned *acc) {
+  unsigned v = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned x = __float_as_uint(in[i].x) & 0x7FFFFFFFu, y = __float_as_uint(in[i].y) & 0x7FFFFFFFu;
+    v = max(v, max(x, y));
+  }
+  v = __reduce_max_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) atomicMax(acc, v);
+}
+
+// a[i] += 2^-60 of the largest part, times a number in [-1, 1) by place.
+__global__ void dither_kernel(double2 *a, int64_t N, const unsigned *largest) {
+  const double s = (double)__uint_as_float(*largest) * 0x1p-60;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+    uint64_t z = 0x9E3779B97F4A7C15ull * (uint64_t)(i + 1);
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    z ^= z >> 31;
+    a[i].x += s * ((double)(int32_t)z * 0x1p-31);
+    a[i].y += s * ((double)(int32_t)(z >> 32) * 0x1p-31);
+  }
+}
+
+// *ok = 1.0 where the reduction's T and reflectors are finite, else 0.0 (one CTA).
+__global__ void reduction_finite(const double *ta, const double *tb, const double2 *tau, int64_t d, double *ok) {
+  bool good = true;
+  for (int64_t i = threadIdx.x; i < d; i += blockDim.x) {
+    good = good && isfinite(ta[i]);
+    if (i + 1 < d) good = good && isfinite(tb[i]) && isfinite(tau[i].x) && isfinite(tau[i].y);
+  }
+  good = __syncthreads_and(good);
+  if (threadIdx.x == 0) *ok = good ? 1.0 : 0.0;
+}
+
 // Serial Smolin walk over the ascending spectrum W (one thread).
 __global__ void smolin_kernel(const double *W, int64_t d, SmolinResult *res) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
@@ -325,23 +360,43 @@ lre_status project_partial(lre_ctx *ctx, cusolverDnHandle_t solver, cublasHandle
     Launch L(ctx, "promote", s);
     promote_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const float2 *>(rho_in), A, C, d * d);
   }
-  {
-    Launch L(ctx, "hetrd(cusolver)", s, 0);
-    if (cusolverDnZhetrd(solver, CUBLAS_FILL_MODE_LOWER, N, reinterpret_cast<cuDoubleComplex *>(A), N, ta, tb,
-                         reinterpret_cast<cuDoubleComplex *>(tau), reinterpret_cast<cuDoubleComplex *>(work),
-                         lw_trd, info) != CUSOLVER_STATUS_SUCCESS) {
-      ctx->last_error = "cusolverDnZhetrd failed";
+  double hst[4];
+  cudaError_t e = cudaSuccess;
+  for (int attempt = 0;; ++attempt) {
+    {
+      Launch L(ctx, "hetrd(cusolver)", s, 0);
+      if (cusolverDnZhetrd(solver, CUBLAS_FILL_MODE_LOWER, N, reinterpret_cast<cuDoubleComplex *>(A), N, ta, tb,
+                           reinterpret_cast<cuDoubleComplex *>(tau), reinterpret_cast<cuDoubleComplex *>(work),
+                           lw_trd, info) != CUSOLVER_STATUS_SUCCESS) {
+        ctx->last_error = "cusolverDnZhetrd failed";
+        return LRE_ERR_EIG_FAILED;
+      }
+    }
+    {
+      Launch L(ctx, "tri_prepare", s, 2);
+      tri_prepare<<<1, 256, 0, s>>>(ta, tb, d, tb2, stats);
+      reduction_finite<<<1, 256, 0, s>>>(ta, tb, tau, d, stats + 3);
+    }
+    e = cudaMemcpyAsync(hst, stats, sizeof(hst), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "tridiagonal bounds");
+    if (hst[3] == 1.0) break;
+    if (attempt == 1) {
+      ctx->last_error = "projection: the tridiagonal reduction is not finite";
       return LRE_ERR_EIG_FAILED;
     }
+    // Exactly structured input of low rank (a stabilizer state, say) leaves columns of
+    // rounding residue of residue, 1e-16, 1e-32, ..., whose reflectors underflow in the
+    // library.  Once more on mu plus 2^-60 of its largest part, far below FP64's rounding
+    // of the reduction: the residue is then a full block of that size.
+    Launch L(ctx, "dither", s, 3);
+    unsigned *const largest = reinterpret_cast<unsigned *>(stats);
+    e = cudaMemsetAsync(largest, 0, sizeof(unsigned), s);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "tridiagonal reduction");
+    largest_part<<<grid, 256, 0, s>>>(reinterpret_cast<const float2 *>(rho_in), d * d, largest);
+    promote_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const float2 *>(rho_in), A, C, d * d);
+    dither_kernel<<<grid, 256, 0, s>>>(A, d * d, largest);
   }
-  {
-    Launch L(ctx, "tri_prepare", s);
-    tri_prepare<<<1, 256, 0, s>>>(ta, tb, d, tb2, stats);
-  }
-  double hst[3];
-  cudaError_t e = cudaMemcpyAsync(hst, stats, sizeof(hst), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "tridiagonal bounds");
   const double tnorm = fmax(fabs(hst[0]), fabs(hst[1]));
   const double pivmin = DBL_MIN * fmax(1.0, hst[2]);
   const double pad = 2.0 * DBL_EPSILON * tnorm + 2.0 * pivmin;

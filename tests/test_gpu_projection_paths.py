@@ -174,3 +174,38 @@ def test_missed_copy_close_to_the_threshold(env, n):
     names, out = _run(env, np.diag(lam).astype(np.complex64), n)
     assert (out > 0).sum() == 3
     assert "hetrd(cusolver)" in names, names
+
+
+@pytest.mark.parametrize("n", [6, 7, 8])
+@pytest.mark.parametrize("mixed", [0.0, 0.1, -0.05])
+def test_reduction_of_structured_states(env, n, mixed):
+    """Few nonzero amplitudes of equal size: the reduction's trailing columns are rounding
+    residue of residue, and the library's reflectors of those are not finite at n = 6."""
+    torch, lre, ctx = env
+    d = 2 ** n
+    v = np.zeros(d, np.complex128)
+    v[[8, 19, 33, 58]] = 0.5, 0.5j, 0.5, -0.5j
+    m = ((1 - mixed) * np.outer(v, v.conj()) + mixed * np.eye(d) / d).astype(np.complex64)
+    _run(env, m, n)
+    mu = torch.from_numpy(m).cuda()
+    out = torch.full_like(mu, float("nan"))
+    em, er = [torch.empty(d, dtype=torch.float64, device="cuda") for _ in range(2)]
+    lre.lre_project(ctx, mu, n, out, em, er)  # eig_mu: by the reduction
+    lre.lre_sync(ctx)
+    ref, lam_mu, lam = project.smolin(m.astype(np.complex128))
+    assert rel_fro(out.cpu().numpy(), ref) <= 1e-6
+    np.testing.assert_allclose(em.cpu().numpy(), lam_mu, atol=EIG_ATOL)
+    np.testing.assert_allclose(er.cpu().numpy(), lam, atol=EIG_ATOL)
+
+
+@pytest.mark.parametrize("n", [6, 8])
+@pytest.mark.parametrize("eig_mu", [True, False])
+def test_input_that_is_not_finite_is_reported(env, n, eig_mu):
+    torch, lre, ctx = env
+    m = (np.eye(2 ** n) / 2 ** n).astype(np.complex64)
+    m[1, 5] = np.nan
+    mu = torch.from_numpy(m).cuda()
+    em = torch.empty(2 ** n, dtype=torch.float64, device="cuda") if eig_mu else None
+    with pytest.raises(lre.LreError) as e:
+        lre.lre_project(ctx, mu, n, torch.empty_like(mu), em)
+    assert e.value.status == lre.LRE_ERR_EIG_FAILED
