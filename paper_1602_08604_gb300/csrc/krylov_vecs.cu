@@ -34,8 +34,8 @@ __global__ void kry_hermitian(const float2 *__restrict__ in, float2 *__restrict_
   }
 }
 
-// acc[0] += sum |in|^2 (a scale: FP32 sums per thread), acc[1] = the trace in
-// FP64 (block 0, a fixed order).
+// acc[0] += sum |in|^2 (a scale: FP32 sums per thread, once more in FP64 where those
+// leave FP32's range), acc[1] = the trace in FP64 (block 0, a fixed order).
 __global__ void __launch_bounds__(256) kry_norm_trace(const float2 *__restrict__ in, int64_t d, double *acc) {
   __shared__ double s[8];
   auto block_sum = [&](double v) {
@@ -53,7 +53,15 @@ __global__ void __launch_bounds__(256) kry_norm_trace(const float2 *__restrict__
     const float2 a = in[i];
     v = fmaf(a.x, a.x, fmaf(a.y, a.y, v));
   }
-  const double t = block_sum((double)v);
+  double w = (double)v;
+  if (!(v > 0x1p-100f && v < 0x1p126f)) {
+    w = 0.0;
+    for (int64_t i = blockIdx.x * 256 + threadIdx.x; i < d * d; i += (int64_t)gridDim.x * 256) {
+      const double x = in[i].x, y = in[i].y;
+      w = fma(x, x, fma(y, y, w));
+    }
+  }
+  const double t = block_sum(w);
   if (threadIdx.x == 0) atomicAdd(acc, t);
   if (blockIdx.x == 0) {
     double tr = 0;

@@ -209,3 +209,20 @@ def test_input_that_is_not_finite_is_reported(env, n, eig_mu):
     with pytest.raises(lre.LreError) as e:
         lre.lre_project(ctx, mu, n, torch.empty_like(mu), em)
     assert e.value.status == lre.LRE_ERR_EIG_FAILED
+
+
+@pytest.mark.parametrize("scale", [1e-25, 1e25])
+def test_norms_beyond_fp32(env, scale):
+    """Entries whose squares leave FP32's range, d = 2048: the Lanczos path still decides
+    (its breakdown threshold goes by the norm), and the result is right."""
+    torch, lre, ctx = env
+    test_scaled_inputs(env, 11, scale)
+    lam = -np.random.default_rng(11).uniform(0, 2e-4, 2048)
+    lam[-4:] = (0.1, 0.2, 0.3, 0.4)
+    mu = torch.from_numpy((_hermitian_with_spectrum(lam / lam.sum(), 16) * np.float32(scale)).astype(np.complex64)).cuda()
+    lre.lre_profile(ctx, True)
+    lre.lre_project(ctx, mu, 11, torch.empty_like(mu))
+    lre.lre_sync(ctx)
+    names = {k for k, _ in lre.lre_profile_records(ctx)}
+    lre.lre_profile(ctx, False)
+    assert "hetrd(cusolver)" not in names, names
