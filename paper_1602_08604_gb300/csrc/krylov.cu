@@ -395,7 +395,9 @@ lre_status lanczos_steps(lre_ctx *ctx, const KryBuffers &B, int64_t d, int64_t b
   return e == cudaSuccess ? LRE_OK : cuda_fail(ctx, e, "Lanczos step");
 }
 
-// A fresh unit start vector in row `row`, orthogonal to rows [0, row).
+// A fresh unit start vector in row `row`, orthogonal to rows [0, row).  Its norm is
+// summed by one CTA, in a fixed order, where the steps are too (krylov_steps.cu): the
+// call then repeats bit for bit.
 lre_status start_vector(lre_ctx *ctx, const KryBuffers &B, int64_t d, int64_t row, uint64_t seed, cudaStream_t s) {
   const int red_grid = (int)std::min<int64_t>((d + RED_THREADS - 1) / RED_THREADS, (int64_t)ctx->num_sms * 4);
   // built in the FP64 work vector, stored into the basis row in split form
@@ -411,7 +413,7 @@ lre_status start_vector(lre_ctx *ctx, const KryBuffers &B, int64_t d, int64_t ro
     }
   }
   cudaMemsetAsync(B.nrm, 0, sizeof(double), s);
-  kry_norm2<<<red_grid, RED_THREADS, 0, s>>>(B.W, d, B.nrm);
+  kry_norm2<<<B.persistent ? 1 : red_grid, RED_THREADS, 0, s>>>(B.W, d, B.nrm);
   kry_scale<<<red_grid, RED_THREADS, 0, s>>>(B.W, B.Q + row * d, d, B.nrm);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? LRE_OK : cuda_fail(ctx, e, "Lanczos start vector");
@@ -455,7 +457,7 @@ lre_status project_krylov(lre_ctx *ctx, const lre_c64 *rho_in, int64_t d, lre_c6
     B.Xr = reinterpret_cast<double *>(take((size_t)B.rows * B.ct_max * sizeof(double)));
     B.lu = reinterpret_cast<double *>(take((size_t)5 * B.rows * B.ct_max * sizeof(double)));
     B.last = reinterpret_cast<double *>(take((size_t)B.ct_max * sizeof(double)));
-    B.nrm = reinterpret_cast<double *>(take(2 * sizeof(double)));
+    B.nrm = reinterpret_cast<double *>(take(sizeof(double)));
     B.cl = reinterpret_cast<int *>(take((size_t)(B.ct_max + 2) * sizeof(int)));
     B.nclust = reinterpret_cast<int *>(take(sizeof(int)));
     B.breakdown = reinterpret_cast<int *>(take(sizeof(int)));
@@ -475,19 +477,23 @@ lre_status project_krylov(lre_ctx *ctx, const lre_c64 *rho_in, int64_t d, lre_c6
   if (!copy) herm = nullptr;
   B.A = copy ? herm : reinterpret_cast<const float2 *>(rho_in);  // the input is unchanged until the rebuild
 
-  if ((st = kry_prepare_mu(ctx, reinterpret_cast<const float2 *>(rho_in), herm, d, B.nrm, s)) != LRE_OK) return st;
-  double fro_tr[2] = {0, 0};
+  // the trace and the shares of the squared norm, in h1 until the first start vector
+  double *const tn = reinterpret_cast<double *>(B.h1);
+  std::vector<double> fro(1 + kry_norm_blocks(ctx, d));
+  if ((st = kry_prepare_mu(ctx, reinterpret_cast<const float2 *>(rho_in), herm, d, tn, s)) != LRE_OK) return st;
   cudaError_t e = cudaMemsetAsync(B.breakdown, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(fro_tr, B.nrm, sizeof(fro_tr), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(fro.data(), tn, fro.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "Krylov set-up");
-  const double tiny = 1e-14 * sqrt(fro_tr[0]);
+  double norm2 = 0.0;
+  for (size_t k = 1; k < fro.size(); ++k) norm2 += fro[k];
+  const double tiny = 1e-14 * sqrt(norm2);
   // the persistent steps hold squared norms in FP32 pairs, down to tiny^2: a density
   // matrix has a norm in [1/64, 1] there; anything far from that takes the FP64 work
   // vector of the multi-launch form, or the reduction where d is too small for it
-  B.persistent = copy && fro_tr[0] >= 0x1p-20 && fro_tr[0] <= 0x1p60;
+  B.persistent = copy && norm2 >= 0x1p-20 && norm2 <= 0x1p60;
   if (copy && !B.persistent && d < 2048) return LRE_OK;
-  const double trace = fro_tr[1];  // Tr mu (1 up to the complex64 rounding of the diagonal)
+  const double trace = fro[0];  // Tr mu (1 up to the complex64 rounding of the diagonal)
   if ((st = start_vector(ctx, B, d, 0, 0x5EED0001ull, s)) != LRE_OK) return st;
 
   int ct_want = 64, cb_want = 32;

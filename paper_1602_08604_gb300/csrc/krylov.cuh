@@ -31,9 +31,10 @@ lre_status kry_steps_run(lre_ctx *ctx, const KryStepBuffers &B, int64_t d, int64
                          double *alpha, double *beta, double tiny, cudaStream_t s);
 
 // krylov_vecs.cu: herm (d x d, or NULL to leave mu as it is) = the Hermitian
-// matrix of in's upper triangle; norm_trace[0] = its squared Frobenius norm,
-// norm_trace[1] = its trace.
-lre_status kry_prepare_mu(lre_ctx *ctx, const float2 *in, float2 *herm, int64_t d, double *norm_trace, cudaStream_t s);
+// matrix of in's upper triangle; trace_norms[0] = its trace, then
+// kry_norm_blocks(ctx, d) shares of its squared Frobenius norm.
+int64_t kry_norm_blocks(const lre_ctx *ctx, int64_t d);
+lre_status kry_prepare_mu(lre_ctx *ctx, const float2 *in, float2 *herm, int64_t d, double *trace_norms, cudaStream_t s);
 // Z[k] = sum_t S[t + k J] q_t for k < m, rows of d double-float entries.
 lre_status kry_ritz_run(lre_ctx *ctx, const float4 *Q, int J, const double *S, int m, float4 *Z, int64_t d,
                         cudaStream_t s);

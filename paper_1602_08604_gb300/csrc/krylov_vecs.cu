@@ -34,8 +34,9 @@ __global__ void kry_hermitian(const float2 *__restrict__ in, float2 *__restrict_
   }
 }
 
-// acc[0] += sum |in|^2 (a scale: FP32 sums per thread, once more in FP64 where those
-// leave FP32's range), acc[1] = the trace in FP64 (block 0, a fixed order).
+// acc[0] = the trace in FP64 (block 0), acc[1 + b] = block b's share of sum |in|^2 (a
+// scale: FP32 sums per thread, once more in FP64 where those leave FP32's range); all
+// in a fixed order.
 __global__ void __launch_bounds__(256) kry_norm_trace(const float2 *__restrict__ in, int64_t d, double *acc) {
   __shared__ double s[8];
   auto block_sum = [&](double v) {
@@ -62,12 +63,12 @@ __global__ void __launch_bounds__(256) kry_norm_trace(const float2 *__restrict__
     }
   }
   const double t = block_sum(w);
-  if (threadIdx.x == 0) atomicAdd(acc, t);
+  if (threadIdx.x == 0) acc[1 + blockIdx.x] = t;
   if (blockIdx.x == 0) {
     double tr = 0;
     for (int64_t i = threadIdx.x; i < d; i += 256) tr += (double)in[i * d + i].x;
     tr = block_sum(tr);
-    if (threadIdx.x == 0) acc[1] = tr;
+    if (threadIdx.x == 0) acc[0] = tr;
   }
 }
 
@@ -257,18 +258,20 @@ __global__ void __launch_bounds__(256) kry_rebuild(const float4 *__restrict__ Z,
 
 }  // namespace
 
-lre_status kry_prepare_mu(lre_ctx *ctx, const float2 *in, float2 *herm, int64_t d, double *norm_trace, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(norm_trace, 0, 2 * sizeof(double), s);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "Krylov set-up");
+int64_t kry_norm_blocks(const lre_ctx *ctx, int64_t d) {
+  const int64_t g = (d * d + 2047) / 2048, cap = (int64_t)ctx->num_sms * 8;
+  return g < cap ? g : cap;
+}
+
+lre_status kry_prepare_mu(lre_ctx *ctx, const float2 *in, float2 *herm, int64_t d, double *trace_norms, cudaStream_t s) {
   Launch L(ctx, "kry_prepare", s, herm ? 2 : 1);
   if (herm) {
     dim3 g((unsigned)(d / 32), (unsigned)(d / 32)), b(32, 8);
     kry_hermitian<<<g, b, 0, s>>>(in, herm, d);
     in = herm;
   }
-  const int64_t g = (d * d + 2047) / 2048, cap = (int64_t)ctx->num_sms * 8;
-  kry_norm_trace<<<(unsigned)(g < cap ? g : cap), 256, 0, s>>>(in, d, norm_trace);
-  e = cudaGetLastError();
+  kry_norm_trace<<<(unsigned)kry_norm_blocks(ctx, d), 256, 0, s>>>(in, d, trace_norms);
+  const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? LRE_OK : cuda_fail(ctx, e, "Krylov set-up");
 }
 

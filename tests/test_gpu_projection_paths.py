@@ -226,3 +226,25 @@ def test_norms_beyond_fp32(env, scale):
     names = {k for k, _ in lre.lre_profile_records(ctx)}
     lre.lre_profile(ctx, False)
     assert "hetrd(cusolver)" not in names, names
+
+
+@pytest.mark.parametrize("n", [6, 10, 11])
+def test_repeats_bit_for_bit(env, n):
+    """With other work on the device, so that CTAs finish in varying order."""
+    torch, lre, ctx = env
+    d = 2 ** n
+    lam = -np.random.default_rng(n).uniform(0, 0.5 / d, d)
+    lam[-4:] = (0.1, 0.2, 0.3, 0.4)
+    mu = torch.from_numpy(_hermitian_with_spectrum(lam / lam.sum(), 7)).cuda()
+    side, a = torch.cuda.Stream(), torch.randn(512, 512, device="cuda")
+    torch.cuda.synchronize()
+    first = None
+    for _ in range(60):
+        with torch.cuda.stream(side):
+            for _ in range(8):
+                a @ a
+        out, er = torch.empty_like(mu), torch.empty(d, dtype=torch.float64, device="cuda")
+        lre.lre_project(ctx, mu, n, out, eig_rho=er)
+        lre.lre_sync(ctx)
+        first = first or (out, er)
+        assert torch.equal(out, first[0]) and torch.equal(er, first[1])
