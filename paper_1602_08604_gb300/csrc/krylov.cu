@@ -395,6 +395,20 @@ lre_status lanczos_steps(lre_ctx *ctx, const KryBuffers &B, int64_t d, int64_t b
   return e == cudaSuccess ? LRE_OK : cuda_fail(ctx, e, "Lanczos step");
 }
 
+// The step (from 1) whose beta vanished in the runs since the flag was zeroed, 0 if none.
+// LRE_ERR_TIMEOUT where a grid barrier gave up: the run's alpha and beta are not all there.
+lre_status read_breakdown(lre_ctx *ctx, const KryBuffers &B, int &brk, cudaStream_t s) {
+  unsigned gave_up = 0;
+  cudaError_t e = cudaMemcpyAsync(&brk, B.breakdown, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess && B.persistent)
+    e = cudaMemcpyAsync(&gave_up, static_cast<unsigned *>(B.sync) + 1, sizeof(gave_up), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "Lanczos breakdown flag");
+  if (!gave_up) return LRE_OK;
+  ctx->last_error = "projection: a grid barrier of the Lanczos steps gave up";
+  return LRE_ERR_TIMEOUT;
+}
+
 // A fresh unit start vector in row `row`, orthogonal to rows [0, row).  Its norm is
 // summed by one CTA, in a fixed order, where the steps are too (krylov_steps.cu): the
 // call then repeats bit for bit.
@@ -510,9 +524,7 @@ lre_status project_krylov(lre_ctx *ctx, const lre_c64 *rho_in, int64_t d, lre_c6
     if ((st = lanczos_steps(ctx, B, d, 0, J, J1, B.alpha, B.beta, tiny, s)) != LRE_OK) return st;
     J = J1;
     int brk = 0;
-    e = cudaMemcpyAsync(&brk, B.breakdown, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "Lanczos breakdown flag");
+    if ((st = read_breakdown(ctx, B, brk, s)) != LRE_OK) return st;
     const bool broke = brk > 0 || J == d;
     if (brk > 0) J = brk;  // an invariant subspace: T_J holds exact eigenvalues
     const bool exact = J == d;  // the whole spectrum of mu
@@ -630,9 +642,7 @@ lre_status project_krylov(lre_ctx *ctx, const lre_c64 *rho_in, int64_t d, lre_c6
     if (e != cudaSuccess) return cuda_fail(ctx, e, "certification set-up");
     if ((st = lanczos_steps(ctx, B, d, m, 0, L2, alpha2, beta2, tiny, s)) != LRE_OK) return st;
     int brk = 0;
-    e = cudaMemcpyAsync(&brk, B.breakdown, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "certification breakdown flag");
+    if ((st = read_breakdown(ctx, B, brk, s)) != LRE_OK) return st;
     const int J2 = brk > 0 ? brk : L2;
     RitzEnds V;
     if ((st = ritz_values(ctx, B, alpha2, beta2, J2, 1, 1, false, s, V)) != LRE_OK) return st;  // smallest, largest

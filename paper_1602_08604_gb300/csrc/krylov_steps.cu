@@ -55,6 +55,8 @@ struct StepArgs {
   double *alpha, *beta;
   float2 *shares;       // [2][G] the CTAs' shares of alpha and of the norm
   unsigned *bar;        // arrivals, then the abort flag; zeroed before the launch
+  uint64_t wait_ns;     // bound of a barrier's wait
+  unsigned stall;       // test hook: arrivals waited for that never come
   int *breakdown, *status;
   float tiny;
   int d, base, j0, j1, rows;
@@ -93,7 +95,7 @@ __device__ __forceinline__ void block_real_sum(float &h, float &l, float2 *red, 
 // Barrier over all CTAs (every one resident: cooperative launch).  Bounded by
 // time; false once a wait gave up anywhere.
 __device__ __forceinline__ bool grid_barrier(const StepArgs &P, unsigned &target, int *s_ok) {
-  target += gridDim.x;
+  target += gridDim.x + P.stall;
   __syncthreads();
   if (gridDim.x == 1) return true;
   if (threadIdx.x == 0) {
@@ -106,7 +108,7 @@ __device__ __forceinline__ bool grid_barrier(const StepArgs &P, unsigned &target
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(P.bar) : "memory");
       if (v >= target) break;
-      if ((it & 255u) == 255u && (*abort || sm103::globaltimer() - t0 > sm103::kWaitNs)) {
+      if ((it & 255u) == 255u && (*abort || sm103::globaltimer() - t0 > P.wait_ns)) {
         ok = 0;
         break;
       }
@@ -505,6 +507,8 @@ lre_status kry_steps_run(lre_ctx *ctx, const KryStepBuffers &B, int64_t d, int64
   P.bar = static_cast<unsigned *>(B.sync);
   P.shares = reinterpret_cast<float2 *>(P.bar + 4);
   P.breakdown = B.breakdown;
+  P.wait_ns = ctx->batch_wait_ns ? ctx->batch_wait_ns : sm103::kWaitNs;
+  P.stall = ctx->steps_stall;
   P.status = ctx->d_status;
   P.tiny = (float)tiny;
   P.d = (int)d;
@@ -524,3 +528,12 @@ lre_status kry_steps_run(lre_ctx *ctx, const KryStepBuffers &B, int64_t d, int64
 }
 
 }  // namespace lre
+
+// Test hook (not part of include/lre.h): from now on each grid barrier of the Lanczos
+// steps waits for arrivals that never come and gives up after wait_ms (0: as usual).
+extern "C" lre_status lre_debug_steps_fault(lre_ctx *ctx, int wait_ms) {
+  if (!ctx || wait_ms < 0) return LRE_ERR_INVALID_ARG;
+  ctx->batch_wait_ns = (uint64_t)wait_ms * 1000000;
+  ctx->steps_stall = wait_ms > 0;
+  return LRE_OK;
+}

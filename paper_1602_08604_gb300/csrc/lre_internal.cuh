@@ -65,7 +65,8 @@ struct lre_ctx {
   int batch_unit = 256;         // batched schedule: items per unit of the other fold and assembly passes
   int batch_occupancy[2] = {0, 0};  // most resident CTAs per SM of batch_kernel<2>, <3>
   std::vector<lre_batch_entry> batch_cache;  // device pass tables of earlier batched calls
-  uint64_t batch_wait_ns = 0;   // batched kernel: bound of a dependency wait (0 = the default 2 s)
+  uint64_t batch_wait_ns = 0;   // batched kernel, Lanczos steps: bound of a wait (0 = the default 2 s)
+  unsigned steps_stall = 0;     // test hook: arrivals the Lanczos steps' barriers wait for in vain
   int batch_stall_phase = -1;   // test hook: the first dependent phase at or after it never becomes ready
   size_t host_chunk_bytes = 256ull << 20; // host-input streaming: bytes of input per chunk
   int records_direct = 0;                 // host shot records: 1 = always the records-fed first pass

@@ -5,6 +5,8 @@ against the oracle's Smolin projection.
 Tolerances: eigenvalues of both paths are at FP64 rounding of a matrix of norm
 at most 1, d eps = 2.3e-13 at d = 1024; the complex64 result is within the
 rounding of its entries, far inside 1e-6 relative Frobenius."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -248,3 +250,30 @@ def test_repeats_bit_for_bit(env, n):
         lre.lre_sync(ctx)
         first = first or (out, er)
         assert torch.equal(out, first[0]) and torch.equal(er, first[1])
+
+
+@pytest.mark.parametrize("n", [6, 11])
+def test_barrier_that_gives_up_is_reported(env, n):
+    """Barriers that wait for arrivals that never come, 5 ms each: the call returns
+    LRE_ERR_TIMEOUT, writes no result, and the context stays usable."""
+    torch, lre, ctx = env
+    f = lre.load().lre_debug_steps_fault
+    f.argtypes, f.restype = [ctypes.c_void_p, ctypes.c_int], ctypes.c_int
+    d = 2 ** n
+    lam = -np.random.default_rng(n).uniform(0, 0.5 / d, d)
+    lam[-4:] = (0.1, 0.2, 0.3, 0.4)
+    m = _hermitian_with_spectrum(lam / lam.sum(), 7)
+    mu = torch.from_numpy(m).cuda()
+    out = torch.full_like(mu, 3.0)
+    assert f(ctx, 5) == 0
+    try:
+        with pytest.raises(lre.LreError) as e:
+            lre.lre_project(ctx, mu, n, out)
+        assert e.value.status == lre.LRE_ERR_TIMEOUT
+        with pytest.raises(lre.LreError) as e:
+            lre.lre_sync(ctx)  # latched by the kernel too
+        assert e.value.status == lre.LRE_ERR_TIMEOUT
+    finally:
+        assert f(ctx, 0) == 0
+    assert (out == 3.0).all()
+    _run(env, m, n)
