@@ -27,8 +27,8 @@
 // fallback also runs when r is not decided within KRYLOV_MAX steps.
 //
 // Up to d = 1024 the run may go on to d steps, where T holds the whole spectrum
-// and nothing is left to certify; the selected values are then replaced by their
-// FP64 Rayleigh quotients (krylov_vecs.cu), so they are as exact as a reduction's.
+// and nothing is left to certify.  Up to d = 4096 the selected values are replaced
+// by their Rayleigh quotients (krylov_vecs.cu), so they are as exact as a reduction's.
 //
 // Layout: the products read mu as complex64 (up to d = 4096 a Hermitian copy of
 // the input's upper triangle); the Krylov basis Q holds one d-vector per row
@@ -652,7 +652,7 @@ lre_status project_krylov(lre_ctx *ctx, const lre_c64 *rho_in, int64_t d, lre_c6
     if (kept_form && V.w.back() > tau + slack) return LRE_OK;
     if (!kept_form && V.w.front() < tau - slack) return LRE_OK;
   }
-  if (whole && m > 0) {  // below d = 2048: the selected values to FP64 rounding
+  if (copy && m > 0) {  // where the steps are double-float: the selected values to FP64 rounding
     std::vector<double> q(m);
     if ((st = kry_rayleigh_run(ctx, B.A, B.Z, (int)m, d, reinterpret_cast<double2 *>(B.lu), B.last, s)) != LRE_OK)
       return st;

@@ -38,7 +38,7 @@ lre_status kry_prepare_mu(lre_ctx *ctx, const float2 *in, float2 *herm, int64_t 
 // Z[k] = sum_t S[t + k J] q_t for k < m, rows of d double-float entries.
 lre_status kry_ritz_run(lre_ctx *ctx, const float4 *Q, int J, const double *S, int m, float4 *Z, int64_t d,
                         cudaStream_t s);
-// w[k] = the Rayleigh quotient of row k of Z in FP64 (d <= 1024; part: m ceil(d / 64) double2).
+// w[k] = the Rayleigh quotient of row k of Z to FP64 rounding (d <= KRY_STEPS_MAX_D; part: m ceil(d / 64) double2).
 lre_status kry_rayleigh_run(lre_ctx *ctx, const float2 *A, const float4 *Z, int m, int64_t d, double2 *part, double *w,
                             cudaStream_t s);
 // out = sum (w + shift) z z^dag (kept form) or mu + shift I - sum (w + shift) z z^dag.

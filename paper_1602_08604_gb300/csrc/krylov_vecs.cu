@@ -111,31 +111,66 @@ __global__ void __launch_bounds__(128) kry_ritz(const float4 *__restrict__ Q, in
       if (k0 + k < m) Z[(int64_t)(k0 + k) * d + i] = df::norm4(h[k], l[k]);
 }
 
-// part[k][b] = block b's rows of z_k^dag A z_k and of z_k^dag z_k in FP64, over the
-// upper triangle of the Hermitian A (a_rr |z_r|^2 + 2 Re conj(z_r) a_rc z_c).
-// The double-float Lanczos leaves its values 2^-48 ||A|| or so off; the quotient
-// of the finished vectors, whose own error enters squared, is at FP64 rounding.
-// d <= RQ_MAX_D: at 4096 the FP64 sums would cost as much as the Lanczos steps.
-constexpr int RQ_ROWS = 64, RQ_MAX_D = 1024;
+// part[k][b] = block b's rows of z_k^dag A z_k and of z_k^dag z_k, over the upper
+// triangle of the Hermitian A (a_rr |z_r|^2 + 2 Re conj(z_r) a_rc z_c).
+// The double-float Lanczos leaves its values 2^-48 ||A|| or so off (the normalisation
+// of a basis vector is one number for all its entries); the quotient of the finished
+// vectors, whose own error enters squared, is at FP64 rounding.
+// FP64 throughout up to d = 1024.  Beyond (WIDE), where that would cost as much as the
+// Lanczos steps, a row's products and their sum are double-float: each row's error is
+// its own, so weighted by z_r and added in FP64 they average out.  Mean error of eig_rho
+// over four product-state estimates, relative to the norm, without the quotients -> now:
+// d = 2048 1.2e-15 -> 0.3e-15, d = 4096 1.6e-15 -> 0.6e-15 (the FP64 coefficients and second
+// Gram-Schmidt pass of one launch per operation: 0.6e-15, 1.3e-15).  d = 4096, 175
+// vectors: 3.0 of 82 ms.
+constexpr int RQ_ROWS = 64, RQ_FP64_D = 1024;
+constexpr size_t RQ_SMEM = (size_t)KRY_STEPS_MAX_D * sizeof(float4);
+template <bool WIDE>
 __global__ void __launch_bounds__(256) kry_rayleigh(const float2 *__restrict__ A, const float4 *__restrict__ Z, int d,
                                                     double2 *part) {
-  __shared__ double2 z[RQ_MAX_D];
+  extern __shared__ __align__(16) unsigned char rq_smem[];
+  float4 *zf = reinterpret_cast<float4 *>(rq_smem);   // WIDE
+  double2 *zd = reinterpret_cast<double2 *>(rq_smem);  // else
   __shared__ double s1[8], s2[8];
   const int k = blockIdx.x, r0 = blockIdx.y * RQ_ROWS, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < d; i += 256) z[i] = df::join(Z[(int64_t)k * d + i]);
+  for (int i = threadIdx.x; i < d; i += 256) {
+    const float4 z = Z[(int64_t)k * d + i];
+    if constexpr (WIDE) zf[i] = z;
+    else zd[i] = df::join(z);
+  }
   __syncthreads();
   double num = 0.0, den = 0.0;
   for (int r = r0 + warp; r < r0 + RQ_ROWS && r < d; r += 8) {
     double re = 0.0, im = 0.0;  // sum_{c > r} a_rc z_c
-    for (int c = r + 1 + lane; c < d; c += 32) {
-      const float2 a = A[(int64_t)r * d + c];
-      const double ax = (double)a.x, ay = (double)a.y;
-      re = fma(ax, z[c].x, fma(-ay, z[c].y, re));
-      im = fma(ax, z[c].y, fma(ay, z[c].x, im));
+    double2 zr;
+    if constexpr (WIDE) {
+      const float2 *a = A + (int64_t)r * d;
+      df::Sum S;
+      int c = r + 1 + lane;
+      for (; c + 224 < d; c += 256) {
+        float2 v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = a[c + 32 * q];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) df::mac_c64(S, v[q], df::hi(zf[c + 32 * q]), df::lo(zf[c + 32 * q]));
+      }
+      for (; c < d; c += 32) df::mac_c64(S, a[c], df::hi(zf[c]), df::lo(zf[c]));
+      const double2 p = df::join(df::df_ab(S));
+      re = p.x;
+      im = p.y;
+      zr = df::join(zf[r]);
+    } else {
+      for (int c = r + 1 + lane; c < d; c += 32) {
+        const float2 a = A[(int64_t)r * d + c];
+        const double ax = (double)a.x, ay = (double)a.y;
+        re = fma(ax, zd[c].x, fma(-ay, zd[c].y, re));
+        im = fma(ax, zd[c].y, fma(ay, zd[c].x, im));
+      }
+      zr = zd[r];
     }
-    num = fma(2.0 * z[r].x, re, fma(2.0 * z[r].y, im, num));
+    num = fma(2.0 * zr.x, re, fma(2.0 * zr.y, im, num));
     if (lane == 0) {
-      const double q = fma(z[r].x, z[r].x, z[r].y * z[r].y);
+      const double q = fma(zr.x, zr.x, zr.y * zr.y);
       num = fma((double)A[(int64_t)r * d + r].x, q, num);
       den += q;
     }
@@ -286,12 +321,15 @@ lre_status kry_ritz_run(lre_ctx *ctx, const float4 *Q, int J, const double *S, i
 
 lre_status kry_rayleigh_run(lre_ctx *ctx, const float2 *A, const float4 *Z, int m, int64_t d, double2 *part, double *w,
                             cudaStream_t s) {
-  if (d > RQ_MAX_D) return LRE_ERR_UNSUPPORTED;
+  if (d > KRY_STEPS_MAX_D) return LRE_ERR_UNSUPPORTED;
   const int nb = (int)((d + RQ_ROWS - 1) / RQ_ROWS);
+  auto k = d > RQ_FP64_D ? kry_rayleigh<true> : kry_rayleigh<false>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RQ_SMEM);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "Rayleigh quotients");
   Launch L(ctx, "kry_rayleigh", s, 2);
-  kry_rayleigh<<<dim3((unsigned)m, (unsigned)nb), 256, 0, s>>>(A, Z, (int)d, part);
+  k<<<dim3((unsigned)m, (unsigned)nb), 256, (size_t)d * sizeof(float4), s>>>(A, Z, (int)d, part);
   kry_quotients<<<(m + 63) / 64, 64, 0, s>>>(part, m, nb, w);
-  const cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   return e == cudaSuccess ? LRE_OK : cuda_fail(ctx, e, "Rayleigh quotients");
 }
 

@@ -277,3 +277,35 @@ def test_barrier_that_gives_up_is_reported(env, n):
         assert f(ctx, 0) == 0
     assert (out == 3.0).all()
     _run(env, m, n)
+
+
+@pytest.mark.parametrize("seed", [1, 2, 3, 4, 5, 6, 7, 8])
+def test_eigenvalues_at_d_2048(env, seed):
+    """eig_rho of 120 kept values, one of them most of the trace: the Rayleigh quotients' double-float rows average out
+    and their sums are FP64, so a few units of rounding of the norm are left (8 allowed).
+    Reference: the quotients of complex128 eigenvectors, whose own error enters squared."""
+    torch, lre, ctx = env
+    n, d, k = 11, 2048, 120
+    rng = np.random.default_rng(seed)
+    lam = -rng.uniform(0.0, 0.5 / d, d)
+    lam[-k:] = 0.0005 * 1.02 ** np.arange(k)
+    lam[-1] = rng.uniform(0.6, 0.9)
+    mu = torch.from_numpy(_hermitian_with_spectrum(lam / lam.sum(), 50 + seed)).cuda()
+    out, er = torch.empty_like(mu), torch.empty(d, dtype=torch.float64, device="cuda")
+    lre.lre_profile(ctx, True)
+    lre.lre_project(ctx, mu, n, out, eig_rho=er)
+    lre.lre_sync(ctx)
+    names = {name for name, _ in lre.lre_profile_records(ctx)}
+    lre.lre_profile(ctx, False)
+    assert "kry_matvec" in names and "hetrd(cusolver)" not in names, names
+    m = mu.to(torch.complex128)
+    w, v = torch.linalg.eigh(m)
+    w = w.cpu().numpy()
+    a, j = 0.0, 0
+    while w[j] + a / (d - j) < 0.0:
+        a += w[j]
+        j += 1
+    v = v[:, j:]
+    q = ((v.conj() * (m @ v)).sum(0).real / (v.conj() * v).sum(0).real).cpu().numpy()
+    want = np.sort(q + (np.trace(mu.cpu().numpy().astype(np.complex128)).real - q.sum()) / len(q))[::-1]
+    assert np.abs(er[:len(q)].cpu().numpy() - want).max() <= 8 * np.finfo(np.float64).eps * q.max()
