@@ -12,6 +12,8 @@
 
 namespace lre {
 
+constexpr int kMaxN = 14;  // qubits
+
 lre_status cuda_fail(lre_ctx *ctx, cudaError_t e, const char *where) {
   if (ctx) ctx->last_error = std::string(where) + ": " + cudaGetErrorString(e);
   return (e == cudaErrorMemoryAllocation) ? LRE_ERR_OOM : LRE_ERR_CUDA;
@@ -133,6 +135,7 @@ lre_status histogram_run(lre_ctx *ctx, const uint16_t *records, int64_t num_base
                          int64_t shots_per_basis, int n, void *counts, lre_count_kind kind,
                          cudaStream_t s) {
   const size_t smem = sizeof(int32_t) << n;
+  constexpr int most = sizeof(int32_t) << kMaxN;  // the functions' limit, shared by all threads: the largest
   int grid = ctx->num_sms * 4;
   if (grid > num_bases) grid = (int)num_bases;
   Launch L(ctx, "histogram", s);
@@ -142,15 +145,15 @@ lre_status histogram_run(lre_ctx *ctx, const uint16_t *records, int64_t num_base
     if (grid16 > num_bases) grid16 = (int)num_bases;
     const bool vec = (shots_per_basis & 7) == 0 && (reinterpret_cast<uintptr_t>(records) & 15) == 0;
     auto k = vec ? histogram16_kernel<true> : histogram16_kernel<false>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem16);
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(int16_t) << kMaxN));
     k<<<grid16, 256, smem16, s>>>(records, num_bases, shots_per_basis, n, static_cast<int16_t *>(counts),
                                   ctx->d_status);
   } else if (kind == LRE_COUNTS_I16) {
-    cudaFuncSetAttribute(histogram_kernel<int16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(histogram_kernel<int16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     histogram_kernel<int16_t><<<grid, 512, smem, s>>>(records, num_bases, shots_per_basis, n,
                                                       static_cast<int16_t *>(counts), ctx->d_status);
   } else {
-    cudaFuncSetAttribute(histogram_kernel<int32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(histogram_kernel<int32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     histogram_kernel<int32_t><<<grid, 512, smem, s>>>(records, num_bases, shots_per_basis, n,
                                                       static_cast<int32_t *>(counts), ctx->d_status);
   }
@@ -163,8 +166,6 @@ lre_status histogram_run(lre_ctx *ctx, const uint16_t *records, int64_t num_base
 using namespace lre;
 
 namespace {
-constexpr int kMaxN = 14;
-
 lre_status check_ctx(lre_ctx *ctx) { return ctx ? LRE_OK : LRE_ERR_INVALID_ARG; }
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }

@@ -299,9 +299,13 @@ lre_status ritz_values(lre_ctx *ctx, const KryBuffers &B, const double *alpha, c
   const double tnorm = fmax(fabs(hst[0]), fabs(hst[1]));
   const double pad = 2.0 * DBL_EPSILON * tnorm + 2.0 * DBL_MIN;
   const int m = CB + CT;
-  const size_t smem = (size_t)40 * J, rsmem = (size_t)41 * J + 48;
-  e = cudaFuncSetAttribute(tri_ends_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(tri_residual, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem);
+  auto ends_smem = [](size_t n) { return 40 * n; };
+  auto residual_smem = [](size_t n) { return 41 * n + 48; };
+  const size_t smem = ends_smem(J), rsmem = residual_smem(J);
+  // the limits are the functions', shared by all threads: always the largest
+  e = cudaFuncSetAttribute(tri_ends_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ends_smem(KRY_MAX_STEPS));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(tri_residual, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)residual_smem(KRY_MAX_STEPS));
   if (e != cudaSuccess) return cuda_fail(ctx, e, "Ritz values");
   {
     Launch L(ctx, "kry_bisect", s);

@@ -8,6 +8,7 @@ namespace lre {
 // whole in shared memory (64 KB at 4096), and from there on a step's data
 // outweigh its launches.
 constexpr int64_t KRY_STEPS_MAX_D = 4096;
+constexpr int64_t KRY_STEPS_MAX_ROWS = 2049;  // basis rows: d / 2 + 1 there
 
 struct KryStepBuffers {
   const float2 *A;   // mu, row-major complex64

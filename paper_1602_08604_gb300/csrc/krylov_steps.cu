@@ -517,7 +517,11 @@ lre_status kry_steps_run(lre_ctx *ctx, const KryStepBuffers &B, int64_t d, int64
   P.j1 = j1;
   P.rows = (int)B.rows;
   const size_t smem = steps_smem(d, B.rows, G);
-  cudaError_t e = cudaFuncSetAttribute(kry_steps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (d > KRY_STEPS_MAX_D || B.rows > KRY_STEPS_MAX_ROWS) return LRE_ERR_UNSUPPORTED;
+  // the limit is the function's, not the context's: one value for every size, so that no
+  // other thread's call lowers it between here and the launch
+  const size_t most = steps_smem(KRY_STEPS_MAX_D, KRY_STEPS_MAX_ROWS, kry_steps_grid(ctx, KRY_STEPS_MAX_D));
+  cudaError_t e = cudaFuncSetAttribute(kry_steps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
   if (e == cudaSuccess) e = cudaMemsetAsync(B.sync, 0, 2 * sizeof(unsigned), s);
   if (e == cudaSuccess) {
     Launch L(ctx, "kry_matvec", s);  // named for its largest part, the products with mu

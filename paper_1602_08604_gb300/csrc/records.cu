@@ -236,7 +236,9 @@ lre_status tile_bucket_run(lre_ctx *ctx, const uint16_t *records, int64_t tile_r
   if (grid > tile_rows) grid = (int)tile_rows;
   const size_t smem = (size_t)BUCKET_WARPS * (2 << (n - 6)) * sizeof(int32_t);
   Launch L(ctx, "tile_bucket", s);
-  cudaFuncSetAttribute(tile_bucket_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the limit is the function's, shared by all threads: always the largest (n = 14)
+  constexpr int most = BUCKET_WARPS * (2 << 8) * (int)sizeof(int32_t);
+  cudaFuncSetAttribute(tile_bucket_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   tile_bucket_kernel<<<grid, BUCKET_THREADS, smem, s>>>(records, tile_rows, shots, n, entries, offs, ctx->d_status);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? LRE_OK : cuda_fail(ctx, e, "tile bucket launch");
@@ -265,7 +267,9 @@ lre_status records_fold_run(lre_ctx *ctx, const uint16_t *records, int64_t shots
   if (grid > cap) grid = cap;
   {
     Launch L(ctx, "records_fold3", s);
-    cudaError_t e = cudaFuncSetAttribute(records_fold3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // as above
+    cudaError_t e =
+        cudaFuncSetAttribute(records_fold3, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * RF_CELLS * (int)sizeof(uint16_t));
     if (e == cudaSuccess) {
       records_fold3<<<(unsigned)grid, threads, smem, s>>>(records, shots, n, groups, static_cast<int16_t *>(sums),
                                                           ctx->d_status);
