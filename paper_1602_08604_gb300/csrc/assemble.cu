@@ -108,8 +108,7 @@ constexpr int TILE_SMEM = ASM_TILE_SMEM;
 // First pass: qubits 0..5 of each block of 4096 coefficients ->
 // [R_lo 64][C_lo 64] per block (its stored part, herm_stored).
 template <class Num>
-__global__ void __launch_bounds__(256) assemble_low6(const typename Num::In *__restrict__ in,
-                                                    typename Num::V *__restrict__ out, int64_t blocks) {
+__global__ void __launch_bounds__(256) assemble_low6(const typename Num::In *in, typename Num::V *out, int64_t blocks) {
   sm103::pdl_wait();
   sm103::pdl_trigger();
   using V = typename Num::V;
@@ -127,8 +126,7 @@ __global__ void __launch_bounds__(256) assemble_low6(const typename Num::In *__r
 // write places nobody reads), and the last pass writes the stored entries of
 // rho only (assemble_mirror fills the rest).
 template <class Num, bool LAST>
-__global__ void __launch_bounds__(256) assemble_high4(const typename Num::V *__restrict__ in,
-                                                     void *__restrict__ out, int t, int64_t units,
+__global__ void __launch_bounds__(256) assemble_high4(const typename Num::V *in, void *out, int t, int64_t units,
                                                      LastScale scale) {
   sm103::pdl_wait();
   sm103::pdl_trigger();

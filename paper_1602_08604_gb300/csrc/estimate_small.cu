@@ -75,7 +75,7 @@ __device__ __forceinline__ void es_item(const InT *in, int item, int32_t (&acc)[
       ld_row_vec<NO>(p + (al << R), v);
     } else if constexpr (FIRST) {
 #pragma unroll
-      for (int o = 0; o < NO; ++o) v[o] = (int32_t)__ldg(p + (al << R) + o);
+      for (int o = 0; o < NO; ++o) v[o] = (int32_t)p[(al << R) + o];
     } else {
 #pragma unroll
       for (int o = 0; o < NO; ++o) v[o] = (int32_t)p[((al << R) + o) * C];

@@ -200,8 +200,7 @@ __device__ __forceinline__ void weighted_upper(const double *z, double *out) {
 
 template <typename InT>
 __global__ void __launch_bounds__(P1_THREADS, 2)
-    fold_first6_weighted(const InT *__restrict__ counts, const double *__restrict__ wgt, double *__restrict__ out, int n,
-                         int64_t num_tiles) {
+    fold_first6_weighted(const InT *counts, const double *wgt, double *out, int n, int64_t num_tiles) {
   sm103::pdl_wait();
   sm103::pdl_trigger();
   extern __shared__ double Zw[];  // [64][P1_ZSTRIDE]
@@ -221,7 +220,7 @@ __global__ void __launch_bounds__(P1_THREADS, 2)
       for (int p = 0; p < 16; ++p) s0[p] = 0.0;
       int32_t next[8];
       load_row8<InT>(row, next);
-      double wn = __ldg(w);
+      double wn = *w;
 #pragma unroll 1
       for (int a2 = 0; a2 < 3; ++a2) {
 #pragma unroll
@@ -235,7 +234,7 @@ __global__ void __launch_bounds__(P1_THREADS, 2)
           if (a01 < 8 || a2 < 2) {  // the next row, in flight during this one
             row += d;
             load_row8<InT>(row, next);
-            wn = __ldg(++w);
+            wn = *++w;
           }
           uint32_t any = 0;
 #pragma unroll

@@ -172,35 +172,38 @@ __host__ __device__ inline bool planes_hi_needed(int64_t c0, int hi_from, int le
   return idc + (half ? 2 : 3) >= hi_from;
 }
 
-// Loads of pass inputs: the read-only path, or (COHERENT) straight from L2 for
-// inputs written earlier by the same kernel launch (the batched kernel).
+// Loads of pass inputs: plain ones, or (COHERENT) straight from L2 for inputs
+// written earlier by the same kernel launch (the batched kernel).  Not the
+// read-only path, here and below: it is for data that no one writes while the
+// kernel runs, and a kernel launched early (launch_pdl) runs before the one that
+// writes its input ends -- its loads have to stay behind pdl_wait.
 template <bool COHERENT, typename T>
 __device__ __forceinline__ T ld_in(const T *p) {
   if constexpr (COHERENT) return __ldcg(p);
-  else return __ldg(p);
+  else return *p;
 }
 
 // The 2^J contiguous counts of one basis row (first pass, C == 1) as vector
-// loads on the read-only path (counts are never written by the kernels).
+// loads.
 template <int NO, typename InT, typename V>
 __device__ __forceinline__ void ld_row_vec(const InT *p, V (&v)[NO]) {
   constexpr int BYTES = NO * (int)sizeof(InT);
   if constexpr (BYTES == 32) {
-    const int4 a = __ldg(reinterpret_cast<const int4 *>(p));
-    const int4 b = __ldg(reinterpret_cast<const int4 *>(p) + 1);
+    const int4 a = *reinterpret_cast<const int4 *>(p);
+    const int4 b = reinterpret_cast<const int4 *>(p)[1];
     const int w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
     for (int k = 0; k < NO; ++k) v[k] = (V)w[k];
   } else {
     uint32_t w[4];
     if constexpr (BYTES == 16) {
-      const uint4 a = __ldg(reinterpret_cast<const uint4 *>(p));
+      const uint4 a = *reinterpret_cast<const uint4 *>(p);
       w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
     } else if constexpr (BYTES == 8) {
-      const uint2 a = __ldg(reinterpret_cast<const uint2 *>(p));
+      const uint2 a = *reinterpret_cast<const uint2 *>(p);
       w[0] = a.x; w[1] = a.y;
     } else {
-      w[0] = __ldg(reinterpret_cast<const uint32_t *>(p));
+      w[0] = *reinterpret_cast<const uint32_t *>(p);
     }
 #pragma unroll
     for (int k = 0; k < NO; ++k) {
@@ -300,7 +303,7 @@ __device__ __forceinline__ void fold_sums(const GenParams &P, int64_t item, AccT
   constexpr int NA = (J == 1) ? 3 : (J == 2) ? 9 : 27;
   constexpr int NO = 1 << J;
   constexpr int NP = 1 << (2 * J);
-  const InT *__restrict__ in = static_cast<const InT *>(P.in);
+  const InT *in = static_cast<const InT *>(P.in);
   const int64_t row_stride = (1ll << P.r) * P.C;  // al stride
   c = item % P.C;
   ahoh = item / P.C;
@@ -316,7 +319,7 @@ __device__ __forceinline__ void fold_sums(const GenParams &P, int64_t item, AccT
 #pragma unroll
       for (int ol = 0; ol < NO; ++ol) v[ol] = (int32_t)ld_in<COHERENT>(in + base + al * row_stride + ol * P.C);
       wht<J>(v);
-      const double w = __ldg(P.wgt + ah * NA + al);
+      const double w = P.wgt[ah * NA + al];
 #pragma unroll
       for (int m = 0; m < NO; ++m) acc[block_pauli(al, m, J)] += (double)v[m] * w;
     } else {
@@ -610,8 +613,8 @@ __device__ __forceinline__ void asm_low6_finish(void *__restrict__ out, int64_t 
 }
 
 template <class Num, bool LAST, bool HERM = false>
-__device__ __forceinline__ void asm_low6_block(const typename Num::In *__restrict__ in, void *__restrict__ out,
-                                               int64_t blk, typename Num::V *S, const LastScale &scale) {
+__device__ __forceinline__ void asm_low6_block(const typename Num::In *in, void *out, int64_t blk, typename Num::V *S,
+                                               const LastScale &scale) {
   const int tid = threadIdx.x;
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
