@@ -283,9 +283,10 @@ size_t mma_fused9_counter_bytes();
 // records grouped by count tile (records.cu) and the first pass over them
 lre_status tile_bucket_run(lre_ctx *ctx, const uint16_t *records, int64_t tile_rows, int64_t shots, int n,
                            uint16_t *entries, int32_t *offs, cudaStream_t s);
-// Shot records -> the six-qubit pass's int32 output, without dense counts, for n <= 12
-// and at most 32767 shots (records.cu).  sums: room for the three-qubit sums; out: the
-// start of the fold workspace.
+// Shot records -> the six-qubit pass's int32 output, without dense counts, for 9 <= n <= 12,
+// shots a multiple of 8 and at most 1213 (27 of a basis' shots within 16 bits) and records
+// on 16 bytes (records.cu; LRE_ERR_UNSUPPORTED outside).  sums: room for the three-qubit
+// sums; out: the start of the fold workspace.
 bool records_fold_takes(lre_ctx *ctx, const void *records, int n, int64_t shots, size_t dense_bytes);
 lre_status records_fold_run(lre_ctx *ctx, const uint16_t *records, int64_t shots, int n, void *sums, void *out,
                             cudaStream_t s);

@@ -251,14 +251,22 @@ lre_status tile_bucket_run(lre_ctx *ctx, const uint16_t *records, int64_t tile_r
 //   sums past 16 bits are stored and read at twice the width: n = 12, 2000 shots 3005 /
 //     2340; n = 11, 2000 shots 634 / 600;
 //   rows off the 16-byte boundary load two bytes a lane: n = 11, 1003 shots 609 / 585.
+namespace {
+// what the kernel itself needs: its bins and sums in 16 bits, whole vector loads
+bool records_fold_fits(const void *records, int n, int64_t shots) {
+  return n >= 9 && n <= 12 && shots > 0 && shots <= 32767 / 27 && (shots & 7) == 0 &&
+         (reinterpret_cast<uintptr_t>(records) & 15) == 0;
+}
+}  // namespace
+
 bool records_fold_takes(lre_ctx *ctx, const void *records, int n, int64_t shots, size_t dense_bytes) {
-  return ctx->first_variant == 1 && ctx->generic_tma && n >= 9 && n <= 12 && shots > 0 && 27 * shots <= 32767 &&
-         (shots & 7) == 0 && (reinterpret_cast<uintptr_t>(records) & 15) == 0 &&
+  return ctx->first_variant == 1 && ctx->generic_tma && records_fold_fits(records, n, shots) &&
          dense_bytes >= (size_t)ipow(6, n - 3) * 64 * 2;
 }
 
 lre_status records_fold_run(lre_ctx *ctx, const uint16_t *records, int64_t shots, int n, void *sums, void *out,
                             cudaStream_t s) {
+  if (!records_fold_fits(records, n, shots)) return LRE_ERR_UNSUPPORTED;
   const int64_t groups = ipow(3, n - 3);
   const int threads = n == 12 ? 512 : 256, per = n == 12 ? 1 : 2048 >> n;
   const size_t smem = (size_t)(n == 12 ? 2 * RF_CELLS : RF_CELLS) * 2;
