@@ -309,3 +309,25 @@ def test_eigenvalues_at_d_2048(env, seed):
     q = ((v.conj() * (m @ v)).sum(0).real / (v.conj() * v).sum(0).real).cpu().numpy()
     want = np.sort(q + (np.trace(mu.cpu().numpy().astype(np.complex128)).real - q.sum()) / len(q))[::-1]
     assert np.abs(er[:len(q)].cpu().numpy() - want).max() <= 8 * np.finfo(np.float64).eps * q.max()
+
+
+@pytest.mark.parametrize("n", [8, 9, 10])
+def test_dense_values_around_the_threshold(env, n):
+    """An exact state's rounding: a few large eigenvalues and a bulk spaced by 1e-12 on both
+    sides of the threshold.  Diagonal input, so the eigenvalues are known exactly; sixteen
+    units of rounding of the norm are left to the Lanczos coefficients and quotients."""
+    torch, lre, ctx = env
+    d = 2 ** n
+    for seed in range(1, 25):
+        rng = np.random.default_rng(seed)
+        lam = rng.normal(0.0, 3e-10, d)
+        lam[:24] = 0.005 * (1 + 1e-4 * np.arange(24))
+        lam[24] = 1.0 - lam[:24].sum() - lam[25:].sum()
+        lam = lam.astype(np.float32)
+        want = project.smolin_eigenvalues(np.sort(lam.astype(np.float64))[::-1])
+        mu = torch.from_numpy(np.diag(lam).astype(np.complex64)).cuda()
+        er = torch.empty(d, dtype=torch.float64, device="cuda")
+        lre.lre_project(ctx, mu, n, torch.empty_like(mu), eig_rho=er)
+        lre.lre_sync(ctx)
+        tol = 16 * np.finfo(np.float64).eps * lam.max()
+        np.testing.assert_allclose(er.cpu().numpy(), want, rtol=0, atol=tol, err_msg=str(seed))
