@@ -197,8 +197,9 @@ lre_status lre_create(lre_ctx **out, int device) {
   ctx->device = device;
   cudaError_t e = cudaSetDevice(device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device);
-  if (e == cudaSuccess) e = cudaMalloc(&ctx->d_status, 2 * sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(ctx->d_status, 0, 2 * sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&ctx->d_status, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(ctx->d_status, 0, sizeof(int));
+  if (e == cudaSuccess) e = cudaHostAlloc(&ctx->h_info, sizeof(int), cudaHostAllocMapped);
   if (e == cudaSuccess) e = cudaMalloc(&ctx->mma_operand, lre::mma_operand_bytes());
   if (e != cudaSuccess) {
     lre_status st = cuda_fail(ctx, e, "lre_create");
@@ -222,6 +223,7 @@ void lre_destroy(lre_ctx *ctx) {
   if (ctx->blas) cublasDestroy(reinterpret_cast<cublasHandle_t>(ctx->blas));
   if (ctx->ws) cudaFree(ctx->ws);
   if (ctx->d_status) cudaFree(ctx->d_status);
+  if (ctx->h_info) cudaFreeHost(ctx->h_info);
   if (ctx->mma_operand) cudaFree(ctx->mma_operand);
   for (auto &en : ctx->batch_cache) cudaFree(en.table);
   if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
@@ -378,7 +380,7 @@ lre_status lre_sync(lre_ctx *ctx, lre_stream stream) {
   int code = 0;
   cudaError_t e = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = cudaMemcpy(&code, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess && code != 0) e = cudaMemset(ctx->d_status, 0, 2 * sizeof(int));
+  if (e == cudaSuccess && code != 0) e = cudaMemset(ctx->d_status, 0, sizeof(int));
   if (e != cudaSuccess) return cuda_fail(ctx, e, "lre_sync");
   return static_cast<lre_status>(code);
 }

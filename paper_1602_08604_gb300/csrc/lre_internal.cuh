@@ -38,7 +38,8 @@ struct lre_ctx {
   size_t ws_limit = 0;        // 0 = unlimited
   void *ws = nullptr;         // device workspace
   size_t ws_bytes = 0;
-  int *d_status = nullptr;    // device-side latched error code (0 = none), then project_small's info word
+  int *d_status = nullptr;    // device-side latched error code (0 = none)
+  int *h_info = nullptr;      // host word that project_small writes (mapped)
   cusolverDnContext *solver = nullptr;
   cublasContext *blas = nullptr;
   std::string last_error;
