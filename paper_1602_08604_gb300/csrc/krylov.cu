@@ -71,35 +71,49 @@ __global__ void kry_split(const double2 *__restrict__ x, float4 *__restrict__ xs
 // Knuth's TwoSum on the leading part: about 2^-44 relative per term, against
 // 2^-53 in FP64 -- far inside the Lanczos tolerances -- at the FP32 rate,
 // where GB300's FP64 rate had made the product FP64-bound, and reading 8
-// bytes per entry of mu instead of 16.  Packed instructions (dfloat.cuh).
-//
+// bytes per entry of mu instead of 16.  Scalar instructions: the packed ones of
+// dfloat.cuh have no higher rate and cost this kernel, which holds 32 entries a lane,
+// 6 % (n = 13, 832 products: 117 against 110 ms).
+
+// (sh, sl) += m (xh + xl)
+__device__ __forceinline__ void mac1(float &sh, float &sl, float m, float xh, float xl) {
+  const float p = __fmul_rn(m, xh), e = __fmaf_rn(m, xh, -p);
+  const float t = __fadd_rn(sh, p), bp = __fsub_rn(t, sh);
+  const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bp)), __fsub_rn(p, bp));
+  sh = t;
+  sl = __fadd_rn(sl, __fadd_rn(err, __fmaf_rn(m, xl, e)));
+}
+
 // M row-major d x d (d a multiple of MV_CHUNK), x a basis row; y also in split
 // form for the reorthogonalisation.  One row per warp, x staged in shared
 // memory; each lane loads its 32 entries of a chunk before their products (more
-// loads in flight: 4.9 against 3.5 TB/s at d = 16384 loading one at a time).
+// loads in flight: 4.9 against 3.5 TB/s at d = 16384 loading one at a time), after
+// the chunk of x is staged (loaded across its barriers: 110 against 97 ms).
 __global__ void __launch_bounds__(256, 3) kry_matvec_df(const float2 *__restrict__ M, const float4 *__restrict__ xsplit,
                                                      double2 *__restrict__ y, float4 *__restrict__ ysplit,
                                                      int64_t d) {
   __shared__ float4 xs[MV_CHUNK];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * 8 + warp;  // d is a multiple of 8
-  df::Sum S;
+  float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
   for (int64_t c0 = 0; c0 < d; c0 += MV_CHUNK) {
     const float2 *row = M + r * d + c0;
-    float2 u[32];
-#pragma unroll
-    for (int q = 0; q < 32; ++q) u[q] = row[lane + 32 * q];
     __syncthreads();
     for (int k = threadIdx.x; k < MV_CHUNK; k += 256) xs[k] = xsplit[c0 + k];
     __syncthreads();
+    float2 u[32];
+#pragma unroll
+    for (int q = 0; q < 32; ++q) u[q] = row[lane + 32 * q];
 #pragma unroll
     for (int q = 0; q < 32; ++q) {
-      const float4 x = xs[lane + 32 * q];
-      df::mac_c64(S, u[q], df::hi(x), df::lo(x));
+      const float4 x = xs[lane + 32 * q];  // {re hi, im hi, re lo, im lo}
+      mac1(rh, rl, u[q].x, x.x, x.z);
+      mac1(rh, rl, -u[q].y, x.y, x.w);
+      mac1(ih, il, u[q].x, x.y, x.w);
+      mac1(ih, il, u[q].y, x.x, x.z);
     }
   }
-  const double2 p = df::join(df::df_ab(S));
-  const double re = warp_sum(p.x), im = warp_sum(p.y);
+  const double re = warp_sum((double)rh + (double)rl), im = warp_sum((double)ih + (double)il);
   if (lane == 0) {
     y[r] = make_double2(re, im);
     ysplit[r] = df::split(make_double2(re, im));
