@@ -210,12 +210,13 @@ lre_status lre_assemble_noalloc(const double *theta, int n, lre_c64 *rho, lre_st
 
 /* Step (iii): rho_out = argmin over density matrices sigma of
  * ||sigma - rho_in||_F (Sec. II, Smolin et al.): the eigenpairs of rho_in
- * on the needed side of the threshold (Lanczos in double-float arithmetic
- * with FP64 scalars, certified, from n = 6 on when eig_mu is NULL; one kernel
- * with FP64 eigenvalues up to n = 5; else an FP64
- * Hermitian eigendecomposition of rho_in promoted to complex128), the
- * eigenvalue correction onto the probability simplex, and the
- * reconstruction in FP64 rounded once to complex64.  rho_in, rho_out: device complex64
+ * on the needed side of the threshold (Lanczos in double-float arithmetic,
+ * about 47 bits, certified, from n = 6 on when eig_mu is NULL, with the
+ * values to FP64 rounding up to n = 12; one kernel with FP64 eigenvalues up to
+ * n = 5; else an FP64 Hermitian eigendecomposition of rho_in promoted to
+ * complex128), the eigenvalue correction onto the probability simplex, and the
+ * reconstruction (in double-float, in FP64 after the decomposition) rounded
+ * once to complex64.  rho_in, rho_out: device complex64
  * [2^n][2^n] (may alias); eig_mu, eig_rho: device FP64 [2^n] or NULL,
  * receiving the spectra of rho_in and rho_out in decreasing order.  The call
  * synchronises `stream`: for n <= 5 once, at its end; above, before the

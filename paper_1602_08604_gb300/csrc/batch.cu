@@ -1,11 +1,13 @@
 // Batched LRE: many small tomography instances (each n <= 9, its own shot
 // count) in ONE persistent kernel launch.
 //
-// Every instance has the pass list of lre_estimate with uniform shots: the
-// fold passes of step (i) (Sec. III, Eq. 3; at most JMAX qubits per pass in
-// registers, int32 partial sums, the last pass dividing by N 3^k and handing
-// the exact integers T = S 3^(n-k) on) and the exact-integer assembly passes
-// of step (ii) (Eq. 4).  All passes of all instances form one list ordered
+// Every instance has its own list of passes, register passes throughout (the
+// single call's six-qubit first pass and its assembly from the last fold pass
+// are not used here): the fold passes of step (i) (Sec. III, Eq. 3; at most
+// JMAX qubits per pass in registers, int32 partial sums, the last pass dividing
+// by N 3^k and handing the exact integers T = S 3^(n-k) on) and the
+// exact-integer assembly passes of step (ii) (Eq. 4), with the single call's
+// results.  All passes of all instances form one list ordered
 // pass-major (the first pass of every instance, then the second, ...), cut
 // into work units of a tuned number of items.  Each CTA of the persistent
 // grid claims units from a device counter; a unit first waits (bounded by

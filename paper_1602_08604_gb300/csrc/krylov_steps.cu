@@ -484,8 +484,8 @@ size_t steps_smem(int64_t d, int64_t rows, int G) {
 // below that (d = 256: 3.6 ms a run on 32 CTAs, 4.0 on 16, 15.8 on one;
 // d = 1024: 7.7 on 128, 9.0 on 64; d = 64: 0.8 on 8, 0.9 on one).
 // Whole projections, before (the reduction path below d = 2048, one launch per
-// operation above) and now: d = 64 4.9 -> 1.1 ms, 256 16 -> 4.4, 512 34 -> 7.5 (before tridiag.cu's last checks),
-// 1024 82.7 -> 11.1 (51 vectors kept), 4096 177 -> 49-51 (100 kept).
+// operation above) and now: d = 64 4.9 -> 1.1 ms, 256 16 -> 4.4, 512 34 -> 7.1,
+// 1024 82.7 -> 11.2 (51 vectors kept), 4096 177 -> 53 (100 kept).
 int kry_steps_grid(lre_ctx *ctx, int64_t d) {
   const int64_t g = d / 8;
   return (int)std::min<int64_t>(g, ctx->num_sms);

@@ -24,9 +24,9 @@
 // about 50.  Double-float operations take 40 to 80 cycles and do not queue on the
 // narrow FP64 pipe, so everything after the eigenvalues, whose 2^-47 is far inside
 // the complex64 result, uses them.  The eigenvalues are FP64 throughout.
-// d = 16: 98 us, against 705 us for the library route (175 with every step in FP64,
-// 111 with the Sturm counts' entries loaded one by one; then d = 4: 33 against 400,
-// d = 32: 280).
+// d = 16: 113 us a call with its synchronisation, against 705 us for the library
+// route, which synchronises too (98 without it and with eigenvalues to 4 eps; 175
+// with every step in FP64); d = 4: 39 against 400, d = 32: 261.
 #include <cuda_runtime.h>
 
 #include <cfloat>
