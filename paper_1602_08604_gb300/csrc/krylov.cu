@@ -88,6 +88,15 @@ __device__ __forceinline__ void mac1(float &sh, float &sl, float m, float xh, fl
   sl = __fadd_rn(sl, __fadd_rn(err, __fmaf_rn(m, xl, e)));
 }
 
+// (sh, sl) += (ah + al)(bh + bl)
+__device__ __forceinline__ void mac2(float &sh, float &sl, float ah, float al, float bh, float bl) {
+  const float p = __fmul_rn(ah, bh), e = __fmaf_rn(al, bh, __fmaf_rn(ah, bl, __fmaf_rn(ah, bh, -p)));
+  const float t = __fadd_rn(sh, p), bp = __fsub_rn(t, sh);
+  const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bp)), __fsub_rn(p, bp));
+  sh = t;
+  sl = __fadd_rn(sl, __fadd_rn(err, e));
+}
+
 // M row-major d x d (d a multiple of MV_CHUNK), x a basis row; y also in split
 // form for the reorthogonalisation.  One row per warp, x staged in shared
 // memory; each lane loads its 32 entries of a chunk before their products (more
@@ -133,13 +142,15 @@ __global__ void __launch_bounds__(RED_THREADS) kry_dots(const float4 *__restrict
   __shared__ double sr[RED_THREADS / 32], si[RED_THREADS / 32];
   for (int t = blockIdx.x; t < m; t += gridDim.x) {
     const float4 *q = Q + (int64_t)t * d;
-    df::Sum S;
+    float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
     for (int64_t i = threadIdx.x; i < d; i += blockDim.x) {
-      const float4 b = w[i];
-      df::mac_df(S, q[i], df::hi(b), df::lo(b));
+      const float4 a = q[i], b = w[i];  // conj(a) b
+      mac2(rh, rl, a.x, a.z, b.x, b.z);
+      mac2(rh, rl, a.y, a.w, b.y, b.w);
+      mac2(ih, il, a.x, a.z, b.y, b.w);
+      mac2(ih, il, -a.y, -a.w, b.x, b.z);
     }
-    const double2 p = df::join(df::df_conj_ab(S));
-    const double re = warp_sum(p.x), im = warp_sum(p.y);
+    const double re = warp_sum((double)rh + (double)rl), im = warp_sum((double)ih + (double)il);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane == 0) {
       sr[warp] = re;
@@ -173,14 +184,17 @@ __global__ void __launch_bounds__(256) kry_update(double2 *__restrict__ w, float
   const int e = threadIdx.x & 63, slice = threadIdx.x >> 6;
   for (int64_t i0 = (int64_t)blockIdx.x * 64; i0 < d; i0 += (int64_t)gridDim.x * 64) {
     const int64_t i = i0 + e;
-    df::Sum S;
+    float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
     if (i < d) {
       for (int t = slice; t < m; t += UPD_SLICES) {
-        const float4 q = Q[(int64_t)t * d + i];
-        df::mac_df(S, hs[t], df::hi(q), df::lo(q));
+        const float4 q = Q[(int64_t)t * d + i], c = hs[t];  // q c
+        mac2(rh, rl, q.x, q.z, c.x, c.z);
+        mac2(rh, rl, -q.y, -q.w, c.y, c.w);
+        mac2(ih, il, q.x, q.z, c.y, c.w);
+        mac2(ih, il, q.y, q.w, c.x, c.z);
       }
     }
-    part[slice][e] = df::join(df::df_ab(S));
+    part[slice][e] = make_double2((double)rh + (double)rl, (double)ih + (double)il);
     __syncthreads();
     if (slice == 0 && i < d) {
       double re = 0, im = 0;
