@@ -331,3 +331,35 @@ def test_dense_values_around_the_threshold(env, n):
         lre.lre_sync(ctx)
         tol = 16 * np.finfo(np.float64).eps * lam.max()
         np.testing.assert_allclose(er.cpu().numpy(), want, rtol=0, atol=tol, err_msg=str(seed))
+
+
+@pytest.mark.parametrize("n", [6, 7, 8, 9, 10])
+@pytest.mark.parametrize("kind", ["physical", "few negative", "half", "cluster"])
+def test_spectrum_of_mostly_kept_values(env, n, kind):
+    """eig_rho where the kept set is the larger one: all its values to a few units of
+    rounding of the norm (8 allowed), from d Lanczos steps (a long cluster of equal values
+    from the reduction).  Reference: quotients of complex128 eigenvectors."""
+    torch, lre, ctx = env
+    d = 2 ** n
+    rng = np.random.default_rng(n)
+    lam = rng.normal(1.0, 1.0, d) if kind == "half" else rng.uniform(0.1, 1.0, d)
+    if kind == "few negative":
+        lam[:d // 16] = -rng.uniform(0.0, 0.3, d // 16)
+    if kind == "cluster":
+        lam[:d - 20] = 0.5
+    mu = torch.from_numpy(_hermitian_with_spectrum(lam / lam.sum(), 90 + n)).cuda()
+    out, er = torch.empty_like(mu), torch.empty(d, dtype=torch.float64, device="cuda")
+    lre.lre_profile(ctx, True)
+    lre.lre_project(ctx, mu, n, out, eig_rho=er)
+    lre.lre_sync(ctx)
+    names = {name for name, _ in lre.lre_profile_records(ctx)}
+    lre.lre_profile(ctx, False)
+    assert ("hetrd(cusolver)" in names) == (kind == "cluster"), names
+    m = mu.to(torch.complex128)
+    _, v = torch.linalg.eigh(m)
+    q = np.sort(((v.conj() * (m @ v)).sum(0).real / (v.conj() * v).sum(0).real).cpu().numpy())[::-1]
+    want = project.smolin_eigenvalues(q)
+    assert (want > 0).sum() > d // 2
+    assert np.abs(er.cpu().numpy() - want).max() <= 8 * np.finfo(np.float64).eps * np.abs(q).max()
+    ref = project.smolin(mu.cpu().numpy().astype(np.complex128))[0]
+    assert rel_fro(out.cpu().numpy(), ref) <= 1e-6
